@@ -170,19 +170,19 @@ fw2_status finalize(fw2_ctx *c) {
   // at that stride), the tissue count rounded up to 4 for the uint16 form
   Q.tab_stride = wide ? (c->n_tissue + 3) / 4 * 4 : kTissues;
   // medium scan: c_max (high-frequency) and validity
-  CK(c, cudaMemsetAsync(c->d_scan, 0, 2 * sizeof(unsigned long long), c->stream));
-  CK(c, cudaMemsetAsync(c->d_bad, 0, sizeof(int), c->stream));
-  CK(c, launch_medium_scan(Q, c->d_scan, c->d_bad, c->stream));
-  c->launches++;
-  unsigned long long mx[2];
-  int bad = 0;
-  CK(c, cudaMemcpyAsync(mx, c->d_scan, sizeof mx, cudaMemcpyDeviceToHost, c->stream));
-  CK(c, cudaMemcpyAsync(&bad, c->d_bad, sizeof bad, cudaMemcpyDeviceToHost, c->stream));
+  CK(c, cudaMemsetAsync(c->d_scan, 0, sizeof(ScanOut), c->stream));
+  CK(c, launch_medium_scan(Q, c->d_scan, c->stream));
+  c->launches += 2;
+  ScanOut scan;
+  CK(c, cudaMemcpyAsync(&scan, c->d_scan, sizeof scan, cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
-  if (bad) return fail(c, FW2_EINVAL, "%d cells have non-positive or non-finite c, rho, kappa or beta", bad);
-  double ce, cm;
-  std::memcpy(&ce, &mx[0], 8);
-  std::memcpy(&cm, &mx[1], 8);
+  if (scan.bad)
+    return fail(c, FW2_EINVAL, "%d cells have non-positive or non-finite c, rho, kappa or beta", (int)scan.bad);
+  double ce;
+  float cmf;
+  std::memcpy(&ce, &scan.speed_bits, 8);
+  std::memcpy(&cmf, &scan.c_bits, 4);
+  const double cm = cmf;
   c->cmax_eff = ce;
   c->cmax = cm;
   c->dt = cfg.dt > 0.0 ? cfg.dt : cfg.cfl * cfg.h / ce;
@@ -239,6 +239,13 @@ fw2_status finalize(fw2_ctx *c) {
       Q.sa2[q] = take(strip_bytes[q]); Q.sb2[q] = take(strip_bytes[q]);
     }
   }
+  if (strips) {
+    void *pb;
+    if ((st = dalloc(c, profile_bytes(Q), &pb)) != FW2_OK) return st;
+    Q.profile = pb;
+    CK(c, launch_profiles(Q, c->stream));
+    c->launches++;
+  }
   // FP16 maps: a scan pass for the largest magnitude of every map, then a
   // power-of-two scale per map that puts it in [2^14, 2^15)
   float scale[kMapScales];
@@ -284,6 +291,7 @@ fw2_status finalize(fw2_ctx *c) {
   }
   dfree(c, c->raw_tissue);
   c->raw_tissue = nullptr;
+  dfree(c, Q.profile);
   c->medium_set = c->relax_set = false;
   // step parameters
   StepParams &P = c->P;
@@ -742,8 +750,7 @@ fw2_status fw2_create(const fw2_config *cfg_in, fw2_ctx **out) {
     for (int q = 0; q < c->nd; ++q) { c->v[q] = (float *)cur; cur += arr; }
     for (int q = 0; q < c->nd; ++q) { c->psi1[q] = (float *)cur; cur += arr * c->N; }
     for (int q = 0; q < c->nd; ++q) { c->psi2[q] = (float *)cur; cur += arr * c->N; }
-    if ((st = dalloc(c, 2 * sizeof(unsigned long long), &m)) == FW2_OK) c->d_scan = (unsigned long long *)m;
-    if (st == FW2_OK && (st = dalloc(c, sizeof(int), &m)) == FW2_OK) c->d_bad = (int *)m;
+    if ((st = dalloc(c, sizeof(ScanOut), &m)) == FW2_OK) c->d_scan = (ScanOut *)m;
     if (st == FW2_OK && (st = dalloc(c, sizeof(unsigned int), &m)) == FW2_OK) c->d_absmax = (unsigned int *)m;
     if (st == FW2_OK && (st = dalloc(c, sizeof(unsigned int), &m)) == FW2_OK) c->d_status = (unsigned int *)m;
   }

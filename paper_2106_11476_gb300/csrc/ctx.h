@@ -74,8 +74,7 @@ struct fw2_ctx {
   float *rec_out = nullptr;
   long long rec_steps = 0;
   // scratch words for scans
-  unsigned long long *d_scan = nullptr;
-  int *d_bad = nullptr;
+  fw2::ScanOut *d_scan = nullptr;
   unsigned int *d_absmax = nullptr;
   unsigned int *d_status = nullptr;  // bit 0: a bounded device-side wait gave up
   long long step = 0, launches = 0;

@@ -36,10 +36,22 @@ struct PrepParams {
   // a scan pass first gathers into f16_max (float bits, device)
   double inv_scale[kMapScales];
   unsigned int *f16_max;
+  void *profile;  // C-PML profile factors of every strip coordinate (profile_bytes), device
 };
 
-cudaError_t launch_medium_scan(const PrepParams &Q, unsigned long long *maxbits, int *bad,
-                               cudaStream_t s);
+// Result of the medium scan (device, zeroed by the caller): bit patterns of
+// non-negative values, which order like the values
+struct ScanOut {
+  unsigned long long speed_bits;  // largest c / sqrt(kappa1 kappa2), double
+  unsigned int quot_bits;         // the same in float (first pass)
+  unsigned int c_bits;            // largest c, float
+  unsigned int bad;               // invalid cells
+  unsigned int pad;
+};
+cudaError_t launch_medium_scan(const PrepParams &Q, ScanOut *out, cudaStream_t s);
+// C-PML profile factors into Q.profile; before launch_prep and launch_prep_scan
+size_t profile_bytes(const PrepParams &Q);
+cudaError_t launch_profiles(const PrepParams &Q, cudaStream_t s);
 // map_kind: 0 float, 1 bf16, 2 uint8 tissue index, 3 uint16 tissue index,
 // 4 FP16 (after launch_prep_scan and with Q.inv_scale set)
 cudaError_t launch_prep(const PrepParams &Q, int map_kind, cudaStream_t s);

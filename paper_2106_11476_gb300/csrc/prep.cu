@@ -16,6 +16,7 @@
 // The profile of a face is evaluated at its exact staggered coordinate; the
 // relaxation parameters of a face are those of its lower-index cell.
 #include "fw2_prep.cuh"
+#include <algorithm>
 #include <type_traits>
 
 #include "maps.cuh"
@@ -121,29 +122,56 @@ __device__ __forceinline__ double depth_of(double x, int n, int L) {
   return d < (double)L ? d : (double)L;
 }
 
-// C-PML / transition value of parameter X0 at `depth` (Table 1).
+// Profile factors of one depth (Table 1): they depend on the depth alone, so
+// they are evaluated once per strip coordinate (profile_kernel, 10 us) and not
+// in every cell: the strips were bound by the FP64 cosine and power of each
+// cell, 55 ms of three strips at 512^3 (N = 3, bf16) against 10 ms now, 0.93
+// against 0.18 ms at 4096^2.
+struct Profile {
+  double depth;  // cells into the boundary region, 0: interior value
+  double gT;     // cosine blend of the transition layer
+  double spow;   // (depth / L)^npow
+};
+
+__device__ __forceinline__ Profile profile_at(const PrepParams &Q, double depth) {
+  Profile f{depth, 1.0, 0.0};
+  const int LT = Q.LT, L = Q.LT + Q.LB;
+  if (LT > 0 && depth < LT) f.gT = 0.5 * (1.0 - cos(M_PI * depth / LT));
+  f.spow = pow(depth / L, Q.npow);
+  return f;
+}
+
+// C-PML / transition value of parameter X0 at a profile's depth (Table 1).
 // nu is 0-based here (nu = 0 is the paper's nu = 1); is_d selects d or alpha.
-__device__ double ramp(const PrepParams &Q, double X0, double depth, int nu, bool is_d) {
-  if (depth <= 0.0) return X0;
-  const int LT = Q.LT, LB = Q.LB, L = LT + LB;
+__device__ __forceinline__ double ramp(const PrepParams &Q, double X0, const Profile &f, int nu, bool is_d) {
+  if (f.depth <= 0.0) return X0;
+  const int L = Q.LT + Q.LB;
   if (nu == 0 && !is_d && (Q.reading == 2 || Q.reading == 3)) {
     // reading C: the tissue's alpha is blended (cosine over the transition
     // layer) into the C-PML profile d_target (1 - x/L), linear to 0 at the
     // outer edge
-    double gT = 1.0;
-    if (LT > 0 && depth < LT) gT = 0.5 * (1.0 - cos(M_PI * depth / LT));
-    const double a_cfs = Q.d_target * (1.0 - depth / L);
-    return (1.0 - gT) * X0 + gT * a_cfs;
+    const double a_cfs = Q.d_target * (1.0 - f.depth / L);
+    return (1.0 - f.gT) * X0 + f.gT * a_cfs;
   }
   if (nu == 0) {
-    const double s = depth / L;
-    if (is_d) return (Q.d_target - X0) * pow(s, Q.npow) + X0;
-    return (0.0 - X0) * s + X0;
+    if (is_d) return (Q.d_target - X0) * f.spow + X0;
+    return (0.0 - X0) * (f.depth / L) + X0;
   }
   if (Q.reading == 3) return X0;  // no transition layer: nu >= 2 kept (unstable, Sec. 3.3)
-  double g = 1.0;
-  if (LT > 0 && depth < LT) g = 0.5 * (1.0 - cos(M_PI * depth / LT));
-  return (0.0 - X0) * g + X0;
+  return (0.0 - X0) * f.gT + X0;
+}
+
+// Profiles of axis q's strip: entry 2 sc of Q.profile[q] for the face, 2 sc +
+// 1 for the centre of strip coordinate sc.
+__global__ void profile_kernel(const PrepParams Q) {
+  const int L = Q.LT + Q.LB, q = blockIdx.y;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 4 * L) return;
+  const int ext = q == 0 ? Q.nx : q == 1 ? Q.ny : Q.nz;
+  const int sc = t >> 1;
+  const int cell = sc < L ? sc : ext - 2 * L + sc;
+  const double x = Q.goff[q] + cell + ((t & 1) ? 0.0 : 0.5);
+  static_cast<Profile *>(Q.profile)[(long long)q * 4 * L + t] = profile_at(Q, depth_of(x, Q.gext[q], L));
 }
 
 template <typename MT, bool SCAN>
@@ -170,17 +198,19 @@ __global__ void cell_maps_kernel(const PrepParams Q) {
       const double chi = Q.nl_mode != 2 ? (1.0 - 2.0 * beta) / K : -2.0 * beta / K;  // 1, 3: Eq. general6
       out.put(kMsChi, Q.chi, o, chi);
     }
-    const double k1 = Q.N ? (double)Q.k1[t] : 1.0, k2 = Q.N ? (double)Q.k2[t] : 1.0;
-    const double ik1 = 1.0 / k1, ik2 = 1.0 / k2;
+    // the rounded float reciprocal equals the FP64 quotient rounded to float
+    // (53 bits are more than 2 x 24 + 2), without two FP64 divisions per cell
+    const float k1 = Q.N ? Q.k1[t] : 1.f, k2 = Q.N ? Q.k2[t] : 1.f;
+    const float ik1 = __frcp_rn(k1), ik2 = __frcp_rn(k2);
     out.put(kMsIk1, Q.ik1, o, ik1);
     out.put(kMsIk2, Q.ik2, o, ik2);
     const float dt = (float)Q.dt;
     for (int nu = 0; nu < Q.N; ++nu) {
       float a, b, omb;
-      relax_ab32(Q.d1[nu * n + t], Q.al1[nu * n + t], (float)k1, (float)ik1, dt, a, b, omb);
+      relax_ab32(Q.d1[nu * n + t], Q.al1[nu * n + t], k1, ik1, dt, a, b, omb);
       out.put(kMsA1 + nu, Q.a1, nu * Q.npts_alloc + o, a);
       out.put_b2(kMsB1 + nu, Q.b1, nu * Q.npts_alloc + o, b, omb);
-      relax_ab32(Q.d2[nu * n + t], Q.al2[nu * n + t], (float)k2, (float)ik2, dt, a, b, omb);
+      relax_ab32(Q.d2[nu * n + t], Q.al2[nu * n + t], k2, ik2, dt, a, b, omb);
       out.put(kMsA2 + nu, Q.a2, nu * Q.npts_alloc + o, a);
       out.put_b2(kMsB2 + nu, Q.b2, nu * Q.npts_alloc + o, b, omb);
     }
@@ -263,22 +293,22 @@ __global__ void strip_maps_kernel(const PrepParams Q, int axis) {
     if (axis == 0) out = ((long long)s[2] * Q.ny + s[1]) * pitch_out + s[0];
     else if (axis == 1) out = ((long long)s[2] * (2 * L) + s[1]) * pitch_out + s[0];
     else out = ((long long)s[2] * Q.ny + s[1]) * pitch_out + s[0];
-    const double dface = depth_of(Q.goff[axis] + cell[axis] + 0.5, Q.gext[axis], L);
-    const double dcent = depth_of((double)(Q.goff[axis] + cell[axis]), Q.gext[axis], L);
+    const Profile *prof = static_cast<const Profile *>(Q.profile) + ((long long)axis * 2 * L + sc) * 2;
+    const Profile fface = prof[0], fcent = prof[1];
     const long long ri = src_of(Q, src), nr = n_src(Q);
-    const double k1 = Q.k1[ri], k2 = Q.k2[ri];
-    const float ik1 = (float)(1.0 / k1), ik2 = (float)(1.0 / k2), dt = (float)Q.dt;
+    const float k1 = Q.k1[ri], k2 = Q.k2[ri];
+    const float ik1 = __frcp_rn(k1), ik2 = __frcp_rn(k2), dt = (float)Q.dt;  // as cell_maps_kernel
     // the ramped parameters (FP64) through the float coefficients of the cells
     for (int nu = 0; nu < Q.N; ++nu) {
       float a, b, omb;
-      const double d1 = ramp(Q, Q.d1[nu * nr + ri], dface, nu, true);
-      const double al1 = ramp(Q, Q.al1[nu * nr + ri], dface, nu, false);
-      relax_ab32((float)d1, (float)al1, (float)k1, ik1, dt, a, b, omb);
+      const double d1 = ramp(Q, Q.d1[nu * nr + ri], fface, nu, true);
+      const double al1 = ramp(Q, Q.al1[nu * nr + ri], fface, nu, false);
+      relax_ab32((float)d1, (float)al1, k1, ik1, dt, a, b, omb);
       sink.put(kMsA1 + nu, Q.sa1[axis], nu * Q.strip_nu[axis] + out, a);
       sink.put_b2(kMsB1 + nu, Q.sb1[axis], nu * Q.strip_nu[axis] + out, b, omb);
-      const double d2 = ramp(Q, Q.d2[nu * nr + ri], dcent, nu, true);
-      const double al2 = ramp(Q, Q.al2[nu * nr + ri], dcent, nu, false);
-      relax_ab32((float)d2, (float)al2, (float)k2, ik2, dt, a, b, omb);
+      const double d2 = ramp(Q, Q.d2[nu * nr + ri], fcent, nu, true);
+      const double al2 = ramp(Q, Q.al2[nu * nr + ri], fcent, nu, false);
+      relax_ab32((float)d2, (float)al2, k2, ik2, dt, a, b, omb);
       sink.put(kMsA2 + nu, Q.sa2[axis], nu * Q.strip_nu[axis] + out, a);
       sink.put_b2(kMsB2 + nu, Q.sb2[axis], nu * Q.strip_nu[axis] + out, b, omb);
     }
@@ -286,38 +316,109 @@ __global__ void strip_maps_kernel(const PrepParams Q, int axis) {
   sink.flush();
 }
 
-// Largest c / sqrt(kappa1 kappa2) and largest c (FP64, as ordered bit
-// patterns of positive doubles) and a count of invalid cells.
-__global__ void medium_scan_kernel(const PrepParams Q, unsigned long long *maxbits, int *bad) {
+// Medium scan: count of invalid cells, largest c, and largest c /
+// sqrt(kappa1 kappa2) in FP64.  Two passes, both bound by reading the medium:
+// the first checks every cell and finds the largest quotient in float, the
+// second evaluates in FP64 only the cells whose float quotient is within its
+// rounding of that (a cell whose float product leaves float's range always
+// is).  Each block reduces before its atomics: two FP64 atomics of every
+// thread on one address took 1.6 to 1.7 ms from 2 M cells up, where the two
+// passes take 0.04 ms (2 M cells) to 0.26 ms (4096^2).
+constexpr float kScanMargin = 1e-5f;  // far above the float quotient's error (about 4 ulp)
+
+struct ScanCell {
+  float c, k1, k2;
+  bool ok;
+};
+__device__ __forceinline__ ScanCell scan_cell(const PrepParams &Q, long long t) {
+  ScanCell s{0.f, 1.f, 1.f, false};
+  if (Q.tissue_in && tissue_at(Q, t) >= Q.n_tissue) return s;
+  const long long r = src_of(Q, t);
+  s.c = Q.c[r];
+  const float rho = Q.rho[r];
+  if (Q.N) {
+    s.k1 = Q.k1[r];
+    s.k2 = Q.k2[r];
+  }
+  s.ok = isfinite(s.c) && s.c > 0.f && isfinite(rho) && rho > 0.f && isfinite(s.k1) && s.k1 > 0.f &&
+         isfinite(s.k2) && s.k2 > 0.f && (Q.nl_mode == 0 || isfinite(Q.beta[r]));
+  return s;
+}
+// float quotient, or -1 where the product or the quotient leaves the normal range
+__device__ __forceinline__ float scan_quot(const ScanCell &s) {
+  const float kk = s.k1 * s.k2;
+  if (!(kk > 1e-30f && kk < 1e30f)) return -1.f;
+  const float e = s.c * rsqrtf(kk);
+  return (e > 1e-30f && e < 1e30f) ? e : -1.f;
+}
+
+__global__ void __launch_bounds__(256) medium_scan_kernel(const PrepParams Q, ScanOut *out) {
   const long long n = (long long)Q.nx * Q.ny * Q.nz;
-  double m_eff = 0.0, m_c = 0.0;
+  float m_e = 0.f, m_c = 0.f;
   int nbad = 0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
-    if (Q.tissue_in && tissue_at(Q, t) >= Q.n_tissue) {
+    const ScanCell s = scan_cell(Q, t);
+    if (!s.ok) {
       ++nbad;
       continue;
     }
-    const long long r = src_of(Q, t);
-    const double c = Q.c[r], rho = Q.rho[r];
-    double k1 = 1.0, k2 = 1.0;
-    if (Q.N) {
-      k1 = Q.k1[r];
-      k2 = Q.k2[r];
-    }
-    const bool ok = isfinite(c) && c > 0.0 && isfinite(rho) && rho > 0.0 && isfinite(k1) && k1 > 0.0 &&
-                    isfinite(k2) && k2 > 0.0 && (Q.nl_mode == 0 || isfinite((double)Q.beta[r]));
-    if (!ok) {
-      ++nbad;
-      continue;
-    }
-    const double ce = c / sqrt(k1 * k2);
-    m_eff = ce > m_eff ? ce : m_eff;
-    m_c = c > m_c ? c : m_c;
+    m_e = fmaxf(m_e, scan_quot(s));
+    m_c = fmaxf(m_c, s.c);
   }
-  if (m_eff > 0.0) atomicMax(&maxbits[0], (unsigned long long)__double_as_longlong(m_eff));
-  if (m_c > 0.0) atomicMax(&maxbits[1], (unsigned long long)__double_as_longlong(m_c));
-  if (nbad) atomicAdd(bad, nbad);
+  // non-negative floats order like their bits
+  const unsigned we = __reduce_max_sync(0xffffffffu, __float_as_uint(m_e));
+  const unsigned wc = __reduce_max_sync(0xffffffffu, __float_as_uint(m_c));
+  const unsigned wb = __reduce_add_sync(0xffffffffu, (unsigned)nbad);
+  __shared__ unsigned red[3][8];
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = we;
+    red[1][threadIdx.x >> 5] = wc;
+    red[2][threadIdx.x >> 5] = wb;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned e = 0, c = 0, b = 0;
+    for (int w = 0; w < 8; ++w) {
+      e = max(e, red[0][w]);
+      c = max(c, red[1][w]);
+      b += red[2][w];
+    }
+    if (e) atomicMax(&out->quot_bits, e);
+    if (c) atomicMax(&out->c_bits, c);
+    if (b) atomicAdd(&out->bad, b);
+  }
+}
+
+__global__ void __launch_bounds__(256) medium_speed_kernel(const PrepParams Q, ScanOut *out) {
+  const long long n = (long long)Q.nx * Q.ny * Q.nz;
+  const float cut = __uint_as_float(out->quot_bits) * (1.f - kScanMargin);
+  double m = 0.0;
+  ScanCell last{0.f, 0.f, 0.f, false};  // a uniform medium is one value, not one per cell
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+       t += (long long)gridDim.x * blockDim.x) {
+    const ScanCell s = scan_cell(Q, t);
+    if (!s.ok) continue;
+    const float e = scan_quot(s);
+    if ((e >= 0.f && e < cut) || (s.c == last.c && s.k1 == last.k1 && s.k2 == last.k2)) continue;
+    last = s;
+    const double ce = (double)s.c / sqrt((double)s.k1 * (double)s.k2);
+    m = ce > m ? ce : m;
+  }
+  unsigned long long bits = (unsigned long long)__double_as_longlong(m);
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, bits, o);
+    bits = x > bits ? x : bits;
+  }
+  __shared__ unsigned long long red[8];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = bits;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) bits = red[w] > bits ? red[w] : bits;
+    // a homogeneous medium has candidates in every block: only a larger value
+    // goes to the atomic (the plain read may be old, which costs an atomic)
+    if (bits > *reinterpret_cast<volatile unsigned long long *>(&out->speed_bits)) atomicMax(&out->speed_bits, bits);
+  }
 }
 
 int grid_for(long long n) {
@@ -329,10 +430,22 @@ int grid_for(long long n) {
 
 }  // namespace
 
-cudaError_t launch_medium_scan(const PrepParams &Q, unsigned long long *maxbits, int *bad,
-                               cudaStream_t s) {
+cudaError_t launch_medium_scan(const PrepParams &Q, ScanOut *out, cudaStream_t s) {
   const long long n = (long long)Q.nx * Q.ny * Q.nz;
-  medium_scan_kernel<<<grid_for(n), 256, 0, s>>>(Q, maxbits, bad);
+  // eight blocks per SM: enough loads in flight for the copy bandwidth, few atomics
+  const int grid = (int)std::min<long long>((n + 255) / 256, 152 * 8);
+  medium_scan_kernel<<<grid, 256, 0, s>>>(Q, out);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  medium_speed_kernel<<<grid, 256, 0, s>>>(Q, out);
+  return cudaGetLastError();
+}
+
+size_t profile_bytes(const PrepParams &Q) { return sizeof(Profile) * 3 * 4 * (size_t)(Q.LT + Q.LB); }
+
+cudaError_t launch_profiles(const PrepParams &Q, cudaStream_t s) {
+  const int L = Q.LT + Q.LB;
+  profile_kernel<<<dim3((4 * L + 127) / 128, Q.nd), 128, 0, s>>>(Q);
   return cudaGetLastError();
 }
 
