@@ -345,7 +345,7 @@ fw2_status finalize(fw2_ctx *c) {
 fw2_status build_sources(fw2_ctx *c) {
   if (!c->src_dirty) return FW2_OK;
   for (DevSource &d : c->dsrc) {
-    dfree(c, d.tgt); dfree(c, d.off); dfree(c, d.col);
+    dfree(c, d.tgt); dfree(c, d.off); dfree(c, d.col); dfree(c, d.unit); dfree(c, d.pos);
     d = DevSource{};
   }
   dfree(c, c->d_signal);
@@ -374,22 +374,39 @@ fw2_status build_sources(fw2_ctx *c) {
     CK(c, cudaStreamSynchronize(c->stream));
   }
   for (int kind = 0; kind < 4; ++kind) {
-    struct E { long long tgt; int col; long long order; };
+    struct E { long long tgt; int unit, pos, col; long long order; };
+    const int ntx = (c->nx + kTX - 1) / kTX, nhy = (c->ny + kPipeHalf - 1) / kPipeHalf;
     std::vector<E> es;
     long long base = 0, order = 0;
     for (const HostSource &s : c->sources) {
       if (s.kind == kind)
-        for (size_t e = 0; e < s.idx.size(); ++e) es.push_back({to_pitched(c, s.idx[e]), (int)(base + s.group[e]), order++});
+        for (size_t e = 0; e < s.idx.size(); ++e) {
+          E x{to_pitched(c, s.idx[e]), 0, 0, (int)(base + s.group[e]), order++};
+          if (c->nd == 2) {
+            const int i = (int)(x.tgt % c->pitch), j = (int)(x.tgt / c->pitch);
+            x.unit = (j / kPipeHalf) * ntx + i / kTX;
+            x.pos = (j % kPipeHalf) * kTX + i % kTX;
+          }
+          es.push_back(x);
+        }
       base += s.n_groups;
     }
     if (es.empty()) continue;
-    std::stable_sort(es.begin(), es.end(), [](const E &a, const E &b) { return a.tgt < b.tgt; });
+    // by half tile (2D), then cell; entries of one cell keep their order
+    std::stable_sort(es.begin(), es.end(), [](const E &a, const E &b) {
+      return a.unit != b.unit ? a.unit < b.unit : a.tgt < b.tgt;
+    });
     std::vector<long long> tgt;
-    std::vector<int> off, col;
+    std::vector<int> off, col, pos, unit;
+    if (c->nd == 2) unit.assign((size_t)ntx * nhy + 1, 0);
     for (size_t e = 0; e < es.size(); ++e) {
       if (e == 0 || es[e].tgt != es[e - 1].tgt) {
         tgt.push_back(es[e].tgt);
         off.push_back((int)col.size());
+        if (c->nd == 2) {
+          pos.push_back(es[e].pos);
+          unit[es[e].unit + 1]++;
+        }
       }
       col.push_back(es[e].col);
     }
@@ -404,6 +421,15 @@ fw2_status build_sources(fw2_ctx *c) {
     if ((st = dalloc(c, col.size() * sizeof(int), &m)) != FW2_OK) return st;
     d.col = (int *)m;
     d.n_tgt = (int)tgt.size();
+    if (c->nd == 2) {
+      for (size_t u = 1; u < unit.size(); ++u) unit[u] += unit[u - 1];
+      if ((st = dalloc(c, unit.size() * sizeof(int), &m)) != FW2_OK) return st;
+      d.unit = (int *)m;
+      if ((st = dalloc(c, pos.size() * sizeof(int), &m)) != FW2_OK) return st;
+      d.pos = (int *)m;
+      CK(c, cudaMemcpyAsync(d.unit, unit.data(), unit.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+      CK(c, cudaMemcpyAsync(d.pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    }
     CK(c, cudaMemcpyAsync(d.tgt, tgt.data(), tgt.size() * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaMemcpyAsync(d.off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaMemcpyAsync(d.col, col.data(), col.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
@@ -475,6 +501,42 @@ int layout_for_step(fw2_ctx *c, bool *timed) {
   return t < 2 ? kLayoutStaged : kLayoutRegisters;
 }
 
+// Sources, recording and grid barrier of a multi-step launch.
+StepIO step_io(const fw2_ctx *c) {
+  StepIO io{};
+  for (int k = 0; k < 3; ++k) {
+    const DevSource &d = c->dsrc[k];
+    if (d.n_tgt > 0) io.src[k] = {d.unit, d.pos, d.off, d.col};
+  }
+  io.signal = c->d_signal;
+  io.sig_cols = c->sig_cols;
+  io.sig_steps = c->sig_steps;
+  io.rec_cell = c->rec_cell;
+  io.rec_off = c->rec_off;
+  io.rec_out = c->rec_out;
+  io.rec_steps = c->rec_steps;
+  io.rec_groups = c->rec_groups;
+  io.sync = c->d_sync;
+  return io;
+}
+
+fw2_status enqueue_record(fw2_ctx *c, long long n) {
+  if (c->rec_groups > 0 && n < c->rec_steps) {
+    CK(c, launch_record(c->p, c->rec_cell, c->rec_off, c->rec_groups, c->rec_out + n * c->rec_groups, c->stream));
+    c->launches++;
+  }
+  return FW2_OK;
+}
+
+// Enqueue n_steps whole steps of a pipelined 2D context from step n: one
+// launch for all of them, then the last step's recording.
+fw2_status enqueue_steps2d(fw2_ctx *c, long long n, long long n_steps) {
+  CK(c, launch_steps2d(c->P, c->map_kind, c->n_sm, c->tm_vel, c->tm_prs, step_io(c), 2 * n, 2 * (n + n_steps),
+                       c->stream));
+  c->launches++;
+  return enqueue_record(c, n + n_steps - 1);
+}
+
 // Enqueue the launches of time step n (Sec. 3.1 order): velocity half step,
 // velocity sources (part 0), pressure half step, pressure sources,
 // recording (part 1); part -1 enqueues both, and only whole steps take part
@@ -489,6 +551,7 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
     return pipe3d_layout_allowed(vel, P, l) ? l : kLayoutRegisters;
   };
   const bool do_vel = part != 1, do_prs = part != 0;
+  const bool pipe2 = c->pipe && c->nd == 2;  // its sources are part of the half steps
   struct TrialEvents {  // destroyed on every return, error paths included
     cudaEvent_t e[4] = {nullptr, nullptr, nullptr, nullptr};
     ~TrialEvents() {
@@ -506,7 +569,8 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
   }
   if (do_vel) {
   if (trial_timed) CK(c, cudaEventRecord(te[0], c->stream));
-  CK(c, c->pipe ? (c->nd == 2 ? launch_pipe2d(true, P, c->map_kind, c->n_sm, c->tm_vel, c->stream)
+  CK(c, c->pipe ? (c->nd == 2 ? launch_steps2d(P, c->map_kind, c->n_sm, c->tm_vel, c->tm_prs, step_io(c), 2 * n,
+                                               2 * n + 1, c->stream)
                               : launch_pipe3d(true, P, c->n_sm, c->tm_vel, c->stream, lay(true)))
                 : c->nd == 2 ? launch_vel2d(P, c->map_kind, c->stream) : launch_vel3d(P, c->map_kind, c->stream));
   c->launches++;
@@ -516,7 +580,7 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
     c->ev_vel.push_back(ev);
     ev = {take_event(c), take_event(c)};
   }
-  if (n < c->sig_steps) {
+  if (!pipe2 && n < c->sig_steps) {
     for (int kind = 1; kind <= c->nd; ++kind) {
       const DevSource &d = c->dsrc[kind];
       if (d.n_tgt == 0) continue;
@@ -535,7 +599,8 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
   if (c->profiling && !do_vel) ev = {take_event(c), take_event(c)};
   if (c->profiling) CK(c, cudaEventRecord(ev.first, c->stream));
   if (trial_timed) CK(c, cudaEventRecord(te[2], c->stream));
-  CK(c, c->pipe ? (c->nd == 2 ? launch_pipe2d(false, P, c->map_kind, c->n_sm, c->tm_prs, c->stream)
+  CK(c, c->pipe ? (c->nd == 2 ? launch_steps2d(P, c->map_kind, c->n_sm, c->tm_vel, c->tm_prs, step_io(c), 2 * n + 1,
+                                               2 * n + 2, c->stream)
                               : launch_pipe3d(false, P, c->n_sm, c->tm_prs, c->stream, lay(false)))
                 : c->nd == 2 ? launch_prs2d(P, c->map_kind, c->stream) : launch_prs3d(P, c->map_kind, c->stream));
   c->launches++;
@@ -544,15 +609,12 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
     CK(c, cudaEventRecord(ev.second, c->stream));
     c->ev_prs.push_back(ev);
   }
-  if (n < c->sig_steps && c->dsrc[0].n_tgt > 0) {
+  if (!pipe2 && n < c->sig_steps && c->dsrc[0].n_tgt > 0) {
     const DevSource &d = c->dsrc[0];
     CK(c, launch_inject(c->p, d.tgt, d.off, d.col, c->d_signal + n * c->sig_cols, d.n_tgt, c->stream));
     c->launches++;
   }
-  if (c->rec_groups > 0 && n < c->rec_steps) {
-    CK(c, launch_record(c->p, c->rec_cell, c->rec_off, c->rec_groups, c->rec_out + n * c->rec_groups, c->stream));
-    c->launches++;
-  }
+  if (const fw2_status st = enqueue_record(c, n); st != FW2_OK) return st;
   if (trial > 0) {
     if (trial_timed) {
       CK(c, cudaEventSynchronize(te[3]));
@@ -753,9 +815,12 @@ fw2_status fw2_create(const fw2_config *cfg_in, fw2_ctx **out) {
     if ((st = dalloc(c, sizeof(ScanOut), &m)) == FW2_OK) c->d_scan = (ScanOut *)m;
     if (st == FW2_OK && (st = dalloc(c, sizeof(unsigned int), &m)) == FW2_OK) c->d_absmax = (unsigned int *)m;
     if (st == FW2_OK && (st = dalloc(c, sizeof(unsigned int), &m)) == FW2_OK) c->d_status = (unsigned int *)m;
+    if (st == FW2_OK && (st = dalloc(c, sizeof(unsigned long long), &m)) == FW2_OK)
+      c->d_sync = (unsigned long long *)m;
   }
   if (st == FW2_OK) {
     cudaError_t e2 = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned int), c->stream);
+    if (e2 == cudaSuccess) e2 = cudaMemsetAsync(c->d_sync, 0, sizeof(unsigned long long), c->stream);
     if (e2 != cudaSuccess) st = cuda_fail(c, e2, "status initialisation");
   }
   if (st == FW2_OK) {
@@ -982,9 +1047,21 @@ fw2_status fw2_step(fw2_ctx *c, int64_t n_steps) {
   fw2_status st;
   if ((st = finalize(c)) != FW2_OK) return st;
   if ((st = build_sources(c)) != FW2_OK) return st;
-  for (int64_t s = 0; s < n_steps; ++s) {
-    if ((st = enqueue_step(c, c->step)) != FW2_OK) return st;
-    c->step += 1;  // every launch of the step is enqueued; it counts even if a later one fails
+  // many steps a launch, up to the next scan (per-launch timing: one launch
+  // per half step)
+  const bool multi = c->pipe && c->nd == 2 && !c->profiling;
+  for (int64_t s = 0; s < n_steps;) {
+    int64_t take = 1;
+    if (multi) {
+      // at most 2^28 cell-steps (about 11 ms) and 256 steps, so that work on
+      // other streams of the device gets its turn
+      const int64_t cap = std::max<int64_t>(1, (1ll << 28) / c->n_pts);
+      take = std::min<int64_t>(n_steps - s, std::min<int64_t>(cap, 256));
+      if (c->watch_every > 0) take = std::min<int64_t>(take, c->watch_every - c->step % c->watch_every);
+    }
+    if ((st = multi ? enqueue_steps2d(c, c->step, take) : enqueue_step(c, c->step)) != FW2_OK) return st;
+    s += take;
+    c->step += take;  // every launch of the steps is enqueued; they count even if a later one fails
     if (c->watch_every > 0 && c->step % c->watch_every == 0) {
       float m = 0.f;
       if ((st = scan_p(c, &m)) != FW2_OK) return st;
@@ -1133,6 +1210,7 @@ fw2_status fw2_reset(fw2_ctx *c) {
   if (!c) return FW2_EINVAL;
   CK(c, cudaMemsetAsync(c->state, 0, c->state_bytes, c->stream));
   CK(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned int), c->stream));
+  CK(c, cudaMemsetAsync(c->d_sync, 0, sizeof(unsigned long long), c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
   c->step = 0;
   c->half = 0;

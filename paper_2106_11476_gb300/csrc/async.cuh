@@ -162,6 +162,57 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(K) : "memory");
 }
 
+// order this thread's generic accesses against async-proxy copies of the same
+// memory (global and shared), both ways: around a grid barrier, so that the
+// copies after it see what other SMs' bulk stores wrote before it
+__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;\n" ::: "memory"); }
+
+// Status word of a context: not 0 after a bounded wait gave up.
+__device__ __forceinline__ unsigned status_of(const unsigned int *status) {
+  unsigned v = 0;
+  if (status) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(status) : "memory");
+  return v;
+}
+
+// Barrier over all blocks of a cooperative launch (thread 0 of each): a
+// counter in global memory that every block adds 1 to per barrier.  It only
+// grows, by the grid size per barrier, so a launch finds its start from the
+// counter itself (this block has not arrived yet, so the counter cannot have
+// passed the next multiple) and a captured launch can be replayed.  The wait
+// is bounded like the copy waits, and ends early once another block has
+// reported a wait that gave up.
+struct GridBarrier {
+  unsigned long long *count;
+  unsigned long long target;
+  __device__ __forceinline__ void init(unsigned long long *c) {
+    count = c;
+    target = 0;
+    if (!c) return;
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(c) : "memory");
+    target = v / gridDim.x * gridDim.x;
+  }
+  __device__ __forceinline__ void arrive() {
+    target += gridDim.x;
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;\n" ::"l"(count), "l"(1ull) : "memory");
+  }
+  __device__ __forceinline__ bool reached() const {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(count) : "memory");
+    return v >= target;
+  }
+  __device__ __forceinline__ bool wait(const unsigned int *status, unsigned long long limit_ns = kWaitLimitNs) {
+    if (reached()) return true;
+    const unsigned long long t0 = global_ns();
+    for (long long polls = 0; polls < (1ll << 34); polls += 64) {
+      for (int i = 0; i < 64; ++i)
+        if (reached()) return true;
+      if (status_of(status) != 0 || global_ns() - t0 > limit_ns) return false;
+    }
+    return false;
+  }
+};
+
 __device__ __forceinline__ void report_status(unsigned int *status, unsigned bits) {
   if (status) atomicOr(status, bits);
 }

@@ -23,6 +23,10 @@ struct DevSource {
   int *off = nullptr;
   int *col = nullptr;
   int n_tgt = 0;
+  // 2D: the targets are ordered by half tile; first target of each half tile
+  // and the targets' positions in theirs (UnitSource)
+  int *unit = nullptr;
+  int *pos = nullptr;
 };
 
 inline size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -76,6 +80,7 @@ struct fw2_ctx {
   // scratch words for scans
   fw2::ScanOut *d_scan = nullptr;
   unsigned int *d_absmax = nullptr;
+  unsigned long long *d_sync = nullptr;  // grid barrier counter of the multi-step launches
   unsigned int *d_status = nullptr;  // bit 0: a bounded device-side wait gave up
   long long step = 0, launches = 0;
   // optional per-kernel event timing

@@ -164,17 +164,38 @@ cudaError_t launch_batched2d_wide(bool vel, const StepParams *Ps, const int4 *ti
 // several contexts sharing N and the map kind (vel: velocity, else pressure)
 cudaError_t launch_batched2d(bool vel, const StepParams *Ps, const int4 *tiles, int n_tiles, int n_relax,
                              int map_kind, int grid, cudaStream_t s);
-// persistent pipelined 2D half step (one block per SM: grid = SM count):
-// edge tiles by the tile path, interior half tiles staged by cp.async;
-// float maps (map_kind 0) and the tissue index (2)
+// persistent pipelined 2D half steps (one block per SM at most): float maps
+// (map_kind 0) and the tissue index (2)
 struct PipeMaps;
 bool pipe2d_supported(const StepParams &P, int map_kind);
 bool pipe2d_preferred(const StepParams &P, int map_kind);
 // encode the tensor maps of both half steps (host); cudaErrorInvalidValue
 // when the driver rejects one (message in *why)
 cudaError_t build_pipe2d_maps(const StepParams &P, int map_kind, PipeMaps *vel, PipeMaps *prs, const char **why);
-cudaError_t launch_pipe2d(bool vel, const StepParams &P, int map_kind, int grid, const PipeMaps &T,
-                          cudaStream_t s);
+// Sources of one field grouped by half tile: targets unit[u] .. unit[u + 1] - 1
+// of half tile u (numbered x fastest; null: none), target t at cell pos[t] of
+// its half tile (row * kTX + column), fed by the signal columns
+// col[off[t]] .. col[off[t + 1] - 1].
+struct UnitSource {
+  const int *unit, *pos, *off, *col;
+};
+// Sources, recording and the grid barrier of a multi-step launch.
+struct StepIO {
+  UnitSource src[3];             // p, v_x, v_y
+  const float *signal;           // [sig_steps][sig_cols]
+  long long sig_cols, sig_steps;
+  const long long *rec_cell;     // recording (rec_groups 0: none in this launch)
+  const int *rec_off;
+  float *rec_out;                // [rec_steps][rec_groups]
+  long long rec_steps;
+  int rec_groups;
+  unsigned long long *sync;      // barrier counter (GridBarrier)
+};
+// Phases ph0 .. ph1 - 1 of the time loop (2n velocity, 2n + 1 pressure half
+// step of step n, with their sources) in one launch; the recording of step n
+// runs in phase 2n + 2, so that of a launch's last step is left to the caller.
+cudaError_t launch_steps2d(const StepParams &P, int map_kind, int n_sm, const PipeMaps &vel, const PipeMaps &prs,
+                           const StepIO &io, long long ph0, long long ph1, cudaStream_t s);
 // batched form over a unit table {ctx, x0, y0, interior} of 128 x 8 half
 // tiles (no periodic context); Ps and Ts in device memory, one per context;
 // block b takes the units runs[b] .. runs[b + 1] - 1 (grid + 1 entries)

@@ -20,6 +20,8 @@
 // C-PML coefficients of each axis from its strip, and store nothing outside
 // the grid (zeros in the row padding).  Periodic grids take the tile kernels.
 // Dense float maps and the tissue-index form take this path.
+#include <numeric>
+
 #include "async.cuh"
 #include "coef.cuh"
 #include "maps.cuh"
@@ -53,10 +55,29 @@ constexpr int round32(int n) { return (n + 31) & ~31; }
 struct Region {
   int nx, ny, Lx, Ly;  // grid, boundary width (at least the halo, 4)
   int ntx, nhy;        // tiles along x, half-tile rows
-  __device__ __forceinline__ int halves() const { return ntx * nhy; }
+  unsigned inv_ntx;    // floor(2^32 / ntx), for the division by ntx
+  // Half tiles of block b of `grid`: one per round of `grid` consecutive ones,
+  // rotated by `rot` blocks from round to round.  Without the rotation a
+  // block meets few columns (grid and ntx share factors: 152 blocks and 16 or
+  // 32 columns), and those at the x edges, whose half tiles take longer, hold
+  // up the rest: 2048 x 1024 cells of the index form took 90 us a step
+  // without it and 78 us with it.
+  int rot;
+  __host__ __device__ __forceinline__ int halves() const { return ntx * nhy; }
+  __device__ __forceinline__ int slot(int round, int b, int grid) const {
+    return (int)((b + (unsigned)round * (unsigned)rot) % (unsigned)grid);
+  }
+  __device__ __forceinline__ int rounds(int b, int grid) const {
+    const int full = halves() / grid;
+    return full + (slot(full, b, grid) < halves() - full * grid ? 1 : 0);
+  }
   __device__ __forceinline__ void half_origin(int h, int &x0, int &y0) const {
-    x0 = (h % ntx) * kTX;
-    y0 = (h / ntx) * kHT;
+    // the product's high word is at most two below the quotient
+    int q = (int)__umulhi((unsigned)h, inv_ntx), r = h - q * ntx;
+    if (r >= ntx) { ++q; r -= ntx; }
+    if (r >= ntx) { ++q; r -= ntx; }
+    x0 = r * kTX;
+    y0 = q * kHT;
   }
   // a half tile clear of the boundary rules and of the C-PML strips
   __device__ __forceinline__ bool interior(int x0, int y0) const {
@@ -116,17 +137,19 @@ __host__ __device__ constexpr unsigned stage_bytes(bool nl, bool nl_vel) {
   }
 }
 
-// Issue the tensor copies of one half tile into a stage (one thread; it
-// first announces the stage's bytes on the stage's mbarrier).  Boxes may
-// reach outside the grid: those cells read as zero.
+// The tensor copies of one half tile into a stage, in two parts (one thread;
+// the first announces the stage's bytes on the stage's mbarrier).  The first
+// part holds what only this half tile's own block writes (the updated arrays)
+// and the maps; the second the stencil operand, which the neighbouring half
+// tiles of the previous half step wrote.  Boxes may reach outside the grid:
+// those cells read as zero.
 template <int N, typename Maps, bool VEL>
-__device__ __forceinline__ void issue_stage(const StepParams &P, const PipeMaps &T, float *st, uint64_t *bar,
-                                            int x0, int y0) {
+__device__ __forceinline__ void issue_own(const StepParams &P, const PipeMaps &T, float *st, uint64_t *bar, int x0,
+                                          int y0) {
   fence_proxy_async_smem();
   mbar_arrive_expect_tx(bar, stage_bytes<N, Maps, VEL>(P.nl != 0, P.nl_vel != 0));
   if (VEL) {
     using S = VelStage<N, Maps>;
-    tma_load_2d(st, &T.m[0], x0 - 4, y0 - 3, bar);
     if (!S::kIdx) tma_load_2d(st + S::kP, &T.m[1], x0, y0, bar);
     float *ss = st + S::kP + S::kR;
     tma_load_2d(ss, &T.m[2], x0, y0, bar);
@@ -147,8 +170,6 @@ __device__ __forceinline__ void issue_stage(const StepParams &P, const PipeMaps 
     }
   } else {
     using S = PrsStage<N, Maps>;
-    tma_load_2d(st, &T.m[0], x0 - 4, y0 - 1, bar);
-    tma_load_2d(st + S::kX, &T.m[1], x0 - 4, y0 - 4, bar);
     float *ss = st + S::kX + S::kY;
     tma_load_2d(ss, &T.m[2], x0, y0, bar);
     if (N > 0) {
@@ -167,6 +188,21 @@ __device__ __forceinline__ void issue_stage(const StepParams &P, const PipeMaps 
       tma_load_2d(ss + S::kS, &T.m[5], x0, y0, bar);  // tissue index
     }
   }
+}
+template <int N, typename Maps, bool VEL>
+__device__ __forceinline__ void issue_operand(const PipeMaps &T, float *st, uint64_t *bar, int x0, int y0) {
+  if (VEL) {
+    tma_load_2d(st, &T.m[0], x0 - 4, y0 - 3, bar);
+  } else {
+    tma_load_2d(st, &T.m[0], x0 - 4, y0 - 1, bar);
+    tma_load_2d(st + PrsStage<N, Maps>::kX, &T.m[1], x0 - 4, y0 - 4, bar);
+  }
+}
+template <int N, typename Maps, bool VEL>
+__device__ __forceinline__ void issue_stage(const StepParams &P, const PipeMaps &T, float *st, uint64_t *bar,
+                                            int x0, int y0) {
+  issue_own<N, Maps, VEL>(P, T, st, bar, x0, y0);
+  issue_operand<N, Maps, VEL>(T, st, bar, x0, y0);
 }
 
 // Store the updated arrays of a half tile from its stage (one thread, after
@@ -640,99 +676,312 @@ struct Ring {
   static_assert(kBytes + 1024 <= 227 * 1024, "stages and table leave 1 KB for static shared memory");
 };
 
-// One half step.  Block (32, 16), one per SM.
+// Ring of the multi-step kernel: stages that hold either half step's half
+// tile, as many as fit (2 .. 4).
+template <int N, typename Maps>
+struct StepRing {
+  static constexpr int kV = VelStage<N, Maps>::kFloats, kP = PrsStage<N, Maps>::kFloats;
+  static constexpr int kStage = kV > kP ? kV : kP;
+  static constexpr int kBudget = (224 * 1024 - 128) / 4 - Maps::kSmemFloats;  // floats
+  static constexpr int kFit = kBudget / kStage;
+  static constexpr int kStages = kFit > 4 ? 4 : kFit;
+  static constexpr int kLag = kStages >= 4 ? 1 : 0;  // as Ring
+  static constexpr int kAhead = kStages - 1 - kLag;
+  static constexpr size_t kBytes = sizeof(float) * ((size_t)kStages * kStage + Maps::kSmemFloats) + 128;
+  static_assert(kStages >= 2, "two stages must fit in shared memory");
+  static_assert(kBytes + 1024 <= 227 * 1024, "stages and table leave 1 KB for static shared memory");
+};
+
+// Which of a block's half tiles hold sources, per half step: one bit per
+// round, looked up once per launch (a load per half tile in the loop would
+// put a memory latency on every one of them).  Rounds beyond the bitmap are
+// looked up each time.
+constexpr int kSrcWords = 64;
+struct SourceBits {
+  unsigned w[2][kSrcWords];
+  __device__ __forceinline__ bool get(int half, int round) const {
+    return round >= 32 * kSrcWords || ((w[half][round >> 5] >> (round & 31)) & 1u);
+  }
+};
+__device__ __forceinline__ void mark_sources(const StepIO &io, const Region &R, int per, SourceBits &bits, int tid) {
+  for (int i = tid; i < 2 * kSrcWords; i += kThreads) (&bits.w[0][0])[i] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    const int *unit = io.src[f].unit;
+    if (!unit) continue;
+    for (int r = tid; r < per && r < 32 * kSrcWords; r += kThreads) {
+      const int u = r * (int)gridDim.x + R.slot(r, blockIdx.x, gridDim.x);
+      if (__ldg(unit + u) < __ldg(unit + u + 1)) atomicOr(&bits.w[f == 0 ? 1 : 0][r >> 5], 1u << (r & 31));
+    }
+  }
+}
+
+// Add the sources of a half tile to its updated arrays in the stage (every
+// thread, after the results of all threads are there): the entries of a
+// target summed in their order, then added, as inject_kernel does.
 template <int N, typename Maps, bool VEL>
+__device__ __forceinline__ void inject_unit(const StepIO &io, int u, long long n, float *st, int tid) {
+  const float *row = io.signal + n * io.sig_cols;
+  float *ss = VEL ? st + VelStage<N, Maps>::kP + VelStage<N, Maps>::kR
+                  : st + PrsStage<N, Maps>::kX + PrsStage<N, Maps>::kY;
+#pragma unroll
+  for (int a = 0; a < (VEL ? 2 : 1); ++a) {
+    const UnitSource &src = io.src[VEL ? 1 + a : 0];
+    if (!src.unit) continue;
+    const int e = __ldg(src.unit + u + 1);
+    for (int t = __ldg(src.unit + u) + tid; t < e; t += kThreads) {
+      float v = 0.f;
+      for (int c = src.off[t]; c < src.off[t + 1]; ++c) v += __ldg(row + src.col[c]);
+      ss[a * kArr + src.pos[t]] += v;
+    }
+  }
+}
+
+// Trace row of one step, groups spread over the blocks' last threads: the
+// mean of p over a group's cells, summed in their order.  p was written by
+// other SMs during this launch: read through L2, eight loads in flight.
+__device__ __forceinline__ void record_row(const StepIO &io, const float *p, long long n, int tid) {
+  for (int g = blockIdx.x + (kThreads - 1 - tid) * gridDim.x; g < io.rec_groups; g += kThreads * gridDim.x) {
+    const int b = __ldg(io.rec_off + g), e = __ldg(io.rec_off + g + 1);
+    float s = 0.f;
+    for (int i = b; i < e; i += 8) {
+      float v[8];
+#pragma unroll
+      for (int m = 0; m < 8; ++m) v[m] = i + m < e ? __ldcg(p + __ldg(io.rec_cell + i + m)) : 0.f;
+#pragma unroll
+      for (int m = 0; m < 8; ++m)
+        if (i + m < e) s += v[m];
+    }
+    io.rec_out[n * io.rec_groups + g] = e > b ? s / (float)(e - b) : 0.f;
+  }
+}
+
+// Phases ph0 .. ph1 - 1 of the time loop in one launch (phase 2n: velocity
+// half step of step n with its v sources, 2n + 1: pressure half step with its
+// p sources; the recording of step n runs in phase 2n + 2).  Block (32, 16),
+// one per SM; more than one phase needs a cooperative launch, since the
+// blocks wait for one another between phases.
+//
+// What bounds it: HBM on grids beyond L2 (4096^2, N = 4: 690 us a step, 0.88
+// of the copy bandwidth on the step's bytes), the latency chain of a phase
+// (operand copy, compute, store, grid barrier: about 5 us) on small ones.
+// Four launches per step (two half steps, sources, recording) added to every
+// one of them a start and a drain and left the SMs without copies in flight
+// meanwhile; here the next phase's first half tiles are copied (all but the
+// operand) while the barrier is under way, and sources and recording need no
+// launch of their own.  A step of 250 x 186 (N = 2) took 21 us and takes 11,
+// 512^2 (N = 4) 30 and 19.5, 1501 x 1237 111 and 98.  The velocity phases walk
+// the half tiles forwards and the pressure phases backwards, so each starts on
+// the rows whose operand the previous one left in L2 (0.8 % at 1501 x 1237).
+template <int N, typename Maps>
 __global__ void __launch_bounds__(kThreads, 1)
-    pipe2d_kernel(const StepParams P, const Region R, const __grid_constant__ PipeMaps T) {
-  using G = Ring<N, Maps, VEL>;
+    steps2d_kernel(const StepParams P, const Region R, const __grid_constant__ PipeMaps TV,
+                   const __grid_constant__ PipeMaps TP, const StepIO io, const long long ph0, const long long ph1) {
+  using G = StepRing<N, Maps>;
   constexpr int kS = G::kStages, kStage = G::kStage;
   extern __shared__ __align__(128) float smem_raw[];
   __shared__ __align__(8) uint64_t bar[kS];
   __shared__ int ok[kS];  // per stage: thread 0 never rewrites a flag a thread has yet to read
+  __shared__ int synced;
+  __shared__ SourceBits sources;
   // TMA destinations need 128-byte alignment: round the base up (the launch
   // adds 128 bytes of slack)
   float *smem = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   float *tab = smem + kS * kStage;
   const int tid = threadIdx.y * 32 + threadIdx.x;
   stage_table<Maps>(P, tab, tid);  // made visible by the barrier below
+  GridBarrier gb;
   if (tid == 0) {
     for (int q = 0; q < kS; ++q) mbar_init(&bar[q], 1);
     fence_mbarrier_init();
+    gb.init(io.sync);
+    // after a wait that gave up the state is incomplete: nothing runs until
+    // the status is cleared
+    synced = ph1 - ph0 > 1 ? (status_of(P.status) == 0) : 1;
   }
   __syncthreads();
-  const int nh = R.halves();
-  int h = blockIdx.x;
-  if (h >= nh) return;
-  // this block's half tiles are h, h + grid, ...; the first kS - 1 go out now,
-  // then each iteration issues one more into the stage freed last
-  unsigned phase = 0;    // bit q: parity of the next completion of stage q
-  unsigned pending = 0;  // bit q: copies issued into stage q, not consumed
-  int hs = h;            // next half tile to issue
-  for (int q = 0; q < G::kAhead; ++q, hs += gridDim.x) {
-    if (hs >= nh) break;
-    if (tid == 0) {
-      int xq, yq;
-      R.half_origin(hs, xq, yq);
-      issue_stage<N, Maps, VEL>(P, T, smem + q * kStage, &bar[q], xq, yq);
+  if (!synced) return;
+  // this block's half tiles in every phase (at least one: grid <= half tiles)
+  const int grid = (int)gridDim.x;
+  const int per = R.rounds(blockIdx.x, grid);
+  const int last_slot = R.slot(per - 1, blockIdx.x, grid);
+  mark_sources(io, R, per, sources, tid);  // made visible by the barrier of the first half tile
+  unsigned phase = 0;     // bit q: parity of the next completion of stage q
+  unsigned pending = 0;   // bit q: copies issued into stage q, not consumed
+  unsigned deferred = 0;  // bit q: the operand copy of stage q waits for the grid barrier
+  int ahead = 0;          // jobs issued and not consumed
+  // the half tile of each stage's job: origin and round
+  int jx[kS], jy[kS], jr[kS];
+  auto at = [&](const int (&a)[kS], int q) {
+    int v = a[0];
+#pragma unroll
+    for (int m = 1; m < kS; ++m) v = q == m ? a[m] : v;
+    return v;
+  };
+  // the next job to issue: phase, round, slot, origin (worked out before it is
+  // needed: thread 0 issues between two barriers) and stage
+  long long iph = ph0;
+  int is = 0, ir = (ph0 & 1) ? per - 1 : 0, islot = (ph0 & 1) ? last_slot : (int)blockIdx.x, ix, iy;
+  R.half_origin(ir * grid + islot, ix, iy);
+  auto advance = [&] {
+    if (iph & 1) {
+      if (ir == 0) {
+        ++iph;  // the velocity phase starts where this one ended
+      } else {
+        --ir;
+        islot -= R.rot;
+        if (islot < 0) islot += grid;
+      }
+    } else if (ir == per - 1) {
+      ++iph;
+    } else {
+      ++ir;
+      islot += R.rot;
+      if (islot >= grid) islot -= grid;
     }
-    pending |= 1u << q;
+    R.half_origin(ir * grid + islot, ix, iy);
+  };
+  auto issue_next = [&](long long ph) {  // every thread keeps the bookkeeping, thread 0 issues
+    if (tid < 32) {
+      if (tid == 0) {
+        float *st = smem + is * kStage;
+        if (iph & 1) issue_own<N, Maps, false>(P, TP, st, &bar[is], ix, iy);
+        else issue_own<N, Maps, true>(P, TV, st, &bar[is], ix, iy);
+        if (iph == ph) {
+          if (iph & 1) issue_operand<N, Maps, false>(TP, st, &bar[is], ix, iy);
+          else issue_operand<N, Maps, true>(TV, st, &bar[is], ix, iy);
+        }
+      }
+      if (!R.interior(ix, iy)) {
+        if (iph & 1) prefetch_strips2<N, 2>(P, ix, iy, tid);
+        else prefetch_strips2<N, 1>(P, ix, iy, tid);
+      }
+    }
+    pending |= 1u << is;
+    if (iph != ph) deferred |= 1u << is;
+#pragma unroll
+    for (int q = 0; q < kS; ++q)
+      if (q == is) {
+        jx[q] = ix;
+        jy[q] = iy;
+        jr[q] = ir;
+      }
+    is = is + 1 == kS ? 0 : is + 1;
+    ++ahead;
+  };
+  auto issue_deferred = [&](long long ph) {  // thread 0, the operands of phase ph
+#pragma unroll
+    for (int q = 0; q < kS; ++q)
+      if ((deferred >> q) & 1u) {
+        if (ph & 1) issue_operand<N, Maps, false>(TP, smem + q * kStage, &bar[q], jx[q], jy[q]);
+        else issue_operand<N, Maps, true>(TV, smem + q * kStage, &bar[q], jx[q], jy[q]);
+      }
+  };
+  // a wait gave up: let this block's copies land (a stage whose operand was
+  // still held back gets it, so that its barrier can complete)
+  auto give_up = [&](long long ph, int s) {
+    if (tid != 0) return;
+    report_status(P.status, kStatusWaitTimeout);
+    issue_deferred(ph + 1);
+    for (int q = 0; q < kS; ++q)
+      if (q != s && ((pending >> q) & 1u)) mbar_wait_bounded(&bar[q], (phase >> q) & 1u);
+    bulk_wait_all();
+  };
+  // the first copies into every stage; a job may be issued up to one phase
+  // ahead (what a later phase updates is still being written)
+  while (ahead < kS && iph < ph1 && iph <= ph0 + 1) {
+    issue_next(ph0);
+    advance();
   }
-  int s = 0;
-  // One barrier per half tile: after the wait for stage s it also marks
-  // the previous half tile computed, so its stage is refilled (and, with
-  // TMA stores, its results sent) right after it.
-  int xp = -1, yp = -1;  // previous half tile of this block
+  long long ph = ph0;
+  int i = 0, s = 0;
+  int xp = -1, yp = -1;  // previous half tile of this block in this phase
 #pragma unroll 1
-  for (; h < nh; h += gridDim.x) {
+  while (true) {
+    // One barrier per half tile: after the wait for stage s it also marks the
+    // previous half tile computed, so its results are sent and a freed stage
+    // is refilled right after it.
     if (tid == 0) ok[s] = mbar_wait_bounded(&bar[s], (phase >> s) & 1u);
     __syncthreads();
     if (!ok[s]) {
-      if (tid == 0) {
-        report_status(P.status, kStatusWaitTimeout);
-        for (int q = 0; q < kS; ++q)
-          if (q != s && ((pending >> q) & 1u)) mbar_wait_bounded(&bar[q], (phase >> q) & 1u);
-        bulk_wait_all();
-      }
+      give_up(ph, s);
       return;
     }
     phase ^= 1u << s;
     pending &= ~(1u << s);
-    const int sp = (s + kS - 1) % kS;       // the previous half tile's stage
-    const int q = (s + G::kAhead) % kS;     // the stage refilled now
-    if constexpr (TmaStore<Maps>::value) {
-      if (tid == 0 && xp >= 0) store_stage<N, Maps, VEL>(T, smem + sp * kStage, xp, yp);
+    --ahead;
+    const bool vel = (ph & 1) == 0;
+    const int sp = (s + kS - 1) % kS;  // the previous half tile's stage
+    if (tid == 0 && xp >= 0) {
+      if (vel) store_stage<N, Maps, true>(TV, smem + sp * kStage, xp, yp);
+      else store_stage<N, Maps, false>(TP, smem + sp * kStage, xp, yp);
     }
-    if (hs < nh) {
-      if (tid < 32) {
-        int xq, yq;
-        R.half_origin(hs, xq, yq);
-        if (tid == 0) {
-          bulk_wait_read<G::kLag>();
-          issue_stage<N, Maps, VEL>(P, T, smem + q * kStage, &bar[q], xq, yq);
-        }
-        if (!R.interior(xq, yq)) prefetch_strips2<N, VEL ? 1 : 2>(P, xq, yq, tid);
-      }
-      pending |= 1u << q;
-      hs += gridDim.x;
+    const int x0 = at(jx, s), y0 = at(jy, s), round = at(jr, s);
+    const bool refill = ahead < G::kAhead && iph < ph1 && iph <= ph + 1;
+    if (refill) {
+      if (tid == 0) bulk_wait_read<G::kLag>();
+      issue_next(ph);
+      advance();
     }
-    int x0, y0;
-    R.half_origin(h, x0, y0);
     float *cur = smem + s * kStage;
     if (R.interior(x0, y0)) {
-      if (VEL) vel_compute<N, Maps, false>(P, tab, cur, x0, y0, tid);
+      if (vel) vel_compute<N, Maps, false>(P, tab, cur, x0, y0, tid);
       else prs_compute<N, Maps, false>(P, tab, cur, x0, y0, tid);
     } else {
-      if (VEL) vel_compute<N, Maps, true>(P, tab, cur, x0, y0, tid);
+      if (vel) vel_compute<N, Maps, true>(P, tab, cur, x0, y0, tid);
       else prs_compute<N, Maps, true>(P, tab, cur, x0, y0, tid);
     }
-    if constexpr (TmaStore<Maps>::value) fence_proxy_async_smem();
+    if ((ph >> 1) < io.sig_steps && sources.get((int)(ph & 1), round)) {
+      const int u = round * grid + R.slot(round, blockIdx.x, grid);
+      __syncthreads();
+      if (vel) inject_unit<N, Maps, true>(io, u, ph >> 1, cur, tid);
+      else inject_unit<N, Maps, false>(io, u, ph >> 1, cur, tid);
+    }
+    fence_proxy_async_smem();
     xp = x0;
     yp = y0;
-    s = (s + 1) % kS;
-  }
-  if constexpr (TmaStore<Maps>::value) {
+    s = s + 1 == kS ? 0 : s + 1;
+    if (++i < per) continue;
+    // ---- end of the phase
     __syncthreads();
-    if (tid == 0 && xp >= 0) store_stage<N, Maps, VEL>(T, smem + ((s + kS - 1) % kS) * kStage, xp, yp);
+    if (tid == 0) {
+      const int sl = (s + kS - 1) % kS;
+      if (vel) store_stage<N, Maps, true>(TV, smem + sl * kStage, xp, yp);
+      else store_stage<N, Maps, false>(TP, smem + sl * kStage, xp, yp);
+    }
+    if (ph + 1 == ph1) break;
+    if (tid == 0) {
+      bulk_wait_all();  // this block's results are in memory
+      fence_proxy_async_all();
+      gb.arrive();
+    }
+    // copies of the next phase's first half tiles, into every stage (none is
+    // being computed), while the other blocks arrive
+    while (ahead < kS && iph < ph1 && iph <= ph + 1) {
+      issue_next(ph);
+      advance();
+    }
+    if (tid == 0) {
+      synced = gb.wait(P.status);
+      fence_proxy_async_all();
+    }
+    __syncthreads();
+    if (!synced) {
+      give_up(ph, -1);
+      return;
+    }
+    ++ph;
+    if (tid == 0) issue_deferred(ph);
+    deferred = 0;
+    if (!(ph & 1) && io.rec_groups > 0 && (ph >> 1) - 1 < io.rec_steps) record_row(io, P.p, (ph >> 1) - 1, tid);
+    // jobs that were held back for being two phases ahead
+    while (ahead < kS && iph < ph1 && iph <= ph + 1) {
+      issue_next(ph);
+      advance();
+    }
+    i = 0;
+    xp = -1;
   }
   if (tid == 0) bulk_wait_all();
 }
@@ -875,36 +1124,53 @@ cudaError_t pipe_batched_dispatch(const StepParams *Ps, const PipeMaps *Ts, cons
   }
 }
 
-template <int N, typename Maps, bool VEL>
-cudaError_t pipe_launch(const StepParams &P, const Region &R, int grid, const PipeMaps &T, cudaStream_t st) {
-  constexpr size_t bytes = Ring<N, Maps, VEL>::kBytes;
-  cudaError_t e = cudaFuncSetAttribute(pipe2d_kernel<N, Maps, VEL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)bytes);
+template <int N, typename Maps>
+cudaError_t steps_launch(const StepParams &P, const Region &R, int grid, const PipeMaps &TV, const PipeMaps &TP,
+                         const StepIO &io, long long ph0, long long ph1, cudaStream_t st) {
+  constexpr size_t bytes = StepRing<N, Maps>::kBytes;
+  cudaError_t e = cudaFuncSetAttribute(steps2d_kernel<N, Maps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
-  pipe2d_kernel<N, Maps, VEL><<<grid, dim3(32, kThreads / 32), bytes, st>>>(P, R, T);
-  return cudaGetLastError();
+  const dim3 block(32, kThreads / 32);
+  if (ph1 - ph0 == 1) {
+    steps2d_kernel<N, Maps><<<grid, block, bytes, st>>>(P, R, TV, TP, io, ph0, ph1);
+    return cudaGetLastError();
+  }
+  // the blocks wait for one another: all of them resident together
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, steps2d_kernel<N, Maps>, P, R, TV, TP, io, ph0, ph1);
 }
 
-template <typename Maps, bool VEL>
-cudaError_t pipe_dispatch(const StepParams &P, const Region &R, int grid, const PipeMaps &T, cudaStream_t st) {
+template <typename Maps>
+cudaError_t steps_dispatch(const StepParams &P, const Region &R, int grid, const PipeMaps &TV, const PipeMaps &TP,
+                           const StepIO &io, long long ph0, long long ph1, cudaStream_t st) {
   switch (P.n_relax) {
-    case 0: return pipe_launch<0, Maps, VEL>(P, R, grid, T, st);
-    case 1: return pipe_launch<1, Maps, VEL>(P, R, grid, T, st);
-    case 2: return pipe_launch<2, Maps, VEL>(P, R, grid, T, st);
-    case 3: return pipe_launch<3, Maps, VEL>(P, R, grid, T, st);
-    case 4: return pipe_launch<4, Maps, VEL>(P, R, grid, T, st);
+    case 0: return steps_launch<0, Maps>(P, R, grid, TV, TP, io, ph0, ph1, st);
+    case 1: return steps_launch<1, Maps>(P, R, grid, TV, TP, io, ph0, ph1, st);
+    case 2: return steps_launch<2, Maps>(P, R, grid, TV, TP, io, ph0, ph1, st);
+    case 3: return steps_launch<3, Maps>(P, R, grid, TV, TP, io, ph0, ph1, st);
+    case 4: return steps_launch<4, Maps>(P, R, grid, TV, TP, io, ph0, ph1, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
 Region region_of(const StepParams &P) {
-  Region R;
+  Region R{};
   R.nx = P.nx;
   R.ny = P.ny;
   R.Lx = P.L[0] > 4 ? P.L[0] : 4;
   R.Ly = P.L[1] > 4 ? P.L[1] : 4;
   R.ntx = (P.nx + kTX - 1) / kTX;
   R.nhy = (P.ny + kHT - 1) / kHT;
+  R.inv_ntx = R.ntx == 1 ? 0xffffffffu : (unsigned)((1ull << 32) / R.ntx);
   return R;
 }
 
@@ -936,14 +1202,15 @@ cudaError_t launch_pipe2d_batched(bool vel, const StepParams *Ps, const PipeMaps
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_pipe2d(bool vel, const StepParams &P, int map_kind, int grid, const PipeMaps &T,
-                          cudaStream_t st) {
-  const Region R = region_of(P);
-  if (map_kind == 2)
-    return vel ? pipe_dispatch<IdxMaps, true>(P, R, grid, T, st) : pipe_dispatch<IdxMaps, false>(P, R, grid, T, st);
-  if (map_kind == 0)
-    return vel ? pipe_dispatch<DenseMaps<float>, true>(P, R, grid, T, st)
-               : pipe_dispatch<DenseMaps<float>, false>(P, R, grid, T, st);
+cudaError_t launch_steps2d(const StepParams &P, int map_kind, int n_sm, const PipeMaps &vel, const PipeMaps &prs,
+                           const StepIO &io, long long ph0, long long ph1, cudaStream_t st) {
+  Region R = region_of(P);
+  const long long nh = (long long)R.ntx * R.nhy;
+  const int grid = (int)(nh < n_sm ? nh : n_sm);
+  // a round advances every block by grid + rot columns: all columns in turn
+  while (R.rot + 1 < grid && std::gcd(grid + R.rot, R.ntx) != 1) ++R.rot;
+  if (map_kind == 2) return steps_dispatch<IdxMaps>(P, R, grid, vel, prs, io, ph0, ph1, st);
+  if (map_kind == 0) return steps_dispatch<DenseMaps<float>>(P, R, grid, vel, prs, io, ph0, ph1, st);
   return cudaErrorInvalidValue;
 }
 

@@ -1,0 +1,75 @@
+"""Many time steps in one launch (2D pipelined path) against the same steps
+taken half step by half step and against the tile kernels: the same bits.
+
+The sizes cover one half tile, fewer half tiles than SMs, one round and a
+ragged last round over the SMs, column counts that share factors with the SM
+count, launches longer than the cap on steps per launch, several sources in
+one cell and sensor groups across half tiles."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fw2(fw2lib):
+    from paper_2106_11476_gb300 import fw2 as m
+    return m
+
+
+def problem(nx, ny, N, nl, steps, seed=0):
+    rng = np.random.default_rng(seed)
+    sets = {0: None, 2: "N2_y1.0_a0.5", 3: "N3_y1.2_brain", 4: "N4_y1.1_a0.5"}[N]
+    prob = synth.homogeneous((nx, ny), 1e-4, 0.0, relax=synth.relaxation_sets()[sets] if sets else None, beta=4.0)
+    g = prob.grid_shape
+    prob.c = (1500 + 100 * rng.random(g)).astype(np.float32)
+    prob.rho = (1000 + 100 * rng.random(g)).astype(np.float32)
+    prob.nl_mode = nl
+    prob.dt = 0.3 * 1e-4 / 2200.0
+    if N and min(nx, ny) >= 16:
+        prob.pml_transition, prob.pml_bound = 5, 3
+    # twelve cells of p (one of them twice) and, in v_x, v_y, a row and a column
+    cells = rng.choice(nx * ny, size=min(12, nx * ny), replace=False).astype(np.int64)
+    cells = np.concatenate([cells, cells[:1]])
+    sig = rng.standard_normal((steps - 2, 3)).astype(np.float32)     # silent for the last two steps
+    row, col = np.arange(nx, dtype=np.int64) + nx * (ny // 2), np.arange(ny, dtype=np.int64) * nx + nx // 3
+    prob.sources = [synth.Source("p", cells, (np.arange(cells.size) % 3).astype(np.int32), 1e3 * sig),
+                    synth.Source("vx", row, np.zeros(row.size, np.int32), 1e-3 * sig[:, :1]),
+                    synth.Source("vy", col, np.zeros(col.size, np.int32), 1e-3 * sig[:, 1:2])]
+    k = min(40, nx * ny)
+    prob.sensors = synth.Sensors(idx=rng.choice(nx * ny, size=k, replace=False).astype(np.int64),
+                                 group=np.sort(rng.integers(0, 5, k)).astype(np.int32), n_groups=5)
+    prob.n_steps = steps - 1                                          # the last step has no trace row
+    return prob
+
+
+def run(fw2, prob, steps, how, path="auto"):
+    sim = fw2.Simulation(prob, kernel_path=path)
+    sim.set_state(synth.random_state(prob, seed=4))
+    if how == "steps":
+        sim.step(steps)
+    else:
+        for _ in range(steps):
+            fw2.fw2_step_part(sim.ctx, 0)
+            fw2.fw2_step_part(sim.ctx, 1)
+    sim.synchronize()
+    names = ["p", "vx", "vy"] + (["psi1x", "psi1y", "psi2x", "psi2y"] if prob.nrelax else [])
+    out = {n: sim.field(n) for n in names}
+    out["trace"] = sim.trace.cpu().numpy()
+    sim.close()
+    return out
+
+
+@pytest.mark.parametrize("nx,ny,N,nl,steps", [
+    (8, 8, 0, "off", 7), (120, 8, 2, "pressure", 7), (129, 9, 4, "literal", 7), (300, 200, 2, "westervelt", 9),
+    (512, 304, 3, "off", 9), (1100, 515, 4, "pressure", 5), (2048, 160, 2, "off", 5), (64, 40, 2, "off", 519)])
+def test_steps_in_one_launch_equal_half_steps_bitwise(fw2, nx, ny, N, nl, steps):
+    prob = problem(nx, ny, N, nl, steps)
+    ref = run(fw2, prob, steps, "steps", path="tile")
+    assert np.abs(ref["p"]).max() > 0 and np.isfinite(ref["p"]).all()
+    for how in ("steps", "parts"):
+        got = run(fw2, prob, steps, how)
+        for n, want in ref.items():
+            np.testing.assert_array_equal(got[n], want, err_msg=f"{how}: {n}")
