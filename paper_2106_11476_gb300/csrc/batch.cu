@@ -346,7 +346,7 @@ fw2_status build_tables(fw2_batch *b) {
     // the pipelined form when every member allows it
     g.pipe = true;
     for (const StepParams &P : params)
-      if (!pipe2d_supported(P, g.map_kind) || P.periodic[0] || P.periodic[1]) g.pipe = false;
+      if (!pipe2d_batched_supported(P, g.map_kind)) g.pipe = false;
     if (g.pipe) {
       std::vector<PipeMaps> mv(params.size()), mp(params.size());
       std::vector<int4> units;

@@ -164,11 +164,12 @@ cudaError_t launch_batched2d_wide(bool vel, const StepParams *Ps, const int4 *ti
 // several contexts sharing N and the map kind (vel: velocity, else pressure)
 cudaError_t launch_batched2d(bool vel, const StepParams *Ps, const int4 *tiles, int n_tiles, int n_relax,
                              int map_kind, int grid, cudaStream_t s);
-// persistent pipelined 2D half steps (one block per SM at most): float maps
-// (map_kind 0) and the tissue index (2)
+// persistent pipelined 2D half steps (one block per SM at most): every map
+// form, the uint16 index while its tables fit in shared memory
 struct PipeMaps;
 bool pipe2d_supported(const StepParams &P, int map_kind);
 bool pipe2d_preferred(const StepParams &P, int map_kind);
+bool pipe2d_batched_supported(const StepParams &P, int map_kind);  // the batched form: float and uint8 index
 // encode the tensor maps of both half steps (host); cudaErrorInvalidValue
 // when the driver rejects one (message in *why)
 cudaError_t build_pipe2d_maps(const StepParams &P, int map_kind, PipeMaps *vel, PipeMaps *prs, const char **why);

@@ -21,6 +21,7 @@
 // the grid (zeros in the row padding).  Periodic grids take the tile kernels.
 // Dense float maps and the tissue-index form take this path.
 #include <numeric>
+#include <type_traits>
 
 #include "async.cuh"
 #include "coef.cuh"
@@ -33,22 +34,44 @@ namespace {
 
 constexpr int kHT = 8;              // rows of a half tile
 constexpr int kCW = kTX + 8;        // staged operand columns x0-4 .. x0+TX+3 (= kPW)
-constexpr int kRWp = kTX + 4;       // density tile columns x0 .. x0+TX+3 (= kRW)
-constexpr int kIW = kTX + 16;       // staged index bytes per row x0 .. x0+TX+15
 constexpr int kArr = kHT * kTX;     // floats of one streamed array per half tile
 
 
+// Storage of a map form: dense maps of type MT (float, bf16 or FP16), or a
+// tissue index of type IT per cell.
 template <typename Maps>
-struct IsIdx {
-  static constexpr bool value = false;
+struct Form;
+template <typename T>
+struct Form<DenseMaps<T>> {
+  static constexpr bool kIdx = false;
+  using MT = T;
+  using IT = unsigned char;
 };
 template <>
-struct IsIdx<IdxMaps> {
-  static constexpr bool value = true;
+struct Form<IdxMaps> {
+  static constexpr bool kIdx = true;
+  using MT = float;
+  using IT = unsigned char;
 };
+template <>
+struct Form<IdxMaps16> {
+  static constexpr bool kIdx = true;
+  using MT = float;
+  using IT = unsigned short;
+};
+template <typename Maps>
+constexpr bool kWideIdx = std::is_same<Maps, IdxMaps16>::value;
+// columns of a box one cell wider than a half tile, rows of 16 bytes: the
+// density (and K) box x0 .. x0+TX+3 (float) or x0+TX+7 (16 bits), the index
+// box x0 .. x0+TX+15 (uint8) or x0+TX+7 (uint16)
+template <typename T>
+constexpr int kWide = kTX + (sizeof(T) == 1 ? 16 : sizeof(T) == 2 ? 8 : 4);
+// floats that n elements of T take
+template <typename T>
+__host__ __device__ constexpr int floats_of(int n) { return (n * (int)sizeof(T) + 3) / 4; }
 
 // shared-memory regions start on 128-byte boundaries (TMA destinations)
-constexpr int round32(int n) { return (n + 31) & ~31; }
+__host__ __device__ constexpr int round32(int n) { return (n + 31) & ~31; }
 
 // Work of one launch: the half tiles of the grid (tiles of 128 x 8 cells,
 // x fastest).
@@ -86,39 +109,42 @@ struct Region {
 };
 
 // ---------------------------------------------------------------- stages ---
-// velocity: operand p rows y0-3 .. y0+kHT+3; density tile rows y0 .. y0+kHT;
-// streamed arrays [ns][kHT][kTX]; tissue bytes rows y0 .. y0+kHT (index form)
+// velocity: operand p rows y0-3 .. y0+kHT+3; density box rows y0 .. y0+kHT;
+// float arrays [k32][kHT][kTX]; map arrays [kM][kHT][kTX] (dense) or the
+// index box rows y0 .. y0+kHT; K box (dense, literal nonlinear system)
 template <int N, typename Maps>
 struct VelStage {
-  static constexpr bool kIdx = IsIdx<Maps>::value;
-  // dense: v_x, v_y, psi_x[N], psi_y[N], 1/kappa1, a1[N], b1[N];
-  // index: v_x, v_y, psi_x[N], psi_y[N]
-  static constexpr int kNs = kIdx ? 2 + 2 * N : 3 + 4 * N;
-  static constexpr int kPb = (kHT + 7) * kCW;    // operand box
-  static constexpr int kRb = (kHT + 1) * kRWp;   // density box
+  using F = Form<Maps>;
+  static constexpr bool kIdx = F::kIdx;
+  static constexpr int k32 = 2 + 2 * N;             // v_x, v_y, psi_x[N], psi_y[N]
+  static constexpr int kM = kIdx ? 0 : 1 + 2 * N;   // 1/kappa1, a1[N], b1[N]
+  static constexpr int kPb = (kHT + 7) * kCW;                       // operand box
+  static constexpr int kRb = (kHT + 1) * kWide<typename F::MT>;     // density box (elements)
+  static constexpr int kIb = (kHT + 1) * kWide<typename F::IT>;     // index box (elements)
   static constexpr int kP = round32(kPb);
-  static constexpr int kR = kIdx ? 0 : round32(kRb);  // the index form looks the density up
-  static constexpr int kS = kNs * kArr;
-  static constexpr int kI = kIdx ? (kHT + 1) * kIW / 4 : 0;  // index bytes / 4
-  // dense, literal nonlinear system: K box of the density box's shape
+  static constexpr int kR = kIdx ? 0 : round32(floats_of<typename F::MT>(kRb));  // the index form looks it up
+  static constexpr int oM = k32 * kArr;                             // maps, from the float arrays
+  static constexpr int kS = oM + floats_of<typename F::MT>(kM * kArr);
+  static constexpr int kI = kIdx ? floats_of<typename F::IT>(kIb) : 0;
   static constexpr int kK = kIdx ? 0 : kR;
   static constexpr int kFloats = round32(kP + kR + kS + kI + kK);
 };
 
-// pressure: v_x rows y0-1 .. y0+kHT, v_y rows y0-4 .. y0+kHT+2; streamed
-// arrays; tissue bytes of the half tile (index form)
+// pressure: v_x rows y0-1 .. y0+kHT, v_y rows y0-4 .. y0+kHT+2; float arrays;
+// map arrays or the index of the half tile
 template <int N, typename Maps>
 struct PrsStage {
-  static constexpr bool kIdx = IsIdx<Maps>::value;
-  // dense: p, psi_x[N], psi_y[N], 1/kappa2, K, chi, a2[N], b2[N];
-  // index: p, psi_x[N], psi_y[N]
-  static constexpr int kNs = kIdx ? 1 + 2 * N : 4 + 4 * N;
+  using F = Form<Maps>;
+  static constexpr bool kIdx = F::kIdx;
+  static constexpr int k32 = 1 + 2 * N;             // p, psi_x[N], psi_y[N]
+  static constexpr int kM = kIdx ? 0 : 3 + 2 * N;   // 1/kappa2, K, chi, a2[N], b2[N]
   static constexpr int kXb = (kHT + 2) * kCW;
   static constexpr int kYb = (kHT + 7) * kCW;
   static constexpr int kX = round32(kXb);
   static constexpr int kY = round32(kYb);
-  static constexpr int kS = kNs * kArr;
-  static constexpr int kI = kIdx ? kHT * kTX / 4 : 0;
+  static constexpr int oM = k32 * kArr;
+  static constexpr int kS = oM + floats_of<typename F::MT>(kM * kArr);
+  static constexpr int kI = kIdx ? floats_of<typename F::IT>(kArr) : 0;
   static constexpr int kFloats = round32(kX + kY + kS + kI);
 };
 
@@ -126,14 +152,16 @@ struct PrsStage {
 // the nonlinear term, the velocity's K box only with the literal system).
 template <int N, typename Maps, bool VEL>
 __host__ __device__ constexpr unsigned stage_bytes(bool nl, bool nl_vel) {
+  using MT = typename Form<Maps>::MT;
+  using IT = typename Form<Maps>::IT;
   if (VEL) {
     using S = VelStage<N, Maps>;
-    return 4u * (S::kPb + (S::kIdx ? 0 : S::kRb) + S::kNs * kArr) + (S::kIdx ? (kHT + 1) * kIW : 0) +
-           ((!S::kIdx && nl_vel) ? 4u * S::kRb : 0u);
+    return 4u * (S::kPb + S::k32 * kArr) + (S::kIdx ? (unsigned)sizeof(IT) * S::kIb
+                                                    : (unsigned)sizeof(MT) * (S::kM * kArr + (nl_vel ? 2 : 1) * S::kRb));
   } else {
     using S = PrsStage<N, Maps>;
-    return 4u * (S::kXb + S::kYb + S::kNs * kArr) - ((!S::kIdx && !nl) ? 4u * kArr : 0u) +
-           (S::kIdx ? kHT * kTX : 0);
+    return 4u * (S::kXb + S::kYb + S::k32 * kArr) +
+           (S::kIdx ? (unsigned)sizeof(IT) * kArr : (unsigned)sizeof(MT) * kArr * (S::kM - (nl ? 0 : 1)));
   }
 }
 
@@ -150,8 +178,9 @@ __device__ __forceinline__ void issue_own(const StepParams &P, const PipeMaps &T
   mbar_arrive_expect_tx(bar, stage_bytes<N, Maps, VEL>(P.nl != 0, P.nl_vel != 0));
   if (VEL) {
     using S = VelStage<N, Maps>;
+    constexpr int kMf = floats_of<typename Form<Maps>::MT>(kArr);  // floats of one map array
     if (!S::kIdx) tma_load_2d(st + S::kP, &T.m[1], x0, y0, bar);
-    float *ss = st + S::kP + S::kR;
+    float *ss = st + S::kP + S::kR, *sm = ss + S::oM;
     tma_load_2d(ss, &T.m[2], x0, y0, bar);
     tma_load_2d(ss + kArr, &T.m[3], x0, y0, bar);
     if (N > 0) {
@@ -159,10 +188,10 @@ __device__ __forceinline__ void issue_own(const StepParams &P, const PipeMaps &T
       tma_load_3d(ss + (2 + N) * kArr, &T.m[5], x0, y0, 0, bar);
     }
     if (!S::kIdx) {
-      tma_load_2d(ss + (2 + 2 * N) * kArr, &T.m[6], x0, y0, bar);
+      tma_load_2d(sm, &T.m[6], x0, y0, bar);
       if (N > 0) {
-        tma_load_3d(ss + (3 + 2 * N) * kArr, &T.m[7], x0, y0, 0, bar);
-        tma_load_3d(ss + (3 + 3 * N) * kArr, &T.m[8], x0, y0, 0, bar);
+        tma_load_3d(sm + kMf, &T.m[7], x0, y0, 0, bar);
+        tma_load_3d(sm + (1 + N) * kMf, &T.m[8], x0, y0, 0, bar);
       }
       if (P.nl_vel) tma_load_2d(ss + S::kS, &T.m[9], x0, y0, bar);  // K, density-box shape
     } else {
@@ -170,19 +199,20 @@ __device__ __forceinline__ void issue_own(const StepParams &P, const PipeMaps &T
     }
   } else {
     using S = PrsStage<N, Maps>;
-    float *ss = st + S::kX + S::kY;
+    constexpr int kMf = floats_of<typename Form<Maps>::MT>(kArr);
+    float *ss = st + S::kX + S::kY, *sm = ss + S::oM;
     tma_load_2d(ss, &T.m[2], x0, y0, bar);
     if (N > 0) {
       tma_load_3d(ss + kArr, &T.m[3], x0, y0, 0, bar);
       tma_load_3d(ss + (1 + N) * kArr, &T.m[4], x0, y0, 0, bar);
     }
     if (!S::kIdx) {
-      tma_load_2d(ss + (1 + 2 * N) * kArr, &T.m[5], x0, y0, bar);
-      tma_load_2d(ss + (2 + 2 * N) * kArr, &T.m[6], x0, y0, bar);
-      if (P.nl) tma_load_2d(ss + (3 + 2 * N) * kArr, &T.m[7], x0, y0, bar);
+      tma_load_2d(sm, &T.m[5], x0, y0, bar);
+      tma_load_2d(sm + kMf, &T.m[6], x0, y0, bar);
+      if (P.nl) tma_load_2d(sm + 2 * kMf, &T.m[7], x0, y0, bar);
       if (N > 0) {
-        tma_load_3d(ss + (4 + 2 * N) * kArr, &T.m[8], x0, y0, 0, bar);
-        tma_load_3d(ss + (4 + 3 * N) * kArr, &T.m[9], x0, y0, 0, bar);
+        tma_load_3d(sm + 3 * kMf, &T.m[8], x0, y0, 0, bar);
+        tma_load_3d(sm + (3 + N) * kMf, &T.m[9], x0, y0, 0, bar);
       }
     } else {
       tma_load_2d(ss + S::kS, &T.m[5], x0, y0, bar);  // tissue index
@@ -346,20 +376,85 @@ __device__ __forceinline__ void prs_derivs2(const StepParams &P, const float *sv
   }
 }
 
-// per-tissue table of the index form into shared memory (all threads)
-template <typename Maps>
+// Per-tissue tables of the index forms in shared memory: fields K, rho, chi,
+// 1/kappa1, 1/kappa2, then a1, b1, a2, b2 of the mechanisms (kSlots each),
+// kStride entries per field.  uint8: the global table as it is.  uint16: the
+// fields of the context's N mechanisms only, tab_stride entries each, while
+// they fit next to two stages.
+template <int N, typename Maps>
+struct Table {
+  static constexpr int kSlots = kWideIdx<Maps> ? N : kTabSlots;
+  const float *t;
+  int stride;
+  __device__ __forceinline__ Table(const StepParams &P, const float *tab)
+      : t(tab), stride(kWideIdx<Maps> ? P.tab_stride : kTissues) {}
+  // field id: kTabK .. kTabIk2, or the relaxation field `group` (a1, b1, a2,
+  // b2) of mechanism nu
+  __device__ __forceinline__ const float *field(int f) const { return t + f * stride; }
+  __device__ __forceinline__ const float *relax(int group, int nu) const {
+    return t + (kTabRelax + group * kSlots + nu) * stride;
+  }
+};
+template <typename IT>
+__device__ __forceinline__ float2 look2(const float *field, const IT *cells) {
+  if constexpr (sizeof(IT) == 1) {
+    const uchar2 c = *reinterpret_cast<const uchar2 *>(cells);
+    return make_float2(field[c.x], field[c.y]);
+  } else {
+    const ushort2 c = *reinterpret_cast<const ushort2 *>(cells);
+    return make_float2(field[c.x], field[c.y]);
+  }
+}
+// the table of the index forms into shared memory (all threads)
+template <int N, typename Maps>
 __device__ __forceinline__ void stage_table(const StepParams &P, float *tab, int tid) {
-  if constexpr (IsIdx<Maps>::value) {
+  if constexpr (kWideIdx<Maps>) {
+    const int S4 = P.tab_stride / 4;
+    float4 *dst = reinterpret_cast<float4 *>(tab);
+    for (int f = 0; f < kTabRelax + 4 * N; ++f) {
+      const int r = f - kTabRelax, g = f < kTabRelax ? f : kTabRelax + (N ? r / N * kTabSlots + r % N : 0);
+      const float4 *src = reinterpret_cast<const float4 *>(P.table + (long long)g * P.tab_stride);
+      for (int t = tid; t < S4; t += kThreads) dst[f * S4 + t] = __ldg(src + t);
+    }
+  } else if constexpr (Form<Maps>::kIdx) {
     const float4 *src = reinterpret_cast<const float4 *>(P.table);
     float4 *dst = reinterpret_cast<float4 *>(tab);
     for (int t = tid; t < kTableFields * kTissues / 4; t += kThreads) dst[t] = __ldg(src + t);
   }
 }
 
-// coefficient of field f at the two cells of a pair (index form)
-__device__ __forceinline__ float2 look2(const float *tab, int f, uchar2 t) {
-  const float *r = tab + f * kTissues;
-  return make_float2(r[t.x], r[t.y]);
+// Pair of staged map values (16-bit maps: FP16 times the map's scale) and of
+// decay factors (16-bit maps hold 1 - b): the tile path's loads.
+__device__ __forceinline__ float2 ldm2(const float *m, float) { return sld2(m); }
+__device__ __forceinline__ float2 ldm2(const __nv_bfloat16 *m, float) {
+  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(m));
+}
+__device__ __forceinline__ float2 ldm2(const __half *m, float sc) {
+  const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(m));
+  return make_float2(v.x * sc, v.y * sc);
+}
+__device__ __forceinline__ float2 ldbm2(const float *m, float) { return sld2(m); }
+template <typename MT>
+__device__ __forceinline__ float2 ldbm2(const MT *m, float sc) {
+  const float2 v = ldm2(m, sc);
+  return make_float2(1.f - v.x, 1.f - v.y);
+}
+__device__ __forceinline__ float ldm1(const float *m, float) { return *m; }
+__device__ __forceinline__ float ldm1(const __nv_bfloat16 *m, float) { return __bfloat162float(*m); }
+__device__ __forceinline__ float ldm1(const __half *m, float sc) { return __half2float(*m) * sc; }
+// the same pairs of C-PML strip values in global memory (aligned pairs)
+__device__ __forceinline__ float2 ldg2(const float *m) { return __ldg(reinterpret_cast<const float2 *>(m)); }
+__device__ __forceinline__ float2 lds2(const float *m, float) { return ldg2(m); }
+__device__ __forceinline__ float2 ldsb2(const float *m, float) { return ldg2(m); }
+template <typename MT>
+__device__ __forceinline__ float2 lds2(const MT *m, float sc) {
+  const unsigned u = __ldg(reinterpret_cast<const unsigned *>(m));
+  return ldm2(reinterpret_cast<const MT *>(&u), sc);
+}
+template <typename MT>
+__device__ __forceinline__ float2 ldsb2(const MT *m, float sc) {
+  const float2 v = lds2(m, sc);
+  return make_float2(1.f - v.x, 1.f - v.y);
 }
 
 // Densities at the faces of a pair, read where the thread needs them: cells
@@ -370,9 +465,10 @@ __device__ __forceinline__ float2 look2(const float *tab, int f, uchar2 t) {
 struct FaceRho {
   float r0, r1, r2, u0, u1;  // row ly: lx .. lx+2; row ly+1: lx, lx+1
 };
-template <typename Maps, bool EDGE>
-__device__ __forceinline__ FaceRho face_rho(const StepParams &P, const float *tab, const float *sr,
-                                            const unsigned char *si, int x0, int y0, int lx, int ly) {
+template <int N, typename Maps, bool EDGE>
+__device__ __forceinline__ FaceRho face_rho(const StepParams &P, const Table<N, Maps> &tab,
+                                            const typename Form<Maps>::MT *sr, const typename Form<Maps>::IT *si,
+                                            int x0, int y0, int lx, int ly) {
   int c0 = lx, c1 = lx + 1, c2 = lx + 2, r0 = ly, r1 = ly + 1;
   if (EDGE) {
     const int mx = P.nx - 1 - x0, my = P.ny - 1 - y0;  // last cell inside, tile coordinates
@@ -383,27 +479,28 @@ __device__ __forceinline__ FaceRho face_rho(const StepParams &P, const float *ta
     r1 = min(r1, my);
   }
   auto at = [&](int r, int cc) -> float {
-    if constexpr (IsIdx<Maps>::value) return tab[kTabRho * kTissues + si[r * kIW + cc]];
-    else return sr[r * kRWp + cc];
+    if constexpr (Form<Maps>::kIdx) return tab.field(kTabRho)[si[r * kWide<typename Form<Maps>::IT> + cc]];
+    else return ldm1(sr + r * kWide<typename Form<Maps>::MT> + cc, P.ms[kMsRho]);
   };
   return FaceRho{at(r0, c0), at(r0, c1), at(r0, c2), at(r1, c0), at(r1, c1)};
 }
 
 // Momentum factors of the literal nonlinear system (Eq. general5) at the x
 // and y faces of the pair: p from the staged operand (cell e at column
-// lx + 4 + e of row sy; zero beyond the grid), K from the staged K box (float
-// maps; the density box's shape) or the staged index (index form),
+// lx + 4 + e of row sy; zero beyond the grid), K from the staged K box (dense
+// maps; the density box's shape) or the staged index (index forms),
 // neighbours clamped to the last cell.
-template <typename Maps, bool EDGE>
-__device__ __forceinline__ void mom_factors2(const StepParams &P, const float *tab, const unsigned char *si,
-                                             const float *sk, const float *sp, int sy, int lx, int ly, int x0,
-                                             int y0, float2 &fx, float2 &fy) {
+template <int N, typename Maps, bool EDGE>
+__device__ __forceinline__ void mom_factors2(const StepParams &P, const Table<N, Maps> &tab,
+                                             const typename Form<Maps>::IT *si, const typename Form<Maps>::MT *sk,
+                                             const float *sp, int sy, int lx, int ly, int x0, int y0, float2 &fx,
+                                             float2 &fy) {
   const float *row = sp + sy * kCW + lx + 4, *up = sp + (sy + 1) * kCW + lx + 4;
   const int mx = P.nx - 1 - x0, my = P.ny - 1 - y0;
   const int r1 = EDGE ? min(ly + 1, my) : ly + 1;
   auto K = [&](int r, int cc) -> float {
-    if constexpr (IsIdx<Maps>::value) return tab[kTabK * kTissues + si[r * kIW + cc]];
-    else return sk[r * kRWp + cc];
+    if constexpr (Form<Maps>::kIdx) return tab.field(kTabK)[si[r * kWide<typename Form<Maps>::IT> + cc]];
+    else return ldm1(sk + r * kWide<typename Form<Maps>::MT> + cc, P.ms[kMsK]);
   };
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
@@ -420,11 +517,11 @@ __device__ __forceinline__ void mom_factors2(const StepParams &P, const float *t
 template <int OP, typename Maps>
 __device__ __forceinline__ void x_strip_coef2(const StepParams &P, int nu, int i0, int j, float2 &a, float2 &b) {
   using ST = typename Maps::StripT;
-  static_assert(sizeof(ST) == 4, "the pipelined 2D kernels read float strips");
   const int L = P.L[0];
   if (!(L > 0 && (i0 < L || i0 + 1 >= P.nx - L))) return;
-  const float *sa = static_cast<const float *>(OP == 1 ? P.sa1[0] : P.sa2[0]);
-  const float *sb = static_cast<const float *>(OP == 1 ? P.sb1[0] : P.sb2[0]);
+  const ST *sa = static_cast<const ST *>(OP == 1 ? P.sa1[0] : P.sa2[0]);
+  const ST *sb = static_cast<const ST *>(OP == 1 ? P.sb1[0] : P.sb2[0]);
+  const float s_a = P.ms[(OP == 1 ? kMsA1 : kMsA2) + nu], s_b = P.ms[(OP == 1 ? kMsB1 : kMsB2) + nu];
   const long long row = (long long)nu * P.strip_nu[0] + (long long)j * (2 * L);
   // both cells on one side of the strip: one aligned pair (i0 and the high
   // side's offset nx - 2L are even)
@@ -432,8 +529,8 @@ __device__ __forceinline__ void x_strip_coef2(const StepParams &P, int nu, int i
   if (i0 + 1 < L) sc0 = i0;
   else if (i0 >= P.nx - L && i0 + 1 < P.nx && ((P.nx - 2 * L) & 1) == 0) sc0 = i0 - (P.nx - 2 * L);
   if (sc0 >= 0) {
-    a = __ldg(reinterpret_cast<const float2 *>(sa + row + sc0));
-    b = __ldg(reinterpret_cast<const float2 *>(sb + row + sc0));
+    a = lds2(sa + row + sc0, s_a);
+    b = ldsb2(sb + row + sc0, s_b);
     return;
   }
 #pragma unroll
@@ -445,8 +542,8 @@ __device__ __forceinline__ void x_strip_coef2(const StepParams &P, int nu, int i
     } else {
       const int sc = strip_coord(x, P.nx, L);
       if (sc >= 0) {
-        el2(a, e) = ldmap(sa, row + sc);
-        el2(b, e) = ldb(sb, row + sc);
+        el2(a, e) = ldmap(sa, row + sc, s_a);
+        el2(b, e) = ldb(sb, row + sc, s_b);
       }
     }
   }
@@ -456,25 +553,27 @@ __device__ __forceinline__ void x_strip_coef2(const StepParams &P, int nu, int i
 // aligned pair: i0 even, pitch a multiple of 16)
 template <int OP, typename Maps>
 __device__ __forceinline__ void y_strip_coef2(const StepParams &P, int nu, int i0, int sc, float2 &a, float2 &b) {
-  const float *sa = static_cast<const float *>(OP == 1 ? P.sa1[1] : P.sa2[1]);
-  const float *sb = static_cast<const float *>(OP == 1 ? P.sb1[1] : P.sb2[1]);
+  using ST = typename Maps::StripT;
+  const ST *sa = static_cast<const ST *>(OP == 1 ? P.sa1[1] : P.sa2[1]);
+  const ST *sb = static_cast<const ST *>(OP == 1 ? P.sb1[1] : P.sb2[1]);
   const long long off = (long long)nu * P.strip_nu[1] + (long long)sc * P.pitch + i0;
-  a = __ldg(reinterpret_cast<const float2 *>(sa + off));
-  b = __ldg(reinterpret_cast<const float2 *>(sb + off));
+  a = lds2(sa + off, P.ms[(OP == 1 ? kMsA1 : kMsA2) + nu]);
+  b = ldsb2(sb + off, P.ms[(OP == 1 ? kMsB1 : kMsB2) + nu]);
 }
 
 // Prefetch into L2 the C-PML strip rows an edge half tile will read (warp 0,
 // when its copies are issued): otherwise they come straight from DRAM while
 // the half tile computes.  OP: 1 velocity (a1, b1), 2 pressure (a2, b2).
 __device__ __forceinline__ void l2_line(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-template <int N, int OP>
+template <int N, int OP, typename ST>
 __device__ __forceinline__ void prefetch_strips2(const StepParams &P, int x0, int y0, int lane) {
   if constexpr (N > 0) {
-    const float *sa[2], *sb[2];
+    constexpr int kLine = 128 / (int)sizeof(ST);  // elements of a 128-byte line
+    const ST *sa[2], *sb[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      sa[q] = static_cast<const float *>(OP == 1 ? P.sa1[q] : P.sa2[q]);
-      sb[q] = static_cast<const float *>(OP == 1 ? P.sb1[q] : P.sb2[q]);
+      sa[q] = static_cast<const ST *>(OP == 1 ? P.sa1[q] : P.sa2[q]);
+      sb[q] = static_cast<const ST *>(OP == 1 ? P.sb1[q] : P.sb2[q]);
     }
     const int Lx = P.L[0];
     if (Lx > 0 && (x0 < Lx || x0 + kTX > P.nx - Lx)) {
@@ -482,8 +581,8 @@ __device__ __forceinline__ void prefetch_strips2(const StepParams &P, int x0, in
         const int r = t % kHT, nu = (t / kHT) % N, ab = t / (kHT * N);
         const int y = y0 + r;
         if (y >= P.ny) continue;
-        const float *b = (ab ? sb[0] : sa[0]) + nu * P.strip_nu[0] + (long long)y * (2 * Lx);
-        for (int o = 0; o < 2 * Lx; o += 32) l2_line(b + o);  // 128-byte lines
+        const ST *b = (ab ? sb[0] : sa[0]) + nu * P.strip_nu[0] + (long long)y * (2 * Lx);
+        for (int o = 0; o < 2 * Lx; o += kLine) l2_line(b + o);
       }
     }
     const int Ly = P.L[1];
@@ -493,8 +592,8 @@ __device__ __forceinline__ void prefetch_strips2(const StepParams &P, int x0, in
         const int y = y0 + r;
         const int sc = y < P.ny ? strip_coord(y, P.ny, Ly) : -1;
         if (sc < 0) continue;
-        const float *b = (ab ? sb[1] : sa[1]) + nu * P.strip_nu[1] + (long long)sc * P.pitch + x0;
-        for (int o = 0; o < kTX && x0 + o < P.nx; o += 32) l2_line(b + o);
+        const ST *b = (ab ? sb[1] : sa[1]) + nu * P.strip_nu[1] + (long long)sc * P.pitch + x0;
+        for (int o = 0; o < kTX && x0 + o < P.nx; o += kLine) l2_line(b + o);
       }
     }
   }
@@ -504,10 +603,13 @@ template <int N, typename Maps, bool EDGE>
 __device__ __forceinline__ void vel_compute(const StepParams &P, const float *tab, float *st, int x0, int y0,
                                             int tid) {
   using S = VelStage<N, Maps>;
+  using MT = typename S::F::MT;
+  using IT = typename S::F::IT;
+  const Table<N, Maps> T(P, tab);
   const float *sp = st;
-  const float *sr = st + S::kP;
-  const float *ss = sr + S::kR;
-  const unsigned char *si = reinterpret_cast<const unsigned char *>(ss + S::kS);
+  const MT *sr = reinterpret_cast<const MT *>(st + S::kP);
+  const float *ss = st + S::kP + S::kR;
+  const IT *si = reinterpret_cast<const IT *>(ss + S::kS);
   const int t2 = tid & 63, ly = tid >> 6, lx = 2 * t2;
   const int i0 = x0 + lx, j = y0 + ly;
   if (EDGE && (i0 >= P.nx || j >= P.ny)) return;
@@ -518,19 +620,20 @@ __device__ __forceinline__ void vel_compute(const StepParams &P, const float *ta
   vel_derivs2(P, sp, ly + 3, lx, Dx, Dy);
   float2 k1, A[N > 0 ? N : 1], B[N > 0 ? N : 1];
   if constexpr (S::kIdx) {
-    const uchar2 cell = *reinterpret_cast<const uchar2 *>(si + ly * kIW + lx);
-    k1 = look2(tab, kTabIk1, cell);
+    const IT *cell = si + ly * kWide<IT> + lx;
+    k1 = look2(T.field(kTabIk1), cell);
 #pragma unroll
     for (int nu = 0; nu < N; ++nu) {
-      A[nu] = look2(tab, kTabRelax + nu, cell);
-      B[nu] = look2(tab, kTabRelax + kTabSlots + nu, cell);
+      A[nu] = look2(T.relax(0, nu), cell);
+      B[nu] = look2(T.relax(1, nu), cell);
     }
   } else {
-    k1 = sld2(own + (2 + 2 * N) * kArr);
+    const MT *mp = reinterpret_cast<const MT *>(ss + S::oM) + ly * kTX + lx;
+    k1 = ldm2(mp, P.ms[kMsIk1]);
 #pragma unroll
     for (int nu = 0; nu < N; ++nu) {
-      A[nu] = sld2(own + (3 + 2 * N + nu) * kArr);
-      B[nu] = sld2(own + (3 + 3 * N + nu) * kArr);
+      A[nu] = ldm2(mp + (1 + nu) * kArr, P.ms[kMsA1 + nu]);
+      B[nu] = ldbm2(mp + (1 + N + nu) * kArr, P.ms[kMsB1 + nu]);
     }
   }
   // per-axis coefficients; in an edge pair the C-PML strips replace them,
@@ -565,10 +668,10 @@ __device__ __forceinline__ void vel_compute(const StepParams &P, const float *ta
     put2<Maps, EDGE>(own, 2 + nu, P.psi1[0], nu * Sn + c, nx_, i0, P.nx);
     put2<Maps, EDGE>(own, 2 + N + nu, P.psi1[1], nu * Sn + c, ny_, i0, P.nx);
   }
-  const FaceRho fr = face_rho<Maps, EDGE>(P, tab, sr, si, x0, y0, lx, ly);
+  const FaceRho fr = face_rho<N, Maps, EDGE>(P, T, sr, si, x0, y0, lx, ly);
   if (P.nl_vel) {
     float2 fx, fy;
-    mom_factors2<Maps, EDGE>(P, tab, si, ss + S::kS, sp, ly + 3, lx, ly, x0, y0, fx, fy);
+    mom_factors2<N, Maps, EDGE>(P, T, si, reinterpret_cast<const MT *>(ss + S::kS), sp, ly + 3, lx, ly, x0, y0, fx, fy);
     vx.x = vel_upd(vx.x, qdiv(P.two_dt, fr.r0 + fr.r1), Sx.x, fx.x);
     vx.y = vel_upd(vx.y, qdiv(P.two_dt, fr.r1 + fr.r2), Sx.y, fx.y);
     vy.x = vel_upd(vy.x, qdiv(P.two_dt, fr.r0 + fr.u0), Sy.x, fy.x);
@@ -587,6 +690,9 @@ template <int N, typename Maps, bool EDGE>
 __device__ __forceinline__ void prs_compute(const StepParams &P, const float *tab, float *st, int x0, int y0,
                                             int tid) {
   using S = PrsStage<N, Maps>;
+  using MT = typename S::F::MT;
+  using IT = typename S::F::IT;
+  const Table<N, Maps> T(P, tab);
   const float *sx = st, *sy = st + S::kX;
   float *ss = st + S::kX + S::kY;
   const int t2 = tid & 63, ly = tid >> 6, lx = 2 * t2;
@@ -599,24 +705,24 @@ __device__ __forceinline__ void prs_compute(const StepParams &P, const float *ta
   prs_derivs2(P, sx, sy, ly, lx, Dx, Dy);
   float2 k2, K, ch = make_float2(0.f, 0.f), A[N > 0 ? N : 1], B[N > 0 ? N : 1];
   if constexpr (S::kIdx) {
-    const uchar2 cell =
-        *reinterpret_cast<const uchar2 *>(reinterpret_cast<const unsigned char *>(ss + S::kS) + ly * kTX + lx);
-    k2 = look2(tab, kTabIk2, cell);
-    K = look2(tab, kTabK, cell);
-    if (P.nl) ch = look2(tab, kTabChi, cell);
+    const IT *cell = reinterpret_cast<const IT *>(ss + S::kS) + ly * kTX + lx;
+    k2 = look2(T.field(kTabIk2), cell);
+    K = look2(T.field(kTabK), cell);
+    if (P.nl) ch = look2(T.field(kTabChi), cell);
 #pragma unroll
     for (int nu = 0; nu < N; ++nu) {
-      A[nu] = look2(tab, kTabRelax + 2 * kTabSlots + nu, cell);
-      B[nu] = look2(tab, kTabRelax + 3 * kTabSlots + nu, cell);
+      A[nu] = look2(T.relax(2, nu), cell);
+      B[nu] = look2(T.relax(3, nu), cell);
     }
   } else {
-    k2 = sld2(own + (1 + 2 * N) * kArr);
-    K = sld2(own + (2 + 2 * N) * kArr);
-    if (P.nl) ch = sld2(own + (3 + 2 * N) * kArr);
+    const MT *mp = reinterpret_cast<const MT *>(ss + S::oM) + ly * kTX + lx;
+    k2 = ldm2(mp, P.ms[kMsIk2]);
+    K = ldm2(mp + kArr, P.ms[kMsK]);
+    if (P.nl) ch = ldm2(mp + 2 * kArr, P.ms[kMsChi]);
 #pragma unroll
     for (int nu = 0; nu < N; ++nu) {
-      A[nu] = sld2(own + (4 + 2 * N + nu) * kArr);
-      B[nu] = sld2(own + (4 + 3 * N + nu) * kArr);
+      A[nu] = ldm2(mp + (3 + nu) * kArr, P.ms[kMsA2 + nu]);
+      B[nu] = ldbm2(mp + (3 + N + nu) * kArr, P.ms[kMsB2 + nu]);
     }
   }
   float2 AX[N > 0 ? N : 1], BX[N > 0 ? N : 1], AY[N > 0 ? N : 1], BY[N > 0 ? N : 1];
@@ -682,15 +788,21 @@ template <int N, typename Maps>
 struct StepRing {
   static constexpr int kV = VelStage<N, Maps>::kFloats, kP = PrsStage<N, Maps>::kFloats;
   static constexpr int kStage = kV > kP ? kV : kP;
-  static constexpr int kBudget = (224 * 1024 - 128) / 4 - Maps::kSmemFloats;  // floats
-  static constexpr int kFit = kBudget / kStage;
+  static constexpr int kTotal = (224 * 1024 - 128) / 4;  // floats
+  // the uint16 form's table takes what two stages leave
+  static constexpr int kTab = kWideIdx<Maps> ? kTotal - 2 * kStage : Maps::kSmemFloats;
+  static constexpr int kFit = (kTotal - kTab) / kStage;
   static constexpr int kStages = kFit > 4 ? 4 : kFit;
   static constexpr int kLag = kStages >= 4 ? 1 : 0;  // as Ring
   static constexpr int kAhead = kStages - 1 - kLag;
-  static constexpr size_t kBytes = sizeof(float) * ((size_t)kStages * kStage + Maps::kSmemFloats) + 128;
+  static constexpr size_t kBytes = sizeof(float) * ((size_t)kStages * kStage + kTab) + 128;
   static_assert(kStages >= 2, "two stages must fit in shared memory");
   static_assert(kBytes + 1024 <= 227 * 1024, "stages and table leave 1 KB for static shared memory");
 };
+// largest table stride of the uint16 index form whose fields fit (about 1480
+// tissues with four mechanisms)
+template <int N>
+constexpr int kWideTissues = StepRing<N, IdxMaps16>::kTab / (kTabRelax + 4 * N) / 4 * 4;
 
 // Which of a block's half tiles hold sources, per half step: one bit per
 // round, looked up once per launch (a load per half tile in the loop would
@@ -790,7 +902,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   float *smem = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   float *tab = smem + kS * kStage;
   const int tid = threadIdx.y * 32 + threadIdx.x;
-  stage_table<Maps>(P, tab, tid);  // made visible by the barrier below
+  stage_table<N, Maps>(P, tab, tid);  // made visible by the barrier below
   GridBarrier gb;
   if (tid == 0) {
     for (int q = 0; q < kS; ++q) mbar_init(&bar[q], 1);
@@ -854,8 +966,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       if (!R.interior(ix, iy)) {
-        if (iph & 1) prefetch_strips2<N, 2>(P, ix, iy, tid);
-        else prefetch_strips2<N, 1>(P, ix, iy, tid);
+        if (iph & 1) prefetch_strips2<N, 2, typename Maps::StripT>(P, ix, iy, tid);
+        else prefetch_strips2<N, 1, typename Maps::StripT>(P, ix, iy, tid);
       }
     }
     pending |= 1u << is;
@@ -1063,7 +1175,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int *dst = reinterpret_cast<int *>(&sP);
       for (int w = tid; w < (int)(sizeof(StepParams) / 4); w += kThreads) dst[w] = __ldg(src + w);
       __syncthreads();
-      stage_table<Maps>(sP, tab, tid);
+      stage_table<N, Maps>(sP, tab, tid);
       __syncthreads();
       cur = e.x;
     }
@@ -1075,7 +1187,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           acquire(en.x);
           issue_stage<N, Maps, VEL>(Ps[en.x], Ts[en.x], smem + q * kStage, &bar[q], en.y, en.z);
         }
-        if (!en.w && en.x == cur) prefetch_strips2<N, VEL ? 1 : 2>(sP, en.y, en.z, tid);
+        if (!en.w && en.x == cur) prefetch_strips2<N, VEL ? 1 : 2, typename Maps::StripT>(sP, en.y, en.z, tid);
       }
       pending |= 1u << q;
       ++hs;
@@ -1178,8 +1290,19 @@ Region region_of(const StepParams &P) {
 
 bool pipe2d_supported(const StepParams &P, int map_kind) {
   // the copies read zero outside the grid: the zero-outside boundary only
-  return P.nz == 1 && (map_kind == 0 || map_kind == 2) && P.n_relax >= 0 && P.n_relax <= kPipe2dMaxRelax &&
-         !P.periodic[0] && !P.periodic[1];
+  if (P.nz != 1 || P.n_relax < 0 || P.n_relax > kPipe2dMaxRelax || P.periodic[0] || P.periodic[1]) return false;
+  // uint16 index: the tables have to fit in shared memory (beyond that the
+  // tile kernels read them through L2; 1160 tissues at 1536 x 2048: 191 us a
+  // step there)
+  if (map_kind == 3) {
+    const int most[] = {kWideTissues<0>, kWideTissues<1>, kWideTissues<2>, kWideTissues<3>, kWideTissues<4>};
+    return P.tab_stride <= most[P.n_relax];
+  }
+  return map_kind >= 0 && map_kind <= 4;
+}
+
+bool pipe2d_batched_supported(const StepParams &P, int map_kind) {
+  return (map_kind == 0 || map_kind == 2) && pipe2d_supported(P, map_kind);
 }
 
 bool pipe2d_preferred(const StepParams &P, int map_kind) { return pipe2d_supported(P, map_kind); }
@@ -1211,6 +1334,9 @@ cudaError_t launch_steps2d(const StepParams &P, int map_kind, int n_sm, const Pi
   while (R.rot + 1 < grid && std::gcd(grid + R.rot, R.ntx) != 1) ++R.rot;
   if (map_kind == 2) return steps_dispatch<IdxMaps>(P, R, grid, vel, prs, io, ph0, ph1, st);
   if (map_kind == 0) return steps_dispatch<DenseMaps<float>>(P, R, grid, vel, prs, io, ph0, ph1, st);
+  if (map_kind == 1) return steps_dispatch<DenseMaps<__nv_bfloat16>>(P, R, grid, vel, prs, io, ph0, ph1, st);
+  if (map_kind == 3) return steps_dispatch<IdxMaps16>(P, R, grid, vel, prs, io, ph0, ph1, st);
+  if (map_kind == 4) return steps_dispatch<DenseMaps<__half>>(P, R, grid, vel, prs, io, ph0, ph1, st);
   return cudaErrorInvalidValue;
 }
 
@@ -1232,16 +1358,14 @@ EncodeTiled encoder() {
   return fn;
 }
 
-// float (or uint8) tensor map over [ny][nx] (rank 2, row stride pitch) or
-// [n3][ny][nx] (rank 3, plane stride s3 elements) with a box of bx x by
-// (x bz)
+// tensor map over [ny][nx] (rank 2, row stride pitch) or [n3][ny][nx] (rank
+// 3, plane stride s3 elements) of es-byte elements with a box of bx x by (x bz)
 bool encode(CUtensorMap *m, const void *base, const StepParams &P, int rank, int n3, long long s3, int bx, int by,
-            int bz, bool u8 = false) {
-  const unsigned long long es = u8 ? 1 : 4;
+            int bz, int es = 4) {
   const unsigned long long dims[3] = {(unsigned long long)P.nx, (unsigned long long)P.ny, (unsigned long long)n3};
   const unsigned long long strides[2] = {(unsigned long long)P.pitch * es, (unsigned long long)s3 * es};
   const unsigned box[3] = {(unsigned)bx, (unsigned)by, (unsigned)bz};
-  return encode_tensor_map(m, base, (int)es, rank, dims, strides, box);
+  return encode_tensor_map(m, base, es, rank, dims, strides, box);
 }
 
 }  // namespace
@@ -1275,13 +1399,17 @@ cudaError_t build_pipe2d_maps(const StepParams &P, int map_kind, PipeMaps *vel, 
   }
   const int N = P.n_relax;
   const long long S = P.npts_alloc;
-  const bool dense = map_kind == 0;
+  const bool dense = map_kind == 0 || map_kind == 1 || map_kind == 4;
+  const int es = map_kind == 1 || map_kind == 4 ? 2 : 4;                     // bytes of a map value
+  const int wide = es == 2 ? kWide<__half> : kWide<float>;                   // density box columns
+  const int ies = map_kind == 3 ? 2 : 1;                                     // bytes of an index
+  const int iwide = ies == 2 ? kWide<unsigned short> : kWide<unsigned char>; // index box columns
   bool ok = true;
   // velocity half step
   ok = ok && encode(&vel->m[0], P.p, P, 2, 1, S, kCW, kHT + 7, 1);
-  if (dense) ok = ok && encode(&vel->m[1], P.rho, P, 2, 1, S, kRWp, kHT + 1, 1);
-  else ok = ok && encode(&vel->m[1], P.tissue, P, 2, 1, S, kIW, kHT + 1, 1, true);
-  if (dense && P.nl_vel) ok = ok && encode(&vel->m[9], P.K, P, 2, 1, S, kRWp, kHT + 1, 1);
+  if (dense) ok = ok && encode(&vel->m[1], P.rho, P, 2, 1, S, wide, kHT + 1, 1, es);
+  else ok = ok && encode(&vel->m[1], P.tissue, P, 2, 1, S, iwide, kHT + 1, 1, ies);
+  if (dense && P.nl_vel) ok = ok && encode(&vel->m[9], P.K, P, 2, 1, S, wide, kHT + 1, 1, es);
   ok = ok && encode(&vel->m[2], P.v[0], P, 2, 1, S, kTX, kHT, 1);
   ok = ok && encode(&vel->m[3], P.v[1], P, 2, 1, S, kTX, kHT, 1);
   if (N > 0) {
@@ -1289,10 +1417,10 @@ cudaError_t build_pipe2d_maps(const StepParams &P, int map_kind, PipeMaps *vel, 
     ok = ok && encode(&vel->m[5], P.psi1[1], P, 3, N, S, kTX, kHT, N);
   }
   if (dense) {
-    ok = ok && encode(&vel->m[6], P.ik1, P, 2, 1, S, kTX, kHT, 1);
+    ok = ok && encode(&vel->m[6], P.ik1, P, 2, 1, S, kTX, kHT, 1, es);
     if (N > 0) {
-      ok = ok && encode(&vel->m[7], P.a1, P, 3, N, S, kTX, kHT, N);
-      ok = ok && encode(&vel->m[8], P.b1, P, 3, N, S, kTX, kHT, N);
+      ok = ok && encode(&vel->m[7], P.a1, P, 3, N, S, kTX, kHT, N, es);
+      ok = ok && encode(&vel->m[8], P.b1, P, 3, N, S, kTX, kHT, N, es);
     }
   }
   // pressure half step
@@ -1303,14 +1431,14 @@ cudaError_t build_pipe2d_maps(const StepParams &P, int map_kind, PipeMaps *vel, 
     ok = ok && encode(&prs->m[3], P.psi2[0], P, 3, N, S, kTX, kHT, N);
     ok = ok && encode(&prs->m[4], P.psi2[1], P, 3, N, S, kTX, kHT, N);
   }
-  if (!dense) ok = ok && encode(&prs->m[5], P.tissue, P, 2, 1, S, kTX, kHT, 1, true);
+  if (!dense) ok = ok && encode(&prs->m[5], P.tissue, P, 2, 1, S, kTX, kHT, 1, ies);
   if (dense) {
-    ok = ok && encode(&prs->m[5], P.ik2, P, 2, 1, S, kTX, kHT, 1);
-    ok = ok && encode(&prs->m[6], P.K, P, 2, 1, S, kTX, kHT, 1);
-    if (P.nl) ok = ok && encode(&prs->m[7], P.chi, P, 2, 1, S, kTX, kHT, 1);
+    ok = ok && encode(&prs->m[5], P.ik2, P, 2, 1, S, kTX, kHT, 1, es);
+    ok = ok && encode(&prs->m[6], P.K, P, 2, 1, S, kTX, kHT, 1, es);
+    if (P.nl) ok = ok && encode(&prs->m[7], P.chi, P, 2, 1, S, kTX, kHT, 1, es);
     if (N > 0) {
-      ok = ok && encode(&prs->m[8], P.a2, P, 3, N, S, kTX, kHT, N);
-      ok = ok && encode(&prs->m[9], P.b2, P, 3, N, S, kTX, kHT, N);
+      ok = ok && encode(&prs->m[8], P.a2, P, 3, N, S, kTX, kHT, N, es);
+      ok = ok && encode(&prs->m[9], P.b2, P, 3, N, S, kTX, kHT, N, es);
     }
   }
   if (!ok) {

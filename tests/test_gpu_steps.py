@@ -73,3 +73,43 @@ def test_steps_in_one_launch_equal_half_steps_bitwise(fw2, nx, ny, N, nl, steps)
         got = run(fw2, prob, steps, how)
         for n, want in ref.items():
             np.testing.assert_array_equal(got[n], want, err_msg=f"{how}: {n}")
+
+
+@pytest.mark.parametrize("maps", ["f16", "bf16"])
+@pytest.mark.parametrize("nx,ny,N,nl,taps", [(129, 9, 0, "off", False), (203, 77, 2, "westervelt", True),
+                                             (333, 140, 3, "off", False), (700, 260, 4, "literal", False)])
+def test_16_bit_maps_on_the_pipelined_path_equal_tile_kernels_bitwise(fw2, maps, nx, ny, N, nl, taps):
+    """FP16 (scaled) and bf16 maps staged by the pipelined kernels: odd widths,
+    both sides of every C-PML strip, the cross taps and the literal system's K."""
+    prob = problem(nx, ny, N, nl, 9, seed=2)
+    if taps:
+        prob.taps = tuple(fw2.fw2_taps_time_space(0.3))
+    out = {}
+    for path in ("tile", "auto"):
+        sim = fw2.Simulation(prob, map_precision=maps, kernel_path=path)
+        sim.set_state(synth.random_state(prob, seed=4))
+        sim.step(9)
+        assert fw2.fw2_kernel_path(sim.ctx) == ("tile" if path == "tile" else "pipe")
+        out[path] = {n: sim.field(n) for n in ("p", "vx", "vy") + (("psi1x", "psi1y", "psi2x", "psi2y") if N else ())}
+        out[path]["trace"] = sim.trace.cpu().numpy()
+        sim.close()
+    for n, want in out["tile"].items():
+        np.testing.assert_array_equal(out["auto"][n], want, err_msg=n)
+
+
+@pytest.mark.parametrize("levels,path", [(64, "pipe"), (369, "pipe"), (370, "tile")])
+def test_uint16_index_takes_the_pipelined_path_while_its_tables_fit(fw2, levels, path):
+    """1476 tissues of four mechanisms are the most that fit next to two
+    stages; the same bits as the tile kernels on either side of the line."""
+    prob = synth.indexed_abdominal_problem(nx=390, ny=220, n_steps=60, n_elements=8, nl="literal", levels=levels)
+    prob.tissue = prob.tissue.astype(np.uint16)
+    out = {}
+    for p in ("tile", "auto"):
+        sim = fw2.Simulation(prob, map_precision="idx16", kernel_path=p)
+        sim.set_state(synth.random_state(prob, seed=4))
+        sim.step(60)
+        assert fw2.fw2_kernel_path(sim.ctx) == ("tile" if p == "tile" else path)
+        out[p] = {n: sim.field(n) for n in ("p", "vx", "vy", "psi1x", "psi2y")}
+        sim.close()
+    for n, want in out["tile"].items():
+        np.testing.assert_array_equal(out["auto"][n], want, err_msg=n)
