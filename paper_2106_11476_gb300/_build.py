@@ -19,8 +19,10 @@ LIB = os.path.join(HERE, "libfw2.so")
 SOURCES = ["api.cu", "prep.cu", "aux.cu", "step2d.cu", "step2d_pipe.cu", "step3d.cu", "step3d_pipe.cu", "noalloc.cu", "batch.cu",
            "fit.cpp"]
 # second compilations of a source: (source, object name, extra flags); the
-# tile kernels for 5..8 mechanisms build beside those for 0..4
-VARIANTS = [("step2d.cu", "step2d_wide", ["-DFW2_WIDE_RELAX"]), ("step3d.cu", "step3d_wide", ["-DFW2_WIDE_RELAX"])]
+# tile kernels for 5..8 mechanisms build beside those for 0..4, the pipelined
+# 3D kernels for float maps beside those for bf16
+VARIANTS = [("step2d.cu", "step2d_wide", ["-DFW2_WIDE_RELAX"]), ("step3d.cu", "step3d_wide", ["-DFW2_WIDE_RELAX"]),
+            ("step3d_pipe.cu", "step3d_pipe_float", ["-DFW2_PIPE3D_FLOAT"])]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

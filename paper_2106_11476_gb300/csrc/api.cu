@@ -319,6 +319,7 @@ fw2_status finalize(fw2_ctx *c) {
   P.tissue = static_cast<const unsigned char *>(Q.tissue_out);
   P.table = Q.table_out;
   P.tab_stride = Q.tab_stride;
+  P.map_kind = c->map_kind;
   for (int m = 0; m < kMapScales; ++m) P.ms[m] = c->map_scale[m];
   P.status = c->d_status;
   const bool forced_pipe = cfg.kernel_path >= FW2_PATH_PIPE;

@@ -426,7 +426,7 @@ fw2_status fw2_batch_create(fw2_ctx *const *ctxs, int32_t n_ctx, fw2_batch **out
       return FW2_EINVAL;
     }
     fw2_status st = ctx_prepare(c);
-    if (st == FW2_OK && c->nd == 3 && !c->pipe)
+    if (st == FW2_OK && c->nd == 3 && !(c->pipe && c->map_kind == FW2_MAP_BF16))
       st = ctx_fail(c, FW2_EUNSUPPORTED,
                     "3D contexts join a batch on the pipelined path only (bf16 maps, N <= 3, no periodic axis)");
     if (st != FW2_OK) {

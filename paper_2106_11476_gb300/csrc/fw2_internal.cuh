@@ -67,6 +67,7 @@ struct StepParams {
   const unsigned char *tissue;
   const float *table;
   int tab_stride;
+  int map_kind;          // FW2_MAP_*
   unsigned int *status;  // device status word: bit 0 set when a bounded wait gave up
   float ms[kMapScales];  // FP16 maps: value = stored x ms[map] (1 for the other storages)
 };
@@ -205,8 +206,8 @@ bool pipe2d_interior_half(const StepParams &P, int x0, int y0);
 cudaError_t launch_pipe2d_batched(bool vel, const StepParams *Ps, const PipeMaps *Ts, const int4 *units,
                                   int n_units, const int *runs, int n_relax, int map_kind, int grid,
                                   cudaStream_t s);
-// persistent pipelined 3D half step (bf16 maps, N <= 3, no periodic axis),
-// in one of two layouts that compute the same result: the memory variables
+// persistent pipelined 3D half step (bf16 or float maps, N <= 3, no periodic
+// axis); float maps take the register layout, bf16 maps one of two layouts that compute the same result: the memory variables
 // staged in shared memory with the other arrays (kLayoutStaged; not with
 // cross taps, nor for the literal system's velocity half step), or loaded
 // into registers one unit ahead with every C-PML strip staged
@@ -222,6 +223,9 @@ cudaError_t launch_pipe3d(bool vel, const StepParams &P, int grid, const PipeMap
 // the context's item count) and the tensor maps, in device memory; items
 // {context, item}; the layout of every context is the default one
 // (pipe3d_staged_layout), which must agree within a launch
+// the kernels for float maps (a second compilation of the file); region: a Region3
+cudaError_t launch_pipe3d_float(bool vel, const StepParams &P, const void *region, int grid, const PipeMaps &T,
+                                cudaStream_t s);
 size_t pipe3d_region_bytes();
 long long pipe3d_region(const StepParams &P, int grid, bool vel, void *out);
 // edge units of each of the context's items (n_edge) and units per item

@@ -33,6 +33,7 @@
 // by this path (the tile kernels run them).
 #include <climits>
 #include <cstring>
+#include <numeric>
 
 #include "async.cuh"
 #include "coef.cuh"
@@ -44,10 +45,17 @@ namespace {
 
 constexpr int kHT = 8;            // rows of a unit
 constexpr int kCW = kTX + 8;      // halo columns x0-4 .. x0+TX+3
-constexpr int kRWb = kTX + 8;     // staged bf16 density / K columns x0 .. x0+TX+7 (16-byte rows)
 constexpr int kArr = kHT * kTX;   // elements of one array per unit
 
 using bf16 = __nv_bfloat16;
+// staged density / K columns x0 .. x0+TX+7 (bf16) or x0+TX+3 (float): rows of
+// 16 bytes one cell wider than the unit
+template <typename MT>
+constexpr int kRW = kTX + 16 / (int)sizeof(MT);
+// bf16 maps: the register layout stages every axis' C-PML strips; float maps
+// leave room for the x strip only, the y and z strips are read per cell
+template <typename MT>
+constexpr bool kStageYZ = sizeof(MT) == 2;
 
 constexpr int round32(int n) { return (n + 31) & ~31; }  // floats: 128-byte regions
 constexpr int fl(int bytes) { return (bytes + 3) / 4; }
@@ -66,58 +74,62 @@ __device__ __forceinline__ int slot_after(int s0, int m) {
   return s >= kSlots ? s - kSlots : s;
 }
 
-// C-PML strip coefficients of a stage (bf16): x strip a then b, each
+// C-PML strip coefficients of a stage (MT): x strip a then b, each
 // [N][8][L] (L <= kXsMax); y strip a, b and z strip a, b, each [N][8][128]
-// (not in the layout that stages the memory variables, PS)
-template <int N, bool PS>
+// (bf16, not in the layout that stages the memory variables, PS)
+template <int N, bool PS, typename MT>
 struct Strips {
-  static constexpr int kX = N * kHT * kXsMax / 2;    // floats of the x strip's a (or b)
-  static constexpr int kYZ = PS ? 0 : N * kArr / 2;  // floats of a y or z strip's a (or b)
+  static constexpr int kE = (int)sizeof(MT);
+  static constexpr int kX = N * kHT * kXsMax * kE / 4;                        // floats of the x strip's a (or b)
+  static constexpr int kYZ = (PS || !kStageYZ<MT>) ? 0 : N * kArr * kE / 4;   // floats of a y or z strip's a (or b)
   static constexpr int oXa = 0, oXb = kX, oYa = 2 * kX, oYb = oYa + kYZ, oZa = oYb + kYZ, oZb = oZa + kYZ;
   static constexpr int kFloats = oZb + kYZ;
 };
 
-// velocity stage: density bf16 [2][9][136] (planes k, k+1), v [3][8][128],
-// 1/kappa1 bf16 [8][128], a1, b1 bf16 [N][8][128], then either (PS) the 3N
-// memory variables [3N][8][128] and the x strip, or K bf16 [2][9][136]
-// (literal system) and the strips of all axes; plane ring: p planes
-// [15][136] (rows y0-3 .. y0+11, columns x0-4 ..)
-template <int N, bool PS>
+// velocity stage (maps of type MT): density [2][9][kRW] (planes k, k+1), v
+// [3][8][128], 1/kappa1 [8][128], a1, b1 [N][8][128], then either (PS) the 3N
+// memory variables [3N][8][128] and the x strip, or K [2][9][kRW] (literal
+// system) and the strips; plane ring: p planes [15][136] (rows y0-3 ..
+// y0+11, columns x0-4 ..)
+template <int N, bool PS, typename MT>
 struct Vel3 {
-  static constexpr int kRho = round32(fl(2 * (kHT + 1) * kRWb * 2));
+  static constexpr int kE = (int)sizeof(MT);
+  static constexpr int kRhoE = 2 * (kHT + 1) * kRW<MT>;  // elements
+  static constexpr int kRho = round32(fl(kRhoE * kE));
   static constexpr int kV = 3 * kArr;
-  static constexpr int kK = round32(fl(kArr * 2));
-  static constexpr int kAB = round32(fl(N * kArr * 2));
+  static constexpr int kK = round32(fl(kArr * kE));
+  static constexpr int kAB = round32(fl(N * kArr * kE));
   static constexpr int kPsi = PS ? 3 * N * kArr : 0;
   static constexpr int kKmF = PS ? 0 : kRho;
   static constexpr int oRho = 0, oV = oRho + kRho, oK = oV + kV, oA = oK + kK, oB = oA + kAB, oPsi = oB + kAB,
                        oKm = oPsi + kPsi, oS = oKm + kKmF;
-  static constexpr int kFloats = round32(oS + Strips<N, PS>::kFloats);
-  static constexpr unsigned kBytes = 4u * (kV + kPsi) + 2u * (2 * (kHT + 1) * kRWb + kArr + 2 * N * kArr);
-  static constexpr unsigned kKmBytes = 2u * 2 * (kHT + 1) * kRWb;
+  static constexpr int kFloats = round32(oS + Strips<N, PS, MT>::kFloats);
+  static constexpr unsigned kBytes = 4u * (kV + kPsi) + (unsigned)kE * (kRhoE + kArr + 2 * N * kArr);
+  static constexpr unsigned kKmBytes = (unsigned)kE * kRhoE;
   static constexpr int kPlane = round32((kHT + 7) * kCW);
   static constexpr unsigned kPlaneBytes = 4u * (kHT + 7) * kCW;
 };
 
-// pressure stage: p [8][128], 1/kappa2, K, chi bf16 [8][128], a2, b2 bf16
-// [N][8][128], then either (PS) the 3N memory variables and the x strip or
-// the strips of all axes; without cross taps also v_x [8][136] (x halo) and
-// v_y [15][128] (rows y0-4 ..), with the plane ring of v_z [8][128]; with
-// cross taps (never PS) the rings hold v_z [10][136] (rows y0-1 .., columns
-// x0-4 ..), v_x [10][136] (rows y0-1 ..) and v_y [15][136] (rows y0-4 ..)
-template <int N, bool CROSS, bool PS>
+// pressure stage: p [8][128], 1/kappa2, K, chi [8][128], a2, b2 [N][8][128]
+// (maps), then either (PS) the 3N memory variables and the x strip or the
+// strips; without cross taps also v_x [8][136] (x halo) and v_y [15][128]
+// (rows y0-4 ..), with the plane ring of v_z [8][128]; with cross taps (never
+// PS) the rings hold v_z [10][136] (rows y0-1 .., columns x0-4 ..), v_x
+// [10][136] (rows y0-1 ..) and v_y [15][136] (rows y0-4 ..)
+template <int N, bool CROSS, bool PS, typename MT>
 struct Prs3 {
+  static constexpr int kE = (int)sizeof(MT);
   static constexpr int kVx = CROSS ? 0 : round32(kHT * kCW);
   static constexpr int kVy = CROSS ? 0 : round32((kHT + 7) * kTX);
   static constexpr int kP = kArr;
-  static constexpr int kK = round32(fl(kArr * 2));
-  static constexpr int kAB = round32(fl(N * kArr * 2));
+  static constexpr int kK = round32(fl(kArr * kE));
+  static constexpr int kAB = round32(fl(N * kArr * kE));
   static constexpr int kPsi = PS ? 3 * N * kArr : 0;
   static constexpr int oVx = 0, oVy = oVx + kVx, oP = oVy + kVy, oIk = oP + kP, oKm = oIk + kK, oChi = oKm + kK,
                        oA = oChi + kK, oB = oA + kAB, oPsi = oB + kAB, oS = oPsi + kPsi;
-  static constexpr int kFloats = round32(oS + Strips<N, PS>::kFloats);
-  static constexpr unsigned kBytesNoChi =
-      4u * ((CROSS ? kP : kHT * kCW + (kHT + 7) * kTX + kP) + kPsi) + 2u * (2 * kArr + 2 * N * kArr);
+  static constexpr int kFloats = round32(oS + Strips<N, PS, MT>::kFloats);
+  static constexpr unsigned kBytesNoChi = 4u * ((CROSS ? kP : kHT * kCW + (kHT + 7) * kTX + kP) + kPsi) +
+                                          (unsigned)kE * (2 * kArr + 2 * N * kArr);
   // v_z ring slot; with cross taps also the v_x and v_y ring slots
   static constexpr int kPlane = CROSS ? round32((kHT + 2) * kCW) : kArr;
   static constexpr unsigned kPlaneBytes = 4u * (CROSS ? (kHT + 2) * kCW : kArr);
@@ -127,13 +139,13 @@ struct Prs3 {
   static constexpr unsigned kYPlaneBytes = 4u * (kHT + 7) * kCW;
 };
 
-template <int N, bool VEL, bool CROSS, bool PS>
+template <int N, bool VEL, bool CROSS, bool PS, typename MT>
 struct Ring3 {
-  static constexpr int kStage = VEL ? Vel3<N, PS>::kFloats : Prs3<N, CROSS, PS>::kFloats;
-  static constexpr int kPlane = VEL ? Vel3<N, PS>::kPlane : Prs3<N, CROSS, PS>::kPlane;
-  static constexpr unsigned kPlaneBytes = VEL ? Vel3<N, PS>::kPlaneBytes : Prs3<N, CROSS, PS>::kPlaneBytes;
+  static constexpr int kStage = VEL ? Vel3<N, PS, MT>::kFloats : Prs3<N, CROSS, PS, MT>::kFloats;
+  static constexpr int kPlane = VEL ? Vel3<N, PS, MT>::kPlane : Prs3<N, CROSS, PS, MT>::kPlane;
+  static constexpr unsigned kPlaneBytes = VEL ? Vel3<N, PS, MT>::kPlaneBytes : Prs3<N, CROSS, PS, MT>::kPlaneBytes;
   static constexpr int kSubFloats =
-      (!VEL && CROSS) ? kSub * (Prs3<N, CROSS, PS>::kXPlane + Prs3<N, CROSS, PS>::kYPlane) : 0;
+      (!VEL && CROSS) ? kSub * (Prs3<N, CROSS, PS, MT>::kXPlane + Prs3<N, CROSS, PS, MT>::kYPlane) : 0;
   static constexpr size_t kBytes =
       sizeof(float) * (2 * (size_t)kStage + (size_t)kSlots * kPlane + (size_t)kSubFloats) + 128;
 };
@@ -146,6 +158,7 @@ struct Region3 {
   int seglen, nseg;  // planes per item, items per column
   int xsL;           // x C-PML strip cells per side when its coefficients come by TMA, else 0
   int ysL, zsL;      // the same for the y and z strips
+  int rot;           // rotation of a round of items over the blocks (pipe3d_kernel)
   // the side of the x strip a unit at x0 reaches: 0 low, 1 high, -1 none
   // (with xsL set no unit reaches both)
   __device__ __forceinline__ int xs_side(int x0) const {
@@ -185,21 +198,22 @@ __host__ __device__ constexpr int ring_first(int k) { return VEL ? k - 3 : k - 4
 // k_lo .. k_hi of the plane ring (one plane, or eight for the first unit of
 // an item) and, with cross taps in the pressure half step, the v_x and v_y
 // planes s_lo .. s_hi of their rings, all completing on the stage's mbarrier.
-template <int N, bool VEL, bool CROSS, bool PS>
+template <int N, bool VEL, bool CROSS, bool PS, typename MT>
 __device__ __forceinline__ void issue3(const PipeMaps &T, const Region3 &R, float *st, float *ring, float *sub,
                                        uint64_t *bar, int x0, int y0, int k, int k_lo, int k_hi, int s_lo, int s_hi,
                                        bool nl, bool nl_vel) {
-  using G = Ring3<N, VEL, CROSS, PS>;
-  using SS = Strips<N, PS>;
+  using G = Ring3<N, VEL, CROSS, PS, MT>;
+  using SS = Strips<N, PS, MT>;
   fence_proxy_async_smem();
   const unsigned planes = G::kPlaneBytes * (unsigned)(k_hi - k_lo + 1);
   // C-PML strip boxes of the axes the unit reaches (all mechanisms)
   const int xside = N > 0 ? R.xs_side(x0) : -1;
   const int yrow = N > 0 ? R.ys_row(y0) : INT_MIN;
   const int zpl = N > 0 ? R.zs_plane(k) : -1;
-  const unsigned xs = xside >= 0 ? 2u * 2u * (unsigned)(N * kHT * R.xsL) : 0u;
-  const unsigned yz = (yrow != INT_MIN ? 2u * 2u * N * kArr : 0u) + (zpl >= 0 ? 2u * 2u * N * kArr : 0u);
-  float *ss = st + (VEL ? Vel3<N, PS>::oS : Prs3<N, CROSS, PS>::oS);
+  constexpr unsigned kE = sizeof(MT);
+  const unsigned xs = xside >= 0 ? 2u * kE * (unsigned)(N * kHT * R.xsL) : 0u;
+  const unsigned yz = (yrow != INT_MIN ? 2u * kE * N * kArr : 0u) + (zpl >= 0 ? 2u * kE * N * kArr : 0u);
+  float *ss = st + (VEL ? Vel3<N, PS, MT>::oS : Prs3<N, CROSS, PS, MT>::oS);
   auto load_strips = [&] {
     if (xside >= 0) {
       tma_load_4d(ss + SS::oXa, &T.m[10], xside * R.xsL, y0, k, 0, bar);
@@ -215,7 +229,7 @@ __device__ __forceinline__ void issue3(const PipeMaps &T, const Region3 &R, floa
     }
   };
   if (VEL) {
-    using S = Vel3<N, PS>;
+    using S = Vel3<N, PS, MT>;
     mbar_arrive_expect_tx(bar, S::kBytes + (nl_vel ? S::kKmBytes : 0u) + planes + xs + yz);
     load_strips();
     for (int kp = k_lo; kp <= k_hi; ++kp) tma_load_3d(ring + ring_slot(kp) * G::kPlane, &T.m[0], x0 - 4, y0 - 3, kp, bar);
@@ -229,9 +243,9 @@ __device__ __forceinline__ void issue3(const PipeMaps &T, const Region3 &R, floa
     }
     if (!PS && nl_vel) tma_load_3d(st + S::oKm, &T.m[12], x0, y0, k, bar);
   } else {
-    using S = Prs3<N, CROSS, PS>;
+    using S = Prs3<N, CROSS, PS, MT>;
     const unsigned subs = CROSS ? (S::kXPlaneBytes + S::kYPlaneBytes) * (unsigned)(s_hi - s_lo + 1) : 0u;
-    mbar_arrive_expect_tx(bar, S::kBytesNoChi + (nl ? 2u * kArr : 0u) + planes + subs + xs + yz);
+    mbar_arrive_expect_tx(bar, S::kBytesNoChi + (nl ? kE * kArr : 0u) + planes + subs + xs + yz);
     load_strips();
     if (CROSS) {
       for (int kp = k_lo; kp <= k_hi; ++kp) tma_load_3d(ring + ring_slot(kp) * G::kPlane, &T.m[2], x0 - 4, y0 - 1, kp, bar);
@@ -270,6 +284,12 @@ __device__ __forceinline__ float2 sldb2(const bf16 *s) {  // bf16 maps hold 1 - 
   const float2 v = sldh2(s);
   return make_float2(1.f - v.x, 1.f - v.y);
 }
+__device__ __forceinline__ float2 sldh2(const float *s) { return sld2(s); }
+__device__ __forceinline__ float2 sldb2(const float *s) { return sld2(s); }
+__device__ __forceinline__ float sldh1(const bf16 *s) { return __bfloat162float(*s); }
+__device__ __forceinline__ float sldh1(const float *s) { return *s; }
+__device__ __forceinline__ float sldb1(const bf16 *s) { return 1.f - __bfloat162float(*s); }
+__device__ __forceinline__ float sldb1(const float *s) { return *s; }
 __device__ __forceinline__ void st_state2(float *p, long long i, float2 v) {
   __stcs(reinterpret_cast<float2 *>(p + i), v);
 }
@@ -327,25 +347,23 @@ __device__ __forceinline__ void load_psi(float *const *psi, long long Sn, long l
 // cells of an edge pair, from that axis' C-PML strip in global memory where
 // the cells lie in it (coef4 of the tile kernels; its zero beyond the grid
 // only reaches masked cells); unchanged elsewhere
-template <int Q, int OP>
+template <int Q, int OP, typename MT>
 __device__ __forceinline__ void strip3(const StepParams &P, int nu, int i0, int j, int k, float2 &a, float2 &b) {
-  const bf16 *sa = static_cast<const bf16 *>(OP == 1 ? P.sa1[Q] : P.sa2[Q]);
-  const bf16 *sb = static_cast<const bf16 *>(OP == 1 ? P.sb1[Q] : P.sb2[Q]);
+  const MT *sa = static_cast<const MT *>(OP == 1 ? P.sa1[Q] : P.sa2[Q]);
+  const MT *sb = static_cast<const MT *>(OP == 1 ? P.sb1[Q] : P.sb2[Q]);
   const int L = P.L[Q];
   if (L <= 0) return;
   if (Q == 0) {
     if (!(i0 < L || i0 + 1 >= P.nx - L)) return;
     const long long row = (long long)nu * P.strip_nu[0] + ((long long)k * P.ny + j) * (2 * L);
-    // both cells on one side of the strip: one aligned bf16 pair (i0 and
+    // both cells on one side of the strip: one aligned pair (i0 and
     // the high side's offset nx - 2L are even)
     int sc0 = -1;
     if (i0 + 1 < L) sc0 = i0;
     else if (i0 >= P.nx - L && i0 + 1 < P.nx && ((P.nx - 2 * L) & 1) == 0) sc0 = i0 - (P.nx - 2 * L);
     if (sc0 >= 0) {
-      const float2 va = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(sa + row + sc0));
-      const float2 vb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(sb + row + sc0));
-      a = va;
-      b = make_float2(1.f - vb.x, 1.f - vb.y);
+      a = sldh2(sa + row + sc0);
+      b = sldb2(sb + row + sc0);
       return;
     }
 #pragma unroll
@@ -364,18 +382,17 @@ __device__ __forceinline__ void strip3(const StepParams &P, int nu, int i0, int 
     if (sc < 0) return;
     const long long off = Q == 1 ? (long long)nu * P.strip_nu[1] + ((long long)k * (2 * L) + sc) * P.pitch + i0
                                  : (long long)nu * P.strip_nu[2] + ((long long)sc * P.ny + j) * P.pitch + i0;
-    // i0 even, pitch a multiple of 16: an aligned bf16 pair
-    const float2 va = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(sa + off));
-    const float2 vb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(sb + off));
-    a = va;
-    b = make_float2(1.f - vb.x, 1.f - vb.y);
+    // i0 even, pitch a multiple of 16: an aligned pair
+    a = sldh2(sa + off);
+    b = sldb2(sb + off);
   }
 }
 
 // a, b of the x strip at the two cells of an edge pair from the staged boxes
-// (each [N][8][L] bf16, the side the unit reaches): the values strip3<0>
+// (each [N][8][L], the side the unit reaches): the values strip3<0>
 // reads from global memory, for the cells in the strip
-__device__ __forceinline__ void strip3x_staged(const StepParams &P, const bf16 *xa, const bf16 *xb, int xsL, int nu,
+template <typename MT>
+__device__ __forceinline__ void strip3x_staged(const StepParams &P, const MT *xa, const MT *xb, int xsL, int nu,
                                                int i0, int ly, float2 &a, float2 &b) {
   const int L = P.L[0];
 #pragma unroll
@@ -385,8 +402,8 @@ __device__ __forceinline__ void strip3x_staged(const StepParams &P, const bf16 *
       const int sc = strip_coord(x, P.nx, L);
       if (sc >= 0) {
         const int i = (nu * kHT + ly) * xsL + (sc >= L ? sc - L : sc);
-        el2(a, e) = __bfloat162float(xa[i]);
-        el2(b, e) = 1.f - __bfloat162float(xb[i]);
+        el2(a, e) = sldh1(xa + i);
+        el2(b, e) = sldb1(xb + i);
       }
     }
   }
@@ -394,31 +411,31 @@ __device__ __forceinline__ void strip3x_staged(const StepParams &P, const bf16 *
 
 // All C-PML coefficient overrides of an edge pair for mechanism nu (axes x,
 // y, z), from the staged boxes where the unit has them, else global memory.
-template <int N, int OP, bool PS>
+template <int N, int OP, bool PS, typename MT>
 __device__ __forceinline__ void strips_of(const StepParams &P, const Region3 &R, const float *ss, int xside, bool ys,
                                           bool zs, int nu, int i0, int j, int k, int ly, int lx, float2 (&A)[3],
                                           float2 (&B)[3]) {
-  using SS = Strips<N, PS>;
+  using SS = Strips<N, PS, MT>;
   if (xside >= 0)
-    strip3x_staged(P, reinterpret_cast<const bf16 *>(ss + SS::oXa), reinterpret_cast<const bf16 *>(ss + SS::oXb),
+    strip3x_staged(P, reinterpret_cast<const MT *>(ss + SS::oXa), reinterpret_cast<const MT *>(ss + SS::oXb),
                    R.xsL, nu, i0, ly, A[0], B[0]);
   else
-    strip3<0, OP>(P, nu, i0, j, k, A[0], B[0]);
+    strip3<0, OP, MT>(P, nu, i0, j, k, A[0], B[0]);
   if (ys) {
     if (strip_coord(j, P.ny, P.L[1]) >= 0) {
       const int o = nu * kArr + ly * kTX + lx;
-      A[1] = sldh2(reinterpret_cast<const bf16 *>(ss + SS::oYa) + o);
-      B[1] = sldb2(reinterpret_cast<const bf16 *>(ss + SS::oYb) + o);
+      A[1] = sldh2(reinterpret_cast<const MT *>(ss + SS::oYa) + o);
+      B[1] = sldb2(reinterpret_cast<const MT *>(ss + SS::oYb) + o);
     }
   } else {
-    strip3<1, OP>(P, nu, i0, j, k, A[1], B[1]);
+    strip3<1, OP, MT>(P, nu, i0, j, k, A[1], B[1]);
   }
   if (zs) {
     const int o = nu * kArr + ly * kTX + lx;
-    A[2] = sldh2(reinterpret_cast<const bf16 *>(ss + SS::oZa) + o);
-    B[2] = sldb2(reinterpret_cast<const bf16 *>(ss + SS::oZb) + o);
+    A[2] = sldh2(reinterpret_cast<const MT *>(ss + SS::oZa) + o);
+    B[2] = sldb2(reinterpret_cast<const MT *>(ss + SS::oZb) + o);
   } else {
-    strip3<2, OP>(P, nu, i0, j, k, A[2], B[2]);
+    strip3<2, OP, MT>(P, nu, i0, j, k, A[2], B[2]);
   }
 }
 
@@ -426,15 +443,16 @@ __device__ __forceinline__ void strips_of(const StepParams &P, const Region3 &R,
 // global memory (warp 0, one unit ahead): only strips without a staged box.
 // OP: 1 velocity (a1, b1), 2 pressure (a2, b2).
 __device__ __forceinline__ void l2_line(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-template <int N, int OP>
+template <int N, int OP, typename MT>
 __device__ __forceinline__ void prefetch_strips(const StepParams &P, const Region3 &R, int x0, int y0, int k,
                                                 int lane) {
   if constexpr (N > 0) {
-    const bf16 *sa[3], *sb[3];
+    constexpr int kLine = 128 / (int)sizeof(MT);  // elements of a 128-byte line
+    const MT *sa[3], *sb[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      sa[q] = static_cast<const bf16 *>(OP == 1 ? P.sa1[q] : P.sa2[q]);
-      sb[q] = static_cast<const bf16 *>(OP == 1 ? P.sb1[q] : P.sb2[q]);
+      sa[q] = static_cast<const MT *>(OP == 1 ? P.sa1[q] : P.sa2[q]);
+      sb[q] = static_cast<const MT *>(OP == 1 ? P.sb1[q] : P.sb2[q]);
     }
     // x strip: rows (k, y) of 2L values, for units reaching into it
     const int Lx = P.L[0];
@@ -443,8 +461,8 @@ __device__ __forceinline__ void prefetch_strips(const StepParams &P, const Regio
         const int r = t % kHT, nu = (t / kHT) % N, ab = t / (kHT * N);
         const int y = y0 + r;
         if (y >= P.ny) continue;
-        const bf16 *b = (ab ? sb[0] : sa[0]) + nu * P.strip_nu[0] + ((long long)k * P.ny + y) * (2 * Lx);
-        for (int o = 0; o < 2 * Lx; o += 64) l2_line(b + o);  // 128-byte lines
+        const MT *b = (ab ? sb[0] : sa[0]) + nu * P.strip_nu[0] + ((long long)k * P.ny + y) * (2 * Lx);
+        for (int o = 0; o < 2 * Lx; o += kLine) l2_line(b + o);
       }
     }
     // y strip: rows (k, sc) of the unit's 128 columns
@@ -455,9 +473,8 @@ __device__ __forceinline__ void prefetch_strips(const StepParams &P, const Regio
         const int y = y0 + r;
         const int sc = y < P.ny ? strip_coord(y, P.ny, Ly) : -1;
         if (sc < 0) continue;
-        const bf16 *b = (ab ? sb[1] : sa[1]) + nu * P.strip_nu[1] + ((long long)k * (2 * Ly) + sc) * P.pitch + x0;
-        l2_line(b);
-        if (x0 + 64 < P.nx) l2_line(b + 64);
+        const MT *b = (ab ? sb[1] : sa[1]) + nu * P.strip_nu[1] + ((long long)k * (2 * Ly) + sc) * P.pitch + x0;
+        for (int o = 0; o < kTX && x0 + o < P.nx; o += kLine) l2_line(b + o);
       }
     }
     // z strip: plane sc, rows y of the unit
@@ -468,9 +485,8 @@ __device__ __forceinline__ void prefetch_strips(const StepParams &P, const Regio
         const int r = t % kHT, nu = (t / kHT) % N, ab = t / (kHT * N);
         const int y = y0 + r;
         if (y >= P.ny) continue;
-        const bf16 *b = (ab ? sb[2] : sa[2]) + nu * P.strip_nu[2] + ((long long)scz * P.ny + y) * P.pitch + x0;
-        l2_line(b);
-        if (x0 + 64 < P.nx) l2_line(b + 64);
+        const MT *b = (ab ? sb[2] : sa[2]) + nu * P.strip_nu[2] + ((long long)scz * P.ny + y) * P.pitch + x0;
+        for (int o = 0; o < kTX && x0 + o < P.nx; o += kLine) l2_line(b + o);
       }
     }
   }
@@ -482,15 +498,15 @@ __device__ __forceinline__ float mom_factor_ik(float ika, float ikb, float pa, f
   return fmaf(0.5f * (ika + ikb), 0.5f * (pa + pb), 1.f);
 }
 
-// Values at the faces of a pair read from a staged bf16 box [2][9][136]
+// Values at the faces of a pair read from a staged box [2][9][kRW]
 // (planes k, k + 1: the density, or K): plane k row ly at lx .. lx+2, row
 // ly+1 at lx, lx+1; plane k+1 row ly at lx, lx+1.  Cells beyond the last one
 // along an axis take that cell's value (rho_coord of the tile kernels).
 struct Face3 {
   float r0, r1, r2, u0, u1, z0, z1;
 };
-template <bool EDGE>
-__device__ __forceinline__ Face3 face3(const StepParams &P, const bf16 *rb, int x0, int y0, int k, int lx, int ly) {
+template <bool EDGE, typename MT>
+__device__ __forceinline__ Face3 face3(const StepParams &P, const MT *rb, int x0, int y0, int k, int lx, int ly) {
   int c0 = lx, c1 = lx + 1, c2 = lx + 2, r0 = ly, r1 = ly + 1, pz = 1;
   if (EDGE) {
     const int mx = P.nx - 1 - x0, my = P.ny - 1 - y0;
@@ -501,7 +517,7 @@ __device__ __forceinline__ Face3 face3(const StepParams &P, const bf16 *rb, int 
     r1 = min(r1, my);
     if (k + 1 >= P.nz) pz = 0;
   }
-  auto at = [&](int z, int r, int cc) { return __bfloat162float(rb[(z * (kHT + 1) + r) * kRWb + cc]); };
+  auto at = [&](int z, int r, int cc) { return sldh1(rb + (z * (kHT + 1) + r) * kRW<MT> + cc); };
   return Face3{at(0, r0, c0), at(0, r0, c1), at(0, r0, c2), at(0, r1, c0), at(0, r1, c1),
                at(pz, r0, c0), at(pz, r0, c1)};
 }
@@ -526,10 +542,10 @@ __device__ __forceinline__ void relax3(const StepParams &P, float *const *psi, l
   }
 }
 
-template <int N, bool EDGE, bool CROSS, bool PS>
+template <int N, bool EDGE, bool CROSS, bool PS, typename MT>
 __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 &R, float *st, const float *ring,
                                              int x0, int y0, int k, int tid, const Psi<N> &q) {
-  using S = Vel3<N, PS>;
+  using S = Vel3<N, PS, MT>;
   const int lx = 2 * (tid & 63), ly = tid >> 6;
   const int i0 = x0 + lx, j = y0 + ly;
   if (EDGE && (i0 >= P.nx || j >= P.ny)) return;
@@ -596,7 +612,7 @@ __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 
                                 ((zp_up.v[2 + e] - up.v[2 + e]) + (zp_dn.v[2 + e] - dn.v[2 + e]))), el2(D[2], e));
     }
   }
-  const float2 k1 = sldh2(reinterpret_cast<const bf16 *>(st + S::oK) + o);
+  const float2 k1 = sldh2(reinterpret_cast<const MT *>(st + S::oK) + o);
   float2 v0 = sld2(st + S::oV + o), v1 = sld2(st + S::oV + kArr + o), v2 = sld2(st + S::oV + 2 * kArr + o);
   float2 Sd[3];
 #pragma unroll
@@ -611,14 +627,14 @@ __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 
   float2 A[N > 0 ? N : 1][3], B[N > 0 ? N : 1][3];
 #pragma unroll
   for (int nu = 0; nu < N; ++nu) {
-    const float2 a = sldh2(reinterpret_cast<const bf16 *>(st + S::oA) + nu * kArr + o);
-    const float2 b = sldb2(reinterpret_cast<const bf16 *>(st + S::oB) + nu * kArr + o);
+    const float2 a = sldh2(reinterpret_cast<const MT *>(st + S::oA) + nu * kArr + o);
+    const float2 b = sldb2(reinterpret_cast<const MT *>(st + S::oB) + nu * kArr + o);
 #pragma unroll
     for (int a3 = 0; a3 < 3; ++a3) {
       A[nu][a3] = a;
       B[nu][a3] = b;
     }
-    if (EDGE) strips_of<N, 1, PS>(P, R, st + S::oS, xside, ys, zs, nu, i0, j, k, ly, lx, A[nu], B[nu]);
+    if (EDGE) strips_of<N, 1, PS, MT>(P, R, st + S::oS, xside, ys, zs, nu, i0, j, k, ly, lx, A[nu], B[nu]);
   }
 #pragma unroll
   for (int nu = 0; nu < N; ++nu) {
@@ -627,13 +643,13 @@ __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 
     for (int a3 = 0; a3 < 3; ++a3) qq[a3] = PS ? sld2(st + S::oPsi + (a3 * N + nu) * kArr + o) : q[a3][nu];
     relax3(P, P.psi1, nu * Sn + c, i0, EDGE, qq, A[nu], B[nu], D, Sd);
   }
-  const Face3 f = face3<EDGE>(P, reinterpret_cast<const bf16 *>(st + S::oRho), x0, y0, k, lx, ly);
+  const Face3 f = face3<EDGE, MT>(P, reinterpret_cast<const MT *>(st + S::oRho), x0, y0, k, lx, ly);
   const float rr[3] = {f.r0, f.r1, f.r2}, ru[2] = {f.u0, f.u1}, rz[2] = {f.z0, f.z1};
   if (P.nl_vel) {
     // momentum factors of the literal system (Eq. general5) at the x, y, z
     // faces: p from the staged planes (zero beyond the grid), K of the cell
     // and of its +1 neighbours from the staged K box, clamped to the last cell
-    const Face3 g = face3<EDGE>(P, reinterpret_cast<const bf16 *>(st + S::oKm), x0, y0, k, lx, ly);
+    const Face3 g = face3<EDGE, MT>(P, reinterpret_cast<const MT *>(st + S::oKm), x0, y0, k, lx, ly);
     // 1 / K of each of the seven cells once (mom_factor takes them the same way)
     const float Kr[3] = {qdiv(1.f, g.r0), qdiv(1.f, g.r1), qdiv(1.f, g.r2)};
     const float Ku[2] = {qdiv(1.f, g.u0), qdiv(1.f, g.u1)}, Kz[2] = {qdiv(1.f, g.z0), qdiv(1.f, g.z1)};
@@ -666,10 +682,10 @@ __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 
   st_state2(P.v[2], c, v2);
 }
 
-template <int N, bool EDGE, bool CROSS, bool PS>
+template <int N, bool EDGE, bool CROSS, bool PS, typename MT>
 __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 &R, const float *st, const float *ring,
                                              const float *sub, int x0, int y0, int k, int tid, const Psi<N> &q) {
-  using S = Prs3<N, CROSS, PS>;
+  using S = Prs3<N, CROSS, PS, MT>;
   const int lx = 2 * (tid & 63), ly = tid >> 6;
   const int i0 = x0 + lx, j = y0 + ly;
   if (EDGE && (i0 >= P.nx || j >= P.ny)) return;
@@ -757,10 +773,10 @@ __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 
                                   ((u0.v[2 + e] - u1.v[2 + e]) + (d0.v[2 + e] - d1.v[2 + e]))), el2(D[2], e));
     }
   }
-  const float2 k2 = sldh2(reinterpret_cast<const bf16 *>(st + S::oIk) + o);
-  const float2 K = sldh2(reinterpret_cast<const bf16 *>(st + S::oKm) + o);
+  const float2 k2 = sldh2(reinterpret_cast<const MT *>(st + S::oIk) + o);
+  const float2 K = sldh2(reinterpret_cast<const MT *>(st + S::oKm) + o);
   float2 ch = make_float2(0.f, 0.f);
-  if (P.nl) ch = sldh2(reinterpret_cast<const bf16 *>(st + S::oChi) + o);
+  if (P.nl) ch = sldh2(reinterpret_cast<const MT *>(st + S::oChi) + o);
   float2 p = sld2(st + S::oP + o);
   float2 Sd[3];
 #pragma unroll
@@ -775,14 +791,14 @@ __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 
   float2 A[N > 0 ? N : 1][3], B[N > 0 ? N : 1][3];
 #pragma unroll
   for (int nu = 0; nu < N; ++nu) {
-    const float2 a = sldh2(reinterpret_cast<const bf16 *>(st + S::oA) + nu * kArr + o);
-    const float2 b = sldb2(reinterpret_cast<const bf16 *>(st + S::oB) + nu * kArr + o);
+    const float2 a = sldh2(reinterpret_cast<const MT *>(st + S::oA) + nu * kArr + o);
+    const float2 b = sldb2(reinterpret_cast<const MT *>(st + S::oB) + nu * kArr + o);
 #pragma unroll
     for (int a3 = 0; a3 < 3; ++a3) {
       A[nu][a3] = a;
       B[nu][a3] = b;
     }
-    if (EDGE) strips_of<N, 2, PS>(P, R, st + S::oS, xside, ys, zs, nu, i0, j, k, ly, lx, A[nu], B[nu]);
+    if (EDGE) strips_of<N, 2, PS, MT>(P, R, st + S::oS, xside, ys, zs, nu, i0, j, k, ly, lx, A[nu], B[nu]);
   }
 #pragma unroll
   for (int nu = 0; nu < N; ++nu) {
@@ -803,10 +819,10 @@ __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 
 
 // One half step.  Block (32, 16), one per SM; items blockIdx.x,
 // blockIdx.x + gridDim.x, ...; within an item the units k0 .. k1-1 in order.
-template <int N, bool VEL, bool CROSS, bool PS>
+template <int N, bool VEL, bool CROSS, bool PS, typename MT>
 __global__ void __launch_bounds__(kThreads, 1)
     pipe3d_kernel(const StepParams P, const Region3 R, const __grid_constant__ PipeMaps T) {
-  using G = Ring3<N, VEL, CROSS, PS>;
+  using G = Ring3<N, VEL, CROSS, PS, MT>;
   constexpr int kStage = G::kStage;
   extern __shared__ __align__(128) float smem_raw[];
   __shared__ __align__(8) uint64_t bar[2];
@@ -822,7 +838,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   __syncthreads();
   const long long n_items = R.items();
-  long long it = blockIdx.x;
+  // this block's items: one per round of gridDim.x consecutive ones, rotated
+  // by R.rot blocks from round to round (without it a block whose grid and
+  // column counts share factors meets few columns: 152 blocks and 4 columns
+  // give half the blocks nothing but x-edge units)
+  const long long grid = gridDim.x;
+  long long slot = blockIdx.x, it = slot;
   if (it >= n_items) return;
   int x0, y0, k0, k1;
   R.item(it, x0, y0, k0, k1);
@@ -830,7 +851,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   unsigned phase = 0, pending = 0;
   const bool nl = P.nl != 0, nlv = VEL && P.nl_vel != 0;
   if (tid == 0)
-    issue3<N, VEL, CROSS, PS>(T, R, smem, ring, sub, &bar[0], x0, y0, k, ring_first<VEL>(k), ring_first<VEL>(k) + 7,
+    issue3<N, VEL, CROSS, PS, MT>(T, R, smem, ring, sub, &bar[0], x0, y0, k, ring_first<VEL>(k), ring_first<VEL>(k) + 7,
                           k - 1, k + 1, nl, nlv);
   pending |= 1u;
   // this thread's memory variables, one unit ahead of the compute
@@ -861,7 +882,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     long long nit = it;
     int nx0 = x0, ny0 = y0, nk0 = k0, nk1 = k1, nk = k + 1;
     if (nk >= k1) {
-      nit = it + gridDim.x;
+      nit = it - slot + grid;
+      slot = slot + R.rot;
+      if (slot >= grid) slot -= grid;
+      nit += slot;
       if (nit < n_items) R.item(nit, nx0, ny0, nk0, nk1);
       nk = nk0;
     }
@@ -871,26 +895,26 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (tid < 32) {
         const int kp = ring_first<VEL>(nk) + 7;
         if (tid == 0)
-          issue3<N, VEL, CROSS, PS>(T, R, smem + q * kStage, ring, sub, &bar[q], nx0, ny0, nk, kp, kp, nk + 1, nk + 1,
+          issue3<N, VEL, CROSS, PS, MT>(T, R, smem + q * kStage, ring, sub, &bar[q], nx0, ny0, nk, kp, kp, nk + 1, nk + 1,
                                 nl, nlv);
-        if (!R.interior(nx0, ny0, nk)) prefetch_strips<N, VEL ? 1 : 2>(P, R, nx0, ny0, nk, tid);
+        if (!R.interior(nx0, ny0, nk)) prefetch_strips<N, VEL ? 1 : 2, MT>(P, R, nx0, ny0, nk, tid);
       }
       pending |= 1u << q;
     }
     if (!PS && more) psi_of(nx0, ny0, nk, qn);
     float *cur = smem + s * kStage;
     if (R.interior(x0, y0, k)) {
-      if (VEL) vel3_compute<N, false, CROSS, PS>(P, R, cur, ring, x0, y0, k, tid, qc);
-      else prs3_compute<N, false, CROSS, PS>(P, R, cur, ring, sub, x0, y0, k, tid, qc);
+      if (VEL) vel3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, x0, y0, k, tid, qc);
+      else prs3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, sub, x0, y0, k, tid, qc);
     } else {
-      if (VEL) vel3_compute<N, true, CROSS, PS>(P, R, cur, ring, x0, y0, k, tid, qc);
-      else prs3_compute<N, true, CROSS, PS>(P, R, cur, ring, sub, x0, y0, k, tid, qc);
+      if (VEL) vel3_compute<N, true, CROSS, PS, MT>(P, R, cur, ring, x0, y0, k, tid, qc);
+      else prs3_compute<N, true, CROSS, PS, MT>(P, R, cur, ring, sub, x0, y0, k, tid, qc);
     }
     if (!more) break;
     if (fresh) {  // a new column: all ring planes, once every thread is done with the rings
       __syncthreads();
       if (tid == 0)
-        issue3<N, VEL, CROSS, PS>(T, R, smem + q * kStage, ring, sub, &bar[q], nx0, ny0, nk, ring_first<VEL>(nk),
+        issue3<N, VEL, CROSS, PS, MT>(T, R, smem + q * kStage, ring, sub, &bar[q], nx0, ny0, nk, ring_first<VEL>(nk),
                               ring_first<VEL>(nk) + 7, nk - 1, nk + 1, nl, nlv);
       pending |= 1u << q;
     }
@@ -906,6 +930,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+#ifndef FW2_PIPE3D_FLOAT
 // The same half step for several contexts in one launch (a batch of 3D
 // problems): a table of work items {context, item of that context}; each
 // block takes a contiguous run of the table, so consecutive items mostly
@@ -917,7 +942,7 @@ template <int N, bool VEL, bool CROSS, bool PS>
 __global__ void __launch_bounds__(kThreads, 1)
     pipe3d_batched_kernel(const StepParams *Ps, const Region3 *Rs, const PipeMaps *Ts, const int2 *items,
                           const int *runs) {
-  using G = Ring3<N, VEL, CROSS, PS>;
+  using G = Ring3<N, VEL, CROSS, PS, bf16>;
   constexpr int kStage = G::kStage;
   extern __shared__ __align__(128) float smem_raw[];
   __shared__ __align__(8) uint64_t bar[2];
@@ -962,7 +987,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   };
   if (tid == 0) acquire(ctx);
   if (tid == 0)
-    issue3<N, VEL, CROSS, PS>(Ts[ctx], sR, smem, ring, sub, &bar[0], x0, y0, k, ring_first<VEL>(k),
+    issue3<N, VEL, CROSS, PS, bf16>(Ts[ctx], sR, smem, ring, sub, &bar[0], x0, y0, k, ring_first<VEL>(k),
                               ring_first<VEL>(k) + 7, k - 1, k + 1, nl, nlv);
   pending |= 1u;
   const int lx = 2 * (tid & 63), ly = tid >> 6;
@@ -1004,20 +1029,20 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (tid < 32) {
         const int kp = ring_first<VEL>(nk) + 7;
         if (tid == 0)
-          issue3<N, VEL, CROSS, PS>(Ts[ctx], sR, smem + q * kStage, ring, sub, &bar[q], nx0, ny0, nk, kp, kp,
+          issue3<N, VEL, CROSS, PS, bf16>(Ts[ctx], sR, smem + q * kStage, ring, sub, &bar[q], nx0, ny0, nk, kp, kp,
                                     nk + 1, nk + 1, nl, nlv);
-        if (!sR.interior(nx0, ny0, nk)) prefetch_strips<N, VEL ? 1 : 2>(sP, sR, nx0, ny0, nk, tid);
+        if (!sR.interior(nx0, ny0, nk)) prefetch_strips<N, VEL ? 1 : 2, bf16>(sP, sR, nx0, ny0, nk, tid);
       }
       pending |= 1u << q;
     }
     if (!PS && more) psi_of(nctx == ctx ? sP : Ps[nctx], nx0, ny0, nk, qn);
     float *cur = smem + s * kStage;
     if (sR.interior(x0, y0, k)) {
-      if (VEL) vel3_compute<N, false, CROSS, PS>(sP, sR, cur, ring, x0, y0, k, tid, qc);
-      else prs3_compute<N, false, CROSS, PS>(sP, sR, cur, ring, sub, x0, y0, k, tid, qc);
+      if (VEL) vel3_compute<N, false, CROSS, PS, bf16>(sP, sR, cur, ring, x0, y0, k, tid, qc);
+      else prs3_compute<N, false, CROSS, PS, bf16>(sP, sR, cur, ring, sub, x0, y0, k, tid, qc);
     } else {
-      if (VEL) vel3_compute<N, true, CROSS, PS>(sP, sR, cur, ring, x0, y0, k, tid, qc);
-      else prs3_compute<N, true, CROSS, PS>(sP, sR, cur, ring, sub, x0, y0, k, tid, qc);
+      if (VEL) vel3_compute<N, true, CROSS, PS, bf16>(sP, sR, cur, ring, x0, y0, k, tid, qc);
+      else prs3_compute<N, true, CROSS, PS, bf16>(sP, sR, cur, ring, sub, x0, y0, k, tid, qc);
     }
     if (!more) break;
     if (fresh) {  // a new item: every thread is done with the rings (and the context's parameters)
@@ -1031,7 +1056,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (tid == 0) acquire(ctx);
       }
       if (tid == 0)
-        issue3<N, VEL, CROSS, PS>(Ts[ctx], sR, smem + q * kStage, ring, sub, &bar[q], nx0, ny0, nk,
+        issue3<N, VEL, CROSS, PS, bf16>(Ts[ctx], sR, smem + q * kStage, ring, sub, &bar[q], nx0, ny0, nk,
                                   ring_first<VEL>(nk), ring_first<VEL>(nk) + 7, nk - 1, nk + 1, nl, nlv);
       pending |= 1u << q;
     }
@@ -1050,7 +1075,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int N, bool VEL, bool CROSS, bool PS>
 cudaError_t pipe3_batched_launch(const StepParams *Ps, const Region3 *Rs, const PipeMaps *Ts, const int2 *items,
                                  const int *runs, int grid, cudaStream_t st) {
-  constexpr size_t bytes = Ring3<N, VEL, CROSS, PS>::kBytes;
+  constexpr size_t bytes = Ring3<N, VEL, CROSS, PS, bf16>::kBytes;
   cudaError_t e = cudaFuncSetAttribute(pipe3d_batched_kernel<N, VEL, CROSS, PS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
@@ -1070,33 +1095,39 @@ cudaError_t pipe3_batched_dispatch(int n_relax, const StepParams *Ps, const Regi
   }
 }
 
-template <int N, bool VEL, bool CROSS, bool PS>
+#endif  // FW2_PIPE3D_FLOAT
+
+template <int N, bool VEL, bool CROSS, bool PS, typename MT>
 cudaError_t pipe3_launch(const StepParams &P, const Region3 &R, int grid, const PipeMaps &T, cudaStream_t st) {
-  constexpr size_t bytes = Ring3<N, VEL, CROSS, PS>::kBytes;
+  constexpr size_t bytes = Ring3<N, VEL, CROSS, PS, MT>::kBytes;
   static_assert(bytes + 64 <= 227 * 1024, "stages exceed shared memory");
-  cudaError_t e = cudaFuncSetAttribute(pipe3d_kernel<N, VEL, CROSS, PS>,
+  cudaError_t e = cudaFuncSetAttribute(pipe3d_kernel<N, VEL, CROSS, PS, MT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
-  pipe3d_kernel<N, VEL, CROSS, PS><<<grid, dim3(32, kThreads / 32), bytes, st>>>(P, R, T);
+  pipe3d_kernel<N, VEL, CROSS, PS, MT><<<grid, dim3(32, kThreads / 32), bytes, st>>>(P, R, T);
   return cudaGetLastError();
 }
 
-template <bool VEL, bool CROSS, bool PS>
+template <bool VEL, bool CROSS, bool PS, typename MT>
 cudaError_t pipe3_dispatch(const StepParams &P, const Region3 &R, int grid, const PipeMaps &T, cudaStream_t st) {
   switch (P.n_relax) {
-    case 0: return pipe3_launch<0, VEL, CROSS, PS>(P, R, grid, T, st);
-    case 1: return pipe3_launch<1, VEL, CROSS, PS>(P, R, grid, T, st);
-    case 2: return pipe3_launch<2, VEL, CROSS, PS>(P, R, grid, T, st);
-    case 3: return pipe3_launch<3, VEL, CROSS, PS>(P, R, grid, T, st);
+    case 0: return pipe3_launch<0, VEL, CROSS, PS, MT>(P, R, grid, T, st);
+    case 1: return pipe3_launch<1, VEL, CROSS, PS, MT>(P, R, grid, T, st);
+    case 2: return pipe3_launch<2, VEL, CROSS, PS, MT>(P, R, grid, T, st);
+    case 3: return pipe3_launch<3, VEL, CROSS, PS, MT>(P, R, grid, T, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
+#ifndef FW2_PIPE3D_FLOAT
 // The layout of a half step: the memory variables staged with the other
 // arrays (PS) unless the stage needs that room for the cross taps' planes
 // or (velocity) the literal system's K box; then they are loaded into
 // registers one unit ahead and the C-PML strips of every axis are staged.
-bool psi_staged(bool vel, const StepParams &P) { return P.g11h == 0.f && !(vel && P.nl_vel); }
+// Float maps take the register layout (the staged one does not fit).
+bool psi_staged(bool vel, const StepParams &P) {
+  return P.map_kind == 1 && P.g11h == 0.f && !(vel && P.nl_vel);
+}
 
 // The x strip's coefficients come by TMA when a box of L values per row
 // starts on a 16-byte boundary and fits the stage (L a multiple of 8, at
@@ -1133,8 +1164,9 @@ Region3 region3_of(const StepParams &P, int grid, bool ps) {
   R.tnx = (P.nx + kTX - 1) / kTX;
   R.nhy = (P.ny + kHT - 1) / kHT;
   R.xsL = x_strip_staged(P) ? P.L[0] : 0;
-  R.ysL = !ps && y_strip_staged(P) ? P.L[1] : 0;
-  R.zsL = !ps && z_strip_staged(P) ? P.L[2] : 0;
+  const bool yz = !ps && P.map_kind == 1;
+  R.ysL = yz && y_strip_staged(P) ? P.L[1] : 0;
+  R.zsL = yz && z_strip_staged(P) ? P.L[2] : 0;
   const long long ncols = (long long)R.tnx * R.nhy;
   double best = 1e300;
   R.seglen = P.nz;
@@ -1151,15 +1183,31 @@ Region3 region3_of(const StepParams &P, int grid, bool ps) {
       R.nseg = used;
     }
   }
+  R.rot = 0;
   return R;
 }
 
+#endif  // FW2_PIPE3D_FLOAT
 }  // namespace
 
+#ifdef FW2_PIPE3D_FLOAT
+// The second object of this file: the kernels for float maps (register
+// layout), built beside those for bf16 maps.
+cudaError_t launch_pipe3d_float(bool vel, const StepParams &P, const void *region, int grid, const PipeMaps &T,
+                                cudaStream_t st) {
+  const Region3 &R = *static_cast<const Region3 *>(region);
+  if (P.g11h != 0.f)
+    return vel ? pipe3_dispatch<true, true, false, float>(P, R, grid, T, st)
+               : pipe3_dispatch<false, true, false, float>(P, R, grid, T, st);
+  return vel ? pipe3_dispatch<true, false, false, float>(P, R, grid, T, st)
+             : pipe3_dispatch<false, false, false, float>(P, R, grid, T, st);
+}
+#else
+
 bool pipe3d_supported(const StepParams &P, int map_kind) {
-  // bf16 maps; N <= 3 keeps the 4D boxes and the stages within shared
-  // memory; no periodic axis
-  return P.nz > 1 && map_kind == 1 && P.n_relax >= 0 && P.n_relax <= 3 && !P.periodic[0] && !P.periodic[1] &&
+  // bf16 or float maps; N <= 3 keeps the 4D boxes and the stages within
+  // shared memory; no periodic axis
+  return P.nz > 1 && (map_kind == 1 || map_kind == 0) && P.n_relax >= 0 && P.n_relax <= 3 && !P.periodic[0] && !P.periodic[1] &&
          !P.periodic[2];
 }
 
@@ -1169,27 +1217,28 @@ cudaError_t build_pipe3d_maps(const StepParams &P, PipeMaps *vel, PipeMaps *prs,
   const int N = P.n_relax;
   const bool cross = P.g11h != 0.f;
   using ull = unsigned long long;
+  const int es = P.map_kind == 1 ? 2 : 4;  // bytes of a map value
   const ull nx = P.nx, ny = P.ny, nz = P.nz, S = P.npts_alloc;
-  const ull f3[2] = {(ull)P.pitch * 4, (ull)P.plane * 4}, h3[2] = {(ull)P.pitch * 2, (ull)P.plane * 2};
-  const ull f4[3] = {(ull)P.pitch * 4, (ull)P.plane * 4, S * 4}, h4[3] = {(ull)P.pitch * 2, (ull)P.plane * 2, S * 2};
+  const ull f3[2] = {(ull)P.pitch * 4, (ull)P.plane * 4}, h3[2] = {(ull)P.pitch * es, (ull)P.plane * es};
+  const ull f4[3] = {(ull)P.pitch * 4, (ull)P.plane * 4, S * 4}, h4[3] = {(ull)P.pitch * es, (ull)P.plane * es, S * es};
   const ull d3[3] = {nx, ny, nz};
   const ull dv[4] = {nx, ny, nz, 3}, dab[4] = {nx, ny, nz, (ull)N}, dpsi[4] = {nx, ny, nz, (ull)(3 * N)};
-  const unsigned halo[3] = {kCW, kHT + 7, 1}, rho[3] = {kRWb, kHT + 1, 2}, one[3] = {kTX, kHT, 1},
+  const unsigned halo[3] = {kCW, kHT + 7, 1}, rho[3] = {(unsigned)(es == 2 ? kRW<bf16> : kRW<float>), kHT + 1, 2}, one[3] = {kTX, kHT, 1},
                  v4[4] = {kTX, kHT, 1, 3}, ab4[4] = {kTX, kHT, 1, (unsigned)N},
                  psi4[4] = {kTX, kHT, 1, (unsigned)(3 * N)}, vx[3] = {kCW, kHT, 1},
                  vy[3] = {kTX, kHT + 7, 1}, halo1[3] = {kCW, kHT + 2, 1};
   bool ok = true;
   // velocity half step
   ok = ok && encode_tensor_map(&vel->m[0], P.p, 4, 3, d3, f3, halo);
-  ok = ok && encode_tensor_map(&vel->m[2], P.rho, 2, 3, d3, h3, rho);
+  ok = ok && encode_tensor_map(&vel->m[2], P.rho, es, 3, d3, h3, rho);
   ok = ok && encode_tensor_map(&vel->m[3], P.v[0], 4, 4, dv, f4, v4);
   if (N > 0) ok = ok && encode_tensor_map(&vel->m[4], P.psi1[0], 4, 4, dpsi, f4, psi4);
-  ok = ok && encode_tensor_map(&vel->m[5], P.ik1, 2, 3, d3, h3, one);
+  ok = ok && encode_tensor_map(&vel->m[5], P.ik1, es, 3, d3, h3, one);
   if (N > 0) {
-    ok = ok && encode_tensor_map(&vel->m[6], P.a1, 2, 4, dab, h4, ab4);
-    ok = ok && encode_tensor_map(&vel->m[7], P.b1, 2, 4, dab, h4, ab4);
+    ok = ok && encode_tensor_map(&vel->m[6], P.a1, es, 4, dab, h4, ab4);
+    ok = ok && encode_tensor_map(&vel->m[7], P.b1, es, 4, dab, h4, ab4);
   }
-  if (P.nl_vel) ok = ok && encode_tensor_map(&vel->m[12], P.K, 2, 3, d3, h3, rho);
+  if (P.nl_vel) ok = ok && encode_tensor_map(&vel->m[12], P.K, es, 3, d3, h3, rho);
   // pressure half step
   if (cross) {
     ok = ok && encode_tensor_map(&prs->m[0], P.v[0], 4, 3, d3, f3, halo1);
@@ -1202,39 +1251,39 @@ cudaError_t build_pipe3d_maps(const StepParams &P, PipeMaps *vel, PipeMaps *prs,
   }
   ok = ok && encode_tensor_map(&prs->m[3], P.p, 4, 3, d3, f3, one);
   if (N > 0) ok = ok && encode_tensor_map(&prs->m[4], P.psi2[0], 4, 4, dpsi, f4, psi4);
-  ok = ok && encode_tensor_map(&prs->m[5], P.ik2, 2, 3, d3, h3, one);
-  ok = ok && encode_tensor_map(&prs->m[6], P.K, 2, 3, d3, h3, one);
-  if (P.nl) ok = ok && encode_tensor_map(&prs->m[7], P.chi, 2, 3, d3, h3, one);
+  ok = ok && encode_tensor_map(&prs->m[5], P.ik2, es, 3, d3, h3, one);
+  ok = ok && encode_tensor_map(&prs->m[6], P.K, es, 3, d3, h3, one);
+  if (P.nl) ok = ok && encode_tensor_map(&prs->m[7], P.chi, es, 3, d3, h3, one);
   if (N > 0) {
-    ok = ok && encode_tensor_map(&prs->m[8], P.a2, 2, 4, dab, h4, ab4);
-    ok = ok && encode_tensor_map(&prs->m[9], P.b2, 2, 4, dab, h4, ab4);
+    ok = ok && encode_tensor_map(&prs->m[8], P.a2, es, 4, dab, h4, ab4);
+    ok = ok && encode_tensor_map(&prs->m[9], P.b2, es, 4, dab, h4, ab4);
   }
-  if (x_strip_staged(P)) {  // x strips [N][z][y][2L] bf16, boxes L x 8 x 1 x N
+  if (x_strip_staged(P)) {  // x strips [N][z][y][2L], boxes L x 8 x 1 x N
     const ull L = (ull)P.L[0];
-    const ull dxs[4] = {2 * L, ny, nz, (ull)N}, sxs[3] = {2 * L * 2, ny * 2 * L * 2, (ull)P.strip_nu[0] * 2};
+    const ull dxs[4] = {2 * L, ny, nz, (ull)N}, sxs[3] = {2 * L * es, ny * 2 * L * es, (ull)P.strip_nu[0] * es};
     const unsigned bxs[4] = {(unsigned)L, kHT, 1, (unsigned)N};
-    ok = ok && encode_tensor_map(&vel->m[10], P.sa1[0], 2, 4, dxs, sxs, bxs);
-    ok = ok && encode_tensor_map(&vel->m[11], P.sb1[0], 2, 4, dxs, sxs, bxs);
-    ok = ok && encode_tensor_map(&prs->m[10], P.sa2[0], 2, 4, dxs, sxs, bxs);
-    ok = ok && encode_tensor_map(&prs->m[11], P.sb2[0], 2, 4, dxs, sxs, bxs);
+    ok = ok && encode_tensor_map(&vel->m[10], P.sa1[0], es, 4, dxs, sxs, bxs);
+    ok = ok && encode_tensor_map(&vel->m[11], P.sb1[0], es, 4, dxs, sxs, bxs);
+    ok = ok && encode_tensor_map(&prs->m[10], P.sa2[0], es, 4, dxs, sxs, bxs);
+    ok = ok && encode_tensor_map(&prs->m[11], P.sb2[0], es, 4, dxs, sxs, bxs);
   }
-  if (y_strip_staged(P)) {  // y strips [N][z][2L][x] bf16, boxes 128 x 8 x 1 x N
+  if (y_strip_staged(P)) {  // y strips [N][z][2L][x], boxes 128 x 8 x 1 x N
     const ull L = (ull)P.L[1];
     const ull dys[4] = {nx, 2 * L, nz, (ull)N},
-              sys[3] = {(ull)P.pitch * 2, 2 * L * (ull)P.pitch * 2, (ull)P.strip_nu[1] * 2};
-    ok = ok && encode_tensor_map(&vel->m[13], P.sa1[1], 2, 4, dys, sys, ab4);
-    ok = ok && encode_tensor_map(&vel->m[14], P.sb1[1], 2, 4, dys, sys, ab4);
-    ok = ok && encode_tensor_map(&prs->m[13], P.sa2[1], 2, 4, dys, sys, ab4);
-    ok = ok && encode_tensor_map(&prs->m[14], P.sb2[1], 2, 4, dys, sys, ab4);
+              sys[3] = {(ull)P.pitch * es, 2 * L * (ull)P.pitch * es, (ull)P.strip_nu[1] * es};
+    ok = ok && encode_tensor_map(&vel->m[13], P.sa1[1], es, 4, dys, sys, ab4);
+    ok = ok && encode_tensor_map(&vel->m[14], P.sb1[1], es, 4, dys, sys, ab4);
+    ok = ok && encode_tensor_map(&prs->m[13], P.sa2[1], es, 4, dys, sys, ab4);
+    ok = ok && encode_tensor_map(&prs->m[14], P.sb2[1], es, 4, dys, sys, ab4);
   }
-  if (z_strip_staged(P)) {  // z strips [N][2L][y][x] bf16, boxes 128 x 8 x 1 x N
+  if (z_strip_staged(P)) {  // z strips [N][2L][y][x], boxes 128 x 8 x 1 x N
     const ull L = (ull)P.L[2];
     const ull dzs[4] = {nx, ny, 2 * L, (ull)N},
-              szs[3] = {(ull)P.pitch * 2, ny * (ull)P.pitch * 2, (ull)P.strip_nu[2] * 2};
-    ok = ok && encode_tensor_map(&vel->m[15], P.sa1[2], 2, 4, dzs, szs, ab4);
-    ok = ok && encode_tensor_map(&vel->m[16], P.sb1[2], 2, 4, dzs, szs, ab4);
-    ok = ok && encode_tensor_map(&prs->m[15], P.sa2[2], 2, 4, dzs, szs, ab4);
-    ok = ok && encode_tensor_map(&prs->m[16], P.sb2[2], 2, 4, dzs, szs, ab4);
+              szs[3] = {(ull)P.pitch * es, ny * (ull)P.pitch * es, (ull)P.strip_nu[2] * es};
+    ok = ok && encode_tensor_map(&vel->m[15], P.sa1[2], es, 4, dzs, szs, ab4);
+    ok = ok && encode_tensor_map(&vel->m[16], P.sb1[2], es, 4, dzs, szs, ab4);
+    ok = ok && encode_tensor_map(&prs->m[15], P.sa2[2], es, 4, dzs, szs, ab4);
+    ok = ok && encode_tensor_map(&prs->m[16], P.sb2[2], es, 4, dzs, szs, ab4);
   }
   if (!ok) {
     *why = "cuTensorMapEncodeTiled rejected a 3D map (or the driver entry point is missing)";
@@ -1287,14 +1336,17 @@ cudaError_t launch_pipe3d_batched(bool vel, bool cross, bool ps, int n_relax, co
 cudaError_t launch_pipe3d(bool vel, const StepParams &P, int grid, const PipeMaps &T, cudaStream_t st, int layout) {
   const bool ps = layout == kLayoutRegisters ? false : psi_staged(vel, P);
   const Region3 R = region3_of(P, grid, ps);
+  if (P.map_kind == 0) return launch_pipe3d_float(vel, P, &R, grid, T, st);
   if (P.g11h != 0.f)
-    return vel ? pipe3_dispatch<true, true, false>(P, R, grid, T, st)
-               : pipe3_dispatch<false, true, false>(P, R, grid, T, st);
+    return vel ? pipe3_dispatch<true, true, false, bf16>(P, R, grid, T, st)
+               : pipe3_dispatch<false, true, false, bf16>(P, R, grid, T, st);
   if (vel)
-    return ps ? pipe3_dispatch<true, false, true>(P, R, grid, T, st)
-              : pipe3_dispatch<true, false, false>(P, R, grid, T, st);
-  return ps ? pipe3_dispatch<false, false, true>(P, R, grid, T, st)
-            : pipe3_dispatch<false, false, false>(P, R, grid, T, st);
+    return ps ? pipe3_dispatch<true, false, true, bf16>(P, R, grid, T, st)
+              : pipe3_dispatch<true, false, false, bf16>(P, R, grid, T, st);
+  return ps ? pipe3_dispatch<false, false, true, bf16>(P, R, grid, T, st)
+            : pipe3_dispatch<false, false, false, bf16>(P, R, grid, T, st);
 }
+
+#endif  // FW2_PIPE3D_FLOAT
 
 }  // namespace fw2

@@ -113,3 +113,25 @@ def test_uint16_index_takes_the_pipelined_path_while_its_tables_fit(fw2, levels,
         sim.close()
     for n, want in out["tile"].items():
         np.testing.assert_array_equal(out["auto"][n], want, err_msg=n)
+
+
+@pytest.mark.parametrize("n,N,nl,pml,taps", [
+    ((300, 70, 45), 3, "westervelt", (6, 2), False), ((300, 70, 45), 3, "literal", (6, 2), True),
+    ((300, 60, 20), 0, "off", (0, 0), True), ((200, 45, 30), 2, "pressure", (5, 2), True),
+    ((100, 40, 20), 2, "literal", (6, 2), False), ((200, 20, 17), 3, "off", (3, 1), False),
+    ((300, 600, 20), 1, "off", (6, 2), False)])
+def test_3d_float_maps_on_the_pipelined_path_equal_tile_kernels_bitwise(fw2, n, N, nl, pml, taps):
+    """Float maps staged by the 3D pipeline: interior and edge units, one x
+    tile reaching both strips, strips read per cell (5 + 2 cells), few planes,
+    more items than blocks, the cross taps and the literal system's K."""
+    from tests.test_gpu_parity import _pipe_vs_tile, small_3d
+    prob = small_3d(n=n, N=max(N, 1), nl=nl, steps=12, pml=pml)
+    if N == 0:
+        prob.nrelax = 0
+        prob.kappa1 = prob.kappa2 = prob.d1 = prob.alpha1 = prob.d2 = prob.alpha2 = None
+    prob.sensors = synth.random_sensors(n, 25, 4, np.random.default_rng(1))
+    prob.sources = [synth.Source("p", np.arange(60, dtype=np.int64) * 11, np.zeros(60, np.int32),
+                                 prob.sources[0].signal)]
+    if taps:
+        prob.taps = tuple(fw2.fw2_taps_time_space(0.35, 3))
+    _pipe_vs_tile(fw2, prob, 12, maps="f32", state=synth.random_state(prob, seed=21))
