@@ -61,6 +61,14 @@ __device__ __forceinline__ float mom_factor(float Ka, float Kb, float pa, float 
   return fmaf(0.5f * (qdiv(1.f, Ka) + qdiv(1.f, Kb)), 0.5f * (pa + pb), 1.f);
 }
 
+// Two cells at a time (packed float instructions, one issue slot for both):
+// each half rounds like the scalar operation.
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, dup2(-1.f), a); }
+
 // The velocity update v - b S (Eq. general5, b = 2 dt / (rho_a + rho_b)),
 // and with the literal system's momentum factor f, v - b (S / f).  One fused
 // multiply-add each, written out so that every kernel of the half step

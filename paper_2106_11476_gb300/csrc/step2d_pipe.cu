@@ -327,13 +327,9 @@ __device__ __forceinline__ void vel_derivs2(const StepParams &P, const float *sp
   float2 col[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) col[m] = sld2(sp + (sy - 3 + m) * kCW + lx + 4);
+  Dy = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    float d = 0.f;
-#pragma unroll
-    for (int m = 1; m <= 4; ++m) d = fmaf(P.gh[m - 1], el2(col[3 + m], e) - el2(col[4 - m], e), d);
-    el2(Dy, e) = d;
-  }
+  for (int m = 1; m <= 4; ++m) Dy = fma2(dup2(P.gh[m - 1]), sub2(col[3 + m], col[4 - m]), Dy);
   if (P.g11h != 0.f) {
     const Win10 up = win10(sp + (sy + 1) * kCW, lx), dn = win10(sp + (sy - 1) * kCW, lx);
 #pragma unroll
@@ -358,13 +354,9 @@ __device__ __forceinline__ void prs_derivs2(const StepParams &P, const float *sv
   float2 col[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) col[m] = sld2(svy + (ly + m) * kCW + lx + 4);
+  Dy = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    float d = 0.f;
-#pragma unroll
-    for (int m = 1; m <= 4; ++m) d = fmaf(P.gh[m - 1], el2(col[4 + m - 1], e) - el2(col[4 - m], e), d);
-    el2(Dy, e) = d;
-  }
+  for (int m = 1; m <= 4; ++m) Dy = fma2(dup2(P.gh[m - 1]), sub2(col[4 + m - 1], col[4 - m]), Dy);
   if (P.g11h != 0.f) {
     const Win10 up = win10(svx + (ly + 2) * kCW, lx), dn = win10(svx + ly * kCW, lx);
     const Win10 y0w = win10(svy + (ly + 4) * kCW, lx), y1w = win10(svy + (ly + 3) * kCW, lx);
@@ -652,19 +644,15 @@ __device__ __forceinline__ void vel_compute(const StepParams &P, const float *ta
     }
   }
   float2 vx = sld2(own), vy = sld2(own + kArr);
-  float2 Sx = make_float2(Dx.x * k1.x, Dx.y * k1.y);
-  float2 Sy = make_float2(Dy.x * k1.x, Dy.y * k1.y);
+  const float2 wn = dup2(P.w_new), wo = dup2(P.w_old);
+  float2 Sx = mul2(Dx, k1), Sy = mul2(Dy, k1);
 #pragma unroll
   for (int nu = 0; nu < N; ++nu) {
     const float2 px = sld2(own + (2 + nu) * kArr), py = sld2(own + (2 + N + nu) * kArr);
-    float2 nx_, ny_;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      el2(nx_, e) = fmaf(el2(BX[nu], e), el2(px, e), el2(AX[nu], e) * el2(Dx, e));
-      el2(ny_, e) = fmaf(el2(BY[nu], e), el2(py, e), el2(AY[nu], e) * el2(Dy, e));
-      el2(Sx, e) += fmaf(P.w_new, el2(nx_, e), P.w_old * el2(px, e));
-      el2(Sy, e) += fmaf(P.w_new, el2(ny_, e), P.w_old * el2(py, e));
-    }
+    const float2 nx_ = fma2(BX[nu], px, mul2(AX[nu], Dx)), ny_ = fma2(BY[nu], py, mul2(AY[nu], Dy));
+    const float2 tx = fma2(wn, nx_, mul2(wo, px)), ty = fma2(wn, ny_, mul2(wo, py));
+    Sx = add2(Sx, tx);
+    Sy = add2(Sy, ty);
     put2<Maps, EDGE>(own, 2 + nu, P.psi1[0], nu * Sn + c, nx_, i0, P.nx);
     put2<Maps, EDGE>(own, 2 + N + nu, P.psi1[1], nu * Sn + c, ny_, i0, P.nx);
   }
@@ -739,19 +727,15 @@ __device__ __forceinline__ void prs_compute(const StepParams &P, const float *ta
     }
   }
   float2 p = sld2(own);
-  float2 Sx = make_float2(Dx.x * k2.x, Dx.y * k2.y);
-  float2 Sy = make_float2(Dy.x * k2.x, Dy.y * k2.y);
+  const float2 wn = dup2(P.w_new), wo = dup2(P.w_old);
+  float2 Sx = mul2(Dx, k2), Sy = mul2(Dy, k2);
 #pragma unroll
   for (int nu = 0; nu < N; ++nu) {
     const float2 px = sld2(own + (1 + nu) * kArr), py = sld2(own + (1 + N + nu) * kArr);
-    float2 nx_, ny_;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      el2(nx_, e) = fmaf(el2(BX[nu], e), el2(px, e), el2(AX[nu], e) * el2(Dx, e));
-      el2(ny_, e) = fmaf(el2(BY[nu], e), el2(py, e), el2(AY[nu], e) * el2(Dy, e));
-      el2(Sx, e) += fmaf(P.w_new, el2(nx_, e), P.w_old * el2(px, e));
-      el2(Sy, e) += fmaf(P.w_new, el2(ny_, e), P.w_old * el2(py, e));
-    }
+    const float2 nx_ = fma2(BX[nu], px, mul2(AX[nu], Dx)), ny_ = fma2(BY[nu], py, mul2(AY[nu], Dy));
+    const float2 tx = fma2(wn, nx_, mul2(wo, px)), ty = fma2(wn, ny_, mul2(wo, py));
+    Sx = add2(Sx, tx);
+    Sy = add2(Sy, ty);
     put2<Maps, EDGE>(own, 1 + nu, P.psi2[0], nu * Sn + c, nx_, i0, P.nx);
     put2<Maps, EDGE>(own, 1 + N + nu, P.psi2[1], nu * Sn + c, ny_, i0, P.nx);
   }

@@ -531,12 +531,8 @@ __device__ __forceinline__ void relax3(const StepParams &P, float *const *psi, l
                                        const float2 (&D)[3], float2 (&S)[3]) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    float2 n;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      el2(n, e) = fmaf(el2(B[a], e), el2(q[a], e), el2(A[a], e) * el2(D[a], e));
-      el2(S[a], e) += fmaf(P.w_new, el2(n, e), P.w_old * el2(q[a], e));
-    }
+    float2 n = fma2(B[a], q[a], mul2(A[a], D[a]));
+    S[a] = add2(S[a], fma2(dup2(P.w_new), n, mul2(dup2(P.w_old), q[a])));
     if (edge) n = mask_pad2(n, i0, P.nx);
     st_state2(psi[a], o, n);
   }
@@ -573,25 +569,17 @@ __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 
     float2 col[8];
 #pragma unroll
     for (int m = 0; m < 8; ++m) col[m] = sld2(sp + (sy - 3 + m) * kCW + lx + 4);
+D[1] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      float d = 0.f;
-#pragma unroll
-      for (int m = 1; m <= 4; ++m) d = fmaf(P.gh[m - 1], el2(col[3 + m], e) - el2(col[4 - m], e), d);
-      el2(D[1], e) = d;
-    }
+    for (int m = 1; m <= 4; ++m) D[1] = fma2(dup2(P.gh[m - 1]), sub2(col[3 + m], col[4 - m]), D[1]);
   }
   {
     float2 zc[8];
 #pragma unroll
     for (int m = 0; m < 8; ++m) zc[m] = sld2(ring + slot_after(s0, m) * kPl + sy * kCW + lx + 4);
+D[2] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      float d = 0.f;
-#pragma unroll
-      for (int m = 1; m <= 4; ++m) d = fmaf(P.gh[m - 1], el2(zc[3 + m], e) - el2(zc[4 - m], e), d);
-      el2(D[2], e) = d;
-    }
+    for (int m = 1; m <= 4; ++m) D[2] = fma2(dup2(P.gh[m - 1]), sub2(zc[3 + m], zc[4 - m]), D[2]);
   }
   if (CROSS) {
     // cross taps (Sec. 3.1) over both transverse axes, in the order of the
@@ -616,9 +604,7 @@ __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 
   float2 v0 = sld2(st + S::oV + o), v1 = sld2(st + S::oV + kArr + o), v2 = sld2(st + S::oV + 2 * kArr + o);
   float2 Sd[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int e = 0; e < 2; ++e) el2(Sd[a], e) = el2(D[a], e) * el2(k1, e);
+  for (int a = 0; a < 3; ++a) Sd[a] = mul2(D[a], k1);
   const int xside = EDGE ? R.xs_side(x0) : -1;
   const bool ys = EDGE && R.ys_row(y0) != INT_MIN, zs = EDGE && R.zs_plane(k) >= 0;
   // coefficients of every mechanism and axis first, C-PML strips included,
@@ -715,13 +701,9 @@ __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 
     for (int m = 0; m < 8; ++m)
       col[m] = CROSS ? sld2(suby + sub_slot(k) * S::kYPlane + (ly + m) * kCW + lx + 4)
                      : sld2(st + S::oVy + (ly + m) * kTX + lx);
+D[1] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      float d = 0.f;
-#pragma unroll
-      for (int m = 1; m <= 4; ++m) d = fmaf(P.gh[m - 1], el2(col[4 + m - 1], e) - el2(col[4 - m], e), d);
-      el2(D[1], e) = d;
-    }
+    for (int m = 1; m <= 4; ++m) D[1] = fma2(dup2(P.gh[m - 1]), sub2(col[4 + m - 1], col[4 - m]), D[1]);
   }
   {
     // v_z planes k-4 .. k+3 of the ring
@@ -730,13 +712,9 @@ __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 
     for (int m = 0; m < 8; ++m)
       zc[m] = CROSS ? sld2(ring + slot_after(s0, m) * kPl + (ly + 1) * kCW + lx + 4)
                     : sld2(ring + slot_after(s0, m) * kPl + o);
+D[2] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      float d = 0.f;
-#pragma unroll
-      for (int m = 1; m <= 4; ++m) d = fmaf(P.gh[m - 1], el2(zc[4 + m - 1], e) - el2(zc[4 - m], e), d);
-      el2(D[2], e) = d;
-    }
+    for (int m = 1; m <= 4; ++m) D[2] = fma2(dup2(P.gh[m - 1]), sub2(zc[4 + m - 1], zc[4 - m]), D[2]);
   }
   if (CROSS) {
     // cross taps (Sec. 3.1) at the centres, in the order of the tile
@@ -780,9 +758,7 @@ __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 
   float2 p = sld2(st + S::oP + o);
   float2 Sd[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int e = 0; e < 2; ++e) el2(Sd[a], e) = el2(D[a], e) * el2(k2, e);
+  for (int a = 0; a < 3; ++a) Sd[a] = mul2(D[a], k2);
   const int xside = EDGE ? R.xs_side(x0) : -1;
   const bool ys = EDGE && R.ys_row(y0) != INT_MIN, zs = EDGE && R.zs_plane(k) >= 0;
   // coefficients of every mechanism and axis first, C-PML strips included,
