@@ -1,25 +1,25 @@
 // Pipelined persistent 2D half steps (sm_103a); the arithmetic of the tile
 // kernels (tile2d.cuh) cell for cell, so the results are bitwise the same;
-// one launch per half step, one block of 512 threads per SM.
+// one block per SM, many steps per launch (steps2d_kernel).
 //
 // The grid is walked in half tiles of 128 x 8 cells through a ring of two to
 // four shared-memory stages (as many as fit).  For a coming half tile one
 // thread issues tiled TMA tensor copies into a free stage, one box per array:
-// the stencil operand with its halo, the density tile (or the uint8 tissue
-// index), every streamed array, the N mechanisms of a memory variable or of a
+// the stencil operand with its halo, the density tile (or the tissue index),
+// every streamed array, the N mechanisms of a memory variable or of a
 // relaxation map in one 3D box.  They complete on the stage's mbarrier while
-// all threads compute the current half tile from another stage, two cells
-// each, so up to ~190 KB stay in flight per SM without registers or load
-// instructions of the computing threads.  With float maps the updated arrays
-// are written back into the stage and leave for HBM as TMA tensor stores;
-// with the index form every thread stores its own results.
+// the computing threads work on the current half tile in another stage, two
+// cells each, so up to ~190 KB stay in flight per SM without registers or load
+// instructions of the computing threads.  The updated arrays are written back
+// into the stage and leave for HBM as TMA tensor stores.
 //
 // Boundaries: the copies read zero outside the grid (the zero-outside rule of
 // the operand halo); half tiles at the edge of the grid or in a C-PML strip
 // (edge half tiles) also clamp the density tile to the last cell, take the
 // C-PML coefficients of each axis from its strip, and store nothing outside
 // the grid (zeros in the row padding).  Periodic grids take the tile kernels.
-// Dense float maps and the tissue-index form take this path.
+// Every storage takes this path, the uint16 tissue index while its tables fit
+// in shared memory.
 #include <numeric>
 #include <type_traits>
 
@@ -165,8 +165,8 @@ __host__ __device__ constexpr unsigned stage_bytes(bool nl, bool nl_vel) {
   }
 }
 
-// The tensor copies of one half tile into a stage, in two parts (one thread;
-// the first announces the stage's bytes on the stage's mbarrier).  The first
+// The tensor copies of one half tile into a stage, in two parts (one thread,
+// which also announces the stage's bytes on the stage's mbarrier).  The first
 // part holds what only this half tile's own block writes (the updated arrays)
 // and the maps; the second the stencil operand, which the neighbouring half
 // tiles of the previous half step wrote.  Boxes may reach outside the grid:
@@ -175,7 +175,6 @@ template <int N, typename Maps, bool VEL>
 __device__ __forceinline__ void issue_own(const StepParams &P, const PipeMaps &T, float *st, uint64_t *bar, int x0,
                                           int y0) {
   fence_proxy_async_smem();
-  mbar_arrive_expect_tx(bar, stage_bytes<N, Maps, VEL>(P.nl != 0, P.nl_vel != 0));
   if (VEL) {
     using S = VelStage<N, Maps>;
     constexpr int kMf = floats_of<typename Form<Maps>::MT>(kArr);  // floats of one map array
@@ -231,6 +230,7 @@ __device__ __forceinline__ void issue_operand(const PipeMaps &T, float *st, uint
 template <int N, typename Maps, bool VEL>
 __device__ __forceinline__ void issue_stage(const StepParams &P, const PipeMaps &T, float *st, uint64_t *bar,
                                             int x0, int y0) {
+  mbar_arrive_expect_tx(bar, stage_bytes<N, Maps, VEL>(P.nl != 0, P.nl_vel != 0));
   issue_own<N, Maps, VEL>(P, T, st, bar, x0, y0);
   issue_operand<N, Maps, VEL>(T, st, bar, x0, y0);
 }
@@ -267,6 +267,7 @@ __device__ __forceinline__ void store_stage(const PipeMaps &T, const float *st, 
 // operations of the tile path in the same order, so results are bitwise the
 // same.
 constexpr int kThreads = 512;
+constexpr int kStepThreads = kThreads + 32;  // and the warp that copies and stores (steps2d_kernel)
 
 __device__ __forceinline__ float2 sld2(const float *s) { return *reinterpret_cast<const float2 *>(s); }
 __device__ __forceinline__ void st_state2(float *p, long long i, float2 v) {
@@ -777,8 +778,6 @@ struct StepRing {
   static constexpr int kTab = kWideIdx<Maps> ? kTotal - 2 * kStage : Maps::kSmemFloats;
   static constexpr int kFit = (kTotal - kTab) / kStage;
   static constexpr int kStages = kFit > 4 ? 4 : kFit;
-  static constexpr int kLag = kStages >= 4 ? 1 : 0;  // as Ring
-  static constexpr int kAhead = kStages - 1 - kLag;
   static constexpr size_t kBytes = sizeof(float) * ((size_t)kStages * kStage + kTab) + 128;
   static_assert(kStages >= 2, "two stages must fit in shared memory");
   static_assert(kBytes + 1024 <= 227 * 1024, "stages and table leave 1 KB for static shared memory");
@@ -813,11 +812,12 @@ __device__ __forceinline__ void mark_sources(const StepIO &io, const Region &R, 
   }
 }
 
-// Add the sources of a half tile to its updated arrays in the stage (every
-// thread, after the results of all threads are there): the entries of a
-// target summed in their order, then added, as inject_kernel does.
+// Add the sources of a half tile to its updated arrays in the stage (one
+// warp, once every result is there): the entries of a target summed in their
+// order, then added, as inject_kernel does.  Four targets a lane at a time:
+// each is a chain of loads.
 template <int N, typename Maps, bool VEL>
-__device__ __forceinline__ void inject_unit(const StepIO &io, int u, long long n, float *st, int tid) {
+__device__ __forceinline__ void inject_unit(const StepIO &io, int u, long long n, float *st, int lane) {
   const float *row = io.signal + n * io.sig_cols;
   float *ss = VEL ? st + VelStage<N, Maps>::kP + VelStage<N, Maps>::kR
                   : st + PrsStage<N, Maps>::kX + PrsStage<N, Maps>::kY;
@@ -825,11 +825,25 @@ __device__ __forceinline__ void inject_unit(const StepIO &io, int u, long long n
   for (int a = 0; a < (VEL ? 2 : 1); ++a) {
     const UnitSource &src = io.src[VEL ? 1 + a : 0];
     if (!src.unit) continue;
-    const int e = __ldg(src.unit + u + 1);
-    for (int t = __ldg(src.unit + u) + tid; t < e; t += kThreads) {
-      float v = 0.f;
-      for (int c = src.off[t]; c < src.off[t + 1]; ++c) v += __ldg(row + src.col[c]);
-      ss[a * kArr + src.pos[t]] += v;
+    const int t1 = __ldg(src.unit + u + 1);
+    for (int t0 = __ldg(src.unit + u) + lane; t0 < t1; t0 += 128) {
+      int b[4], e[4], pos[4];
+      float v[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int t = t0 + 32 * m;
+        const bool in = t < t1;
+        b[m] = in ? __ldg(src.off + t) : 0;
+        e[m] = in ? __ldg(src.off + t + 1) : 0;
+        pos[m] = in ? __ldg(src.pos + t) : 0;
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) v[m] = b[m] < e[m] ? 0.f + __ldg(row + __ldg(src.col + b[m])) : 0.f;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        for (int c = b[m] + 1; c < e[m]; ++c) v[m] += __ldg(row + __ldg(src.col + c));
+        if (t0 + 32 * m < t1) ss[a * kArr + pos[m]] += v[m];
+      }
     }
   }
 }
@@ -855,231 +869,228 @@ __device__ __forceinline__ void record_row(const StepIO &io, const float *p, lon
 
 // Phases ph0 .. ph1 - 1 of the time loop in one launch (phase 2n: velocity
 // half step of step n with its v sources, 2n + 1: pressure half step with its
-// p sources; the recording of step n runs in phase 2n + 2).  Block (32, 16),
-// one per SM; more than one phase needs a cooperative launch, since the
-// blocks wait for one another between phases.
+// p sources; the recording of step n runs in phase 2n + 2).  Block (32, 17),
+// one per SM: sixteen warps compute, the last one issues the copies and
+// stores and adds the sources.  More than one phase needs a cooperative launch, since the blocks
+// wait for one another between phases.
 //
-// What bounds it: HBM on grids beyond L2 (4096^2, N = 4: 690 us a step, 0.88
-// of the copy bandwidth on the step's bytes), the latency chain of a phase
+// What bounds it: HBM on grids beyond L2 (4096^2, N = 4: 655 us a step,
+// 0.91 of the copy bandwidth on the step's bytes), the latency chain of a phase
 // (operand copy, compute, store, grid barrier: about 5 us) on small ones.
 // Four launches per step (two half steps, sources, recording) added to every
 // one of them a start and a drain and left the SMs without copies in flight
 // meanwhile; here the next phase's first half tiles are copied (all but the
 // operand) while the barrier is under way, and sources and recording need no
-// launch of their own.  A step of 250 x 186 (N = 2) took 21 us and takes 11,
-// 512^2 (N = 4) 30 and 19.5, 1501 x 1237 111 and 98.  The velocity phases walk
+// launch of their own.  A step of 250 x 186 (N = 2) took 21 us and takes 9.8,
+// 512^2 (N = 4) 30 and 17, 1501 x 1237 111 and 87.  The velocity phases walk
 // the half tiles forwards and the pressure phases backwards, so each starts on
 // the rows whose operand the previous one left in L2 (0.8 % at 1501 x 1237).
+//
+// A stage goes round full -> computed -> stored -> refilled.  The computing
+// warps wait for "full" and announce "computed" each on its own, so that a
+// warp starts on the next stage while others are still busy with the last one
+// and nobody waits for a store to leave; one barrier per half tile for all
+// threads, with the copies issued by one of the computing threads, took 19
+// us a step at 512^2 (17 now), 82 at 2048 x 1024 of the uint8 index form (74),
+// 681 at 4096^2 (655).
 template <int N, typename Maps>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kStepThreads, 1)
     steps2d_kernel(const StepParams P, const Region R, const __grid_constant__ PipeMaps TV,
                    const __grid_constant__ PipeMaps TP, const StepIO io, const long long ph0, const long long ph1) {
   using G = StepRing<N, Maps>;
   constexpr int kS = G::kStages, kStage = G::kStage;
   extern __shared__ __align__(128) float smem_raw[];
-  __shared__ __align__(8) uint64_t bar[kS];
-  __shared__ int ok[kS];  // per stage: thread 0 never rewrites a flag a thread has yet to read
-  __shared__ int synced;
+  __shared__ __align__(8) uint64_t full[kS], done[kS];
+  __shared__ int blocked;
   __shared__ SourceBits sources;
   // TMA destinations need 128-byte alignment: round the base up (the launch
   // adds 128 bytes of slack)
   float *smem = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   float *tab = smem + kS * kStage;
   const int tid = threadIdx.y * 32 + threadIdx.x;
-  stage_table<N, Maps>(P, tab, tid);  // made visible by the barrier below
-  GridBarrier gb;
+  if (tid < kThreads) stage_table<N, Maps>(P, tab, tid);  // made visible by the barrier below
   if (tid == 0) {
-    for (int q = 0; q < kS; ++q) mbar_init(&bar[q], 1);
+    for (int q = 0; q < kS; ++q) {
+      mbar_init(&full[q], 1);
+      mbar_init(&done[q], kThreads / 32);
+    }
     fence_mbarrier_init();
-    gb.init(io.sync);
     // after a wait that gave up the state is incomplete: nothing runs until
     // the status is cleared
-    synced = ph1 - ph0 > 1 ? (status_of(P.status) == 0) : 1;
+    blocked = ph1 - ph0 > 1 && status_of(P.status) != 0;
   }
-  __syncthreads();
-  if (!synced) return;
   // this block's half tiles in every phase (at least one: grid <= half tiles)
   const int grid = (int)gridDim.x;
   const int per = R.rounds(blockIdx.x, grid);
   const int last_slot = R.slot(per - 1, blockIdx.x, grid);
-  mark_sources(io, R, per, sources, tid);  // made visible by the barrier of the first half tile
-  unsigned phase = 0;     // bit q: parity of the next completion of stage q
-  unsigned pending = 0;   // bit q: copies issued into stage q, not consumed
-  unsigned deferred = 0;  // bit q: the operand copy of stage q waits for the grid barrier
-  int ahead = 0;          // jobs issued and not consumed
-  // the half tile of each stage's job: origin and round
-  int jx[kS], jy[kS], jr[kS];
-  auto at = [&](const int (&a)[kS], int q) {
-    int v = a[0];
-#pragma unroll
-    for (int m = 1; m < kS; ++m) v = q == m ? a[m] : v;
-    return v;
+  mark_sources(io, R, per, sources, tid);
+  __syncthreads();
+  if (blocked) return;
+  // Walk over the jobs (phase, half tile): rounds upwards in velocity phases,
+  // downwards in pressure phases; a job's stage is its number modulo kS.
+  struct Walk {
+    long long ph;
+    int round, slot, x, y;  // origin of the half tile
+    int stage;
+    unsigned parity;        // of the stage's barriers for this job
   };
-  // the next job to issue: phase, round, slot, origin (worked out before it is
-  // needed: thread 0 issues between two barriers) and stage
-  long long iph = ph0;
-  int is = 0, ir = (ph0 & 1) ? per - 1 : 0, islot = (ph0 & 1) ? last_slot : (int)blockIdx.x, ix, iy;
-  R.half_origin(ir * grid + islot, ix, iy);
-  auto advance = [&] {
-    if (iph & 1) {
-      if (ir == 0) {
-        ++iph;  // the velocity phase starts where this one ended
-      } else {
-        --ir;
-        islot -= R.rot;
-        if (islot < 0) islot += grid;
-      }
-    } else if (ir == per - 1) {
-      ++iph;
+  auto start = [&] {
+    Walk w{ph0, (ph0 & 1) ? per - 1 : 0, (ph0 & 1) ? last_slot : (int)blockIdx.x, 0, 0, 0, 0};
+    R.half_origin(w.round * grid + w.slot, w.x, w.y);
+    return w;
+  };
+  auto last_of_phase = [&](const Walk &w) { return w.round == ((w.ph & 1) ? 0 : per - 1); };
+  auto next = [&](Walk &w) {
+    if (last_of_phase(w)) {
+      ++w.ph;  // the next phase starts where this one ended
     } else {
-      ++ir;
-      islot += R.rot;
-      if (islot >= grid) islot -= grid;
+      const bool down = w.ph & 1;
+      w.round += down ? -1 : 1;
+      w.slot += down ? -R.rot : R.rot;
+      if (w.slot < 0) w.slot += grid;
+      if (w.slot >= grid) w.slot -= grid;
+      R.half_origin(w.round * grid + w.slot, w.x, w.y);
     }
-    R.half_origin(ir * grid + islot, ix, iy);
+    if (++w.stage == kS) {
+      w.stage = 0;
+      w.parity ^= 1u;
+    }
   };
-  auto issue_next = [&](long long ph) {  // every thread keeps the bookkeeping, thread 0 issues
-    if (tid < 32) {
-      if (tid == 0) {
-        float *st = smem + is * kStage;
-        if (iph & 1) issue_own<N, Maps, false>(P, TP, st, &bar[is], ix, iy);
-        else issue_own<N, Maps, true>(P, TV, st, &bar[is], ix, iy);
-        if (iph == ph) {
-          if (iph & 1) issue_operand<N, Maps, false>(TP, st, &bar[is], ix, iy);
-          else issue_operand<N, Maps, true>(TV, st, &bar[is], ix, iy);
+
+  if (tid >= kThreads) {
+    // ---------------------------------------------------- copies and stores
+    const int lane = tid - kThreads;
+    GridBarrier gb;
+    gb.init(io.sync);
+    Walk wi = start(), ws = wi;  // next job to issue, next job to store
+    int ahead = 0;               // jobs issued and not stored
+    Walk wd = wi;                // first job whose operand waits for the grid barrier
+    int held = 0;                // and their number
+    auto operand = [&](const Walk &w) {  // lane 0: the job may start once these have landed
+      float *st = smem + w.stage * kStage;
+      uint64_t *bar = &full[w.stage];
+      if (w.ph & 1) {
+        mbar_arrive_expect_tx(bar, stage_bytes<N, Maps, false>(P.nl != 0, P.nl_vel != 0));
+        issue_operand<N, Maps, false>(TP, st, bar, w.x, w.y);
+      } else {
+        mbar_arrive_expect_tx(bar, stage_bytes<N, Maps, true>(P.nl != 0, P.nl_vel != 0));
+        issue_operand<N, Maps, true>(TV, st, bar, w.x, w.y);
+      }
+    };
+    // fill free stages, at most one phase ahead of the phase `ph` under way
+    // (what a later phase updates is still being written)
+    auto fill = [&](long long ph) {
+      while (ahead < kS && wi.ph < ph1 && wi.ph <= ph + 1) {
+        if (lane == 0) {
+          float *st = smem + wi.stage * kStage;
+          uint64_t *bar = &full[wi.stage];
+          if (wi.ph & 1) issue_own<N, Maps, false>(P, TP, st, bar, wi.x, wi.y);
+          else issue_own<N, Maps, true>(P, TV, st, bar, wi.x, wi.y);
+          if (wi.ph == ph) operand(wi);
         }
+        if (wi.ph != ph && held++ == 0) wd = wi;
+        if (!R.interior(wi.x, wi.y)) {
+          if (wi.ph & 1) prefetch_strips2<N, 2, typename Maps::StripT>(P, wi.x, wi.y, lane);
+          else prefetch_strips2<N, 1, typename Maps::StripT>(P, wi.x, wi.y, lane);
+        }
+        ++ahead;
+        next(wi);
       }
-      if (!R.interior(ix, iy)) {
-        if (iph & 1) prefetch_strips2<N, 2, typename Maps::StripT>(P, ix, iy, tid);
-        else prefetch_strips2<N, 1, typename Maps::StripT>(P, ix, iy, tid);
+    };
+    auto release_held = [&] {
+      for (; held > 0; --held) {
+        if (lane == 0) operand(wd);
+        next(wd);
+      }
+    };
+    fill(ph0);
+    bool ok = true;
+#pragma unroll 1
+    while (true) {
+      ok = mbar_wait_bounded(&done[ws.stage], ws.parity);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      if ((ws.ph >> 1) < io.sig_steps && sources.get((int)(ws.ph & 1), ws.round)) {
+        float *st = smem + ws.stage * kStage;
+        const int u = ws.round * grid + ws.slot;
+        if (ws.ph & 1) inject_unit<N, Maps, false>(io, u, ws.ph >> 1, st, lane);
+        else inject_unit<N, Maps, true>(io, u, ws.ph >> 1, st, lane);
+        fence_proxy_async_smem();
+        __syncwarp();
+      }
+      if (lane == 0) {
+        if (ws.ph & 1) store_stage<N, Maps, false>(TP, smem + ws.stage * kStage, ws.x, ws.y);
+        else store_stage<N, Maps, true>(TV, smem + ws.stage * kStage, ws.x, ws.y);
+      }
+      --ahead;
+      const long long ph = ws.ph;
+      const bool last = last_of_phase(ws);
+      next(ws);
+      if (!last) {
+        if (lane == 0) bulk_wait_read<0>();
+        __syncwarp();
+        fill(ph);
+        continue;
+      }
+      if (ph + 1 == ph1) break;
+      if (lane == 0) {
+        bulk_wait_all();  // this block's results are in memory
+        fence_proxy_async_all();
+        gb.arrive();
+      }
+      __syncwarp();
+      // copies of the next phase's first half tiles while the others arrive
+      fill(ph);
+      if (lane == 0) {
+        ok = gb.wait(P.status);
+        fence_proxy_async_all();
+      }
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!ok) break;
+      release_held();
+      fill(ph + 1);
+    }
+    if (!ok) {
+      // a wait gave up: let this block's copies land (a stage whose operand
+      // was still held back gets it, so that its barrier can complete)
+      if (lane == 0) report_status(P.status, kStatusWaitTimeout);
+      release_held();
+      for (; ahead > 0; --ahead) {
+        mbar_wait_bounded(&full[ws.stage], ws.parity);
+        next(ws);
       }
     }
-    pending |= 1u << is;
-    if (iph != ph) deferred |= 1u << is;
-#pragma unroll
-    for (int q = 0; q < kS; ++q)
-      if (q == is) {
-        jx[q] = ix;
-        jy[q] = iy;
-        jr[q] = ir;
-      }
-    is = is + 1 == kS ? 0 : is + 1;
-    ++ahead;
-  };
-  auto issue_deferred = [&](long long ph) {  // thread 0, the operands of phase ph
-#pragma unroll
-    for (int q = 0; q < kS; ++q)
-      if ((deferred >> q) & 1u) {
-        if (ph & 1) issue_operand<N, Maps, false>(TP, smem + q * kStage, &bar[q], jx[q], jy[q]);
-        else issue_operand<N, Maps, true>(TV, smem + q * kStage, &bar[q], jx[q], jy[q]);
-      }
-  };
-  // a wait gave up: let this block's copies land (a stage whose operand was
-  // still held back gets it, so that its barrier can complete)
-  auto give_up = [&](long long ph, int s) {
-    if (tid != 0) return;
-    report_status(P.status, kStatusWaitTimeout);
-    issue_deferred(ph + 1);
-    for (int q = 0; q < kS; ++q)
-      if (q != s && ((pending >> q) & 1u)) mbar_wait_bounded(&bar[q], (phase >> q) & 1u);
-    bulk_wait_all();
-  };
-  // the first copies into every stage; a job may be issued up to one phase
-  // ahead (what a later phase updates is still being written)
-  while (ahead < kS && iph < ph1 && iph <= ph0 + 1) {
-    issue_next(ph0);
-    advance();
+    if (lane == 0) bulk_wait_all();
+    return;
   }
-  long long ph = ph0;
-  int i = 0, s = 0;
-  int xp = -1, yp = -1;  // previous half tile of this block in this phase
+
+  // ------------------------------------------------------------- compute ---
+  Walk w = start();
 #pragma unroll 1
   while (true) {
-    // One barrier per half tile: after the wait for stage s it also marks the
-    // previous half tile computed, so its results are sent and a freed stage
-    // is refilled right after it.
-    if (tid == 0) ok[s] = mbar_wait_bounded(&bar[s], (phase >> s) & 1u);
-    __syncthreads();
-    if (!ok[s]) {
-      give_up(ph, s);
+    if (!mbar_wait_bounded(&full[w.stage], w.parity)) {
+      if ((tid & 31) == 0) report_status(P.status, kStatusWaitTimeout);
       return;
     }
-    phase ^= 1u << s;
-    pending &= ~(1u << s);
-    --ahead;
-    const bool vel = (ph & 1) == 0;
-    const int sp = (s + kS - 1) % kS;  // the previous half tile's stage
-    if (tid == 0 && xp >= 0) {
-      if (vel) store_stage<N, Maps, true>(TV, smem + sp * kStage, xp, yp);
-      else store_stage<N, Maps, false>(TP, smem + sp * kStage, xp, yp);
-    }
-    const int x0 = at(jx, s), y0 = at(jy, s), round = at(jr, s);
-    const bool refill = ahead < G::kAhead && iph < ph1 && iph <= ph + 1;
-    if (refill) {
-      if (tid == 0) bulk_wait_read<G::kLag>();
-      issue_next(ph);
-      advance();
-    }
-    float *cur = smem + s * kStage;
-    if (R.interior(x0, y0)) {
-      if (vel) vel_compute<N, Maps, false>(P, tab, cur, x0, y0, tid);
-      else prs_compute<N, Maps, false>(P, tab, cur, x0, y0, tid);
+    const bool vel = (w.ph & 1) == 0;
+    const long long n = w.ph >> 1;
+    // the previous step's trace row, before this warp's first half tile of the
+    // velocity phase (the operand is there, so every block's p is complete)
+    if (vel && w.round == 0 && w.ph != ph0 && io.rec_groups > 0 && n - 1 < io.rec_steps) record_row(io, P.p, n - 1, tid);
+    float *cur = smem + w.stage * kStage;
+    if (R.interior(w.x, w.y)) {
+      if (vel) vel_compute<N, Maps, false>(P, tab, cur, w.x, w.y, tid);
+      else prs_compute<N, Maps, false>(P, tab, cur, w.x, w.y, tid);
     } else {
-      if (vel) vel_compute<N, Maps, true>(P, tab, cur, x0, y0, tid);
-      else prs_compute<N, Maps, true>(P, tab, cur, x0, y0, tid);
-    }
-    if ((ph >> 1) < io.sig_steps && sources.get((int)(ph & 1), round)) {
-      const int u = round * grid + R.slot(round, blockIdx.x, grid);
-      __syncthreads();
-      if (vel) inject_unit<N, Maps, true>(io, u, ph >> 1, cur, tid);
-      else inject_unit<N, Maps, false>(io, u, ph >> 1, cur, tid);
+      if (vel) vel_compute<N, Maps, true>(P, tab, cur, w.x, w.y, tid);
+      else prs_compute<N, Maps, true>(P, tab, cur, w.x, w.y, tid);
     }
     fence_proxy_async_smem();
-    xp = x0;
-    yp = y0;
-    s = s + 1 == kS ? 0 : s + 1;
-    if (++i < per) continue;
-    // ---- end of the phase
-    __syncthreads();
-    if (tid == 0) {
-      const int sl = (s + kS - 1) % kS;
-      if (vel) store_stage<N, Maps, true>(TV, smem + sl * kStage, xp, yp);
-      else store_stage<N, Maps, false>(TP, smem + sl * kStage, xp, yp);
-    }
-    if (ph + 1 == ph1) break;
-    if (tid == 0) {
-      bulk_wait_all();  // this block's results are in memory
-      fence_proxy_async_all();
-      gb.arrive();
-    }
-    // copies of the next phase's first half tiles, into every stage (none is
-    // being computed), while the other blocks arrive
-    while (ahead < kS && iph < ph1 && iph <= ph + 1) {
-      issue_next(ph);
-      advance();
-    }
-    if (tid == 0) {
-      synced = gb.wait(P.status);
-      fence_proxy_async_all();
-    }
-    __syncthreads();
-    if (!synced) {
-      give_up(ph, -1);
-      return;
-    }
-    ++ph;
-    if (tid == 0) issue_deferred(ph);
-    deferred = 0;
-    if (!(ph & 1) && io.rec_groups > 0 && (ph >> 1) - 1 < io.rec_steps) record_row(io, P.p, (ph >> 1) - 1, tid);
-    // jobs that were held back for being two phases ahead
-    while (ahead < kS && iph < ph1 && iph <= ph + 1) {
-      issue_next(ph);
-      advance();
-    }
-    i = 0;
-    xp = -1;
+    __syncwarp();
+    if ((tid & 31) == 0) mbar_arrive(&done[w.stage]);
+    if (last_of_phase(w) && w.ph + 1 == ph1) return;
+    next(w);
   }
-  if (tid == 0) bulk_wait_all();
 }
 
 // Batched half step over a unit table of several contexts (one group: same
@@ -1226,7 +1237,7 @@ cudaError_t steps_launch(const StepParams &P, const Region &R, int grid, const P
   constexpr size_t bytes = StepRing<N, Maps>::kBytes;
   cudaError_t e = cudaFuncSetAttribute(steps2d_kernel<N, Maps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
-  const dim3 block(32, kThreads / 32);
+  const dim3 block(32, kStepThreads / 32);
   if (ph1 - ph0 == 1) {
     steps2d_kernel<N, Maps><<<grid, block, bytes, st>>>(P, R, TV, TP, io, ph0, ph1);
     return cudaGetLastError();
