@@ -793,11 +793,12 @@ D[2] = make_float2(0.f, 0.f);
   st_state2(P.p, c, p);
 }
 
-// One half step.  Block (32, 16), one per SM; items blockIdx.x,
+// One half step of the register layout.  Block (32, 16), one per SM; items blockIdx.x,
 // blockIdx.x + gridDim.x, ...; within an item the units k0 .. k1-1 in order.
-template <int N, bool VEL, bool CROSS, bool PS, typename MT>
+template <int N, bool VEL, bool CROSS, typename MT>
 __global__ void __launch_bounds__(kThreads, 1)
     pipe3d_kernel(const StepParams P, const Region3 R, const __grid_constant__ PipeMaps T) {
+  constexpr bool PS = false;
   using G = Ring3<N, VEL, CROSS, PS, MT>;
   constexpr int kStage = G::kStage;
   extern __shared__ __align__(128) float smem_raw[];
@@ -840,7 +841,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 q);
   };
   Psi<N> qc, qn;
-  if (!PS) psi_of(x0, y0, k, qc);
+  psi_of(x0, y0, k, qc);
   int s = 0;
 #pragma unroll 1
   while (true) {
@@ -878,7 +879,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       pending |= 1u << q;
     }
-    if (!PS && more) psi_of(nx0, ny0, nk, qn);
+    if (more) psi_of(nx0, ny0, nk, qn);
     float *cur = smem + s * kStage;
     if (R.interior(x0, y0, k)) {
       if (VEL) vel3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, x0, y0, k, tid, qc);
@@ -898,14 +899,131 @@ __global__ void __launch_bounds__(kThreads, 1)
     it = nit;
     x0 = nx0; y0 = ny0; k0 = nk0; k1 = nk1; k = nk;
     s = q;
-    if (!PS) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+    for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int nu = 0; nu < N; ++nu) qc[a][nu] = qn[a][nu];
-    }
+      for (int nu = 0; nu < N; ++nu) qc[a][nu] = qn[a][nu];
   }
 }
+
+#ifndef FW2_PIPE3D_FLOAT  // float maps have no such layout
+// One half step of the layout that stages the memory variables, without a
+// barrier of the block.  Block (32, 17), one per SM: sixteen warps compute,
+// the last one issues the copies; items as in pipe3d_kernel.
+//
+// The computing warps wait for a stage ("full") and announce that they are
+// through with it ("done") each on its own, so a warp starts on the next unit
+// while others still work on the last one.  A unit's copies go out once every
+// warp is done with the unit before the previous one (whose stage and oldest
+// ring plane they take), the first ones of an item once the rings are free
+// altogether.  512^3, N = 3: velocity 2.93 to 2.76 ms, pressure 2.81 to 2.53
+// ms (301 x 222 x 190, mostly edge units: 0.458 to 0.425 and 0.452 to 0.396).
+// Seventeen warps leave 96 registers a thread: the register layout spills
+// there and loses more than it gains (0.418 to 0.490 ms at 301 x 222 x 190),
+// so it keeps pipe3d_kernel's barrier.  Without a warp of its own, the copies
+// issued by the last warp through with a unit, every layout was 5 to 20 %
+// slower than with the barrier.
+template <int N, bool VEL, typename MT>
+__global__ void __launch_bounds__(kThreads + 32, 1)
+    pipe3d_staged_kernel(const StepParams P, const Region3 R, const __grid_constant__ PipeMaps T) {
+  constexpr bool CROSS = false, PS = true;
+  using G = Ring3<N, VEL, CROSS, PS, MT>;
+  constexpr int kStage = G::kStage;
+  extern __shared__ __align__(128) float smem_raw[];
+  __shared__ __align__(8) uint64_t full[2], done[2];
+  float *smem = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+  float *ring = smem + 2 * kStage;
+  const int tid = threadIdx.y * 32 + threadIdx.x;
+  if (tid == 0) {
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&full[q], 1);
+      mbar_init(&done[q], kThreads / 32);
+    }
+    fence_mbarrier_init();
+  }
+  __syncthreads();
+  const long long n_items = R.items();
+  const long long grid = gridDim.x;
+  if (blockIdx.x >= n_items) return;
+  // a unit of this block: its item, plane and job number (stage and parity)
+  struct Unit {
+    long long it, slot;
+    int x0, y0, k0, k1, k;
+    unsigned job;
+    __device__ __forceinline__ int stage() const { return job & 1u; }
+    __device__ __forceinline__ unsigned parity() const { return (job >> 1) & 1u; }
+  };
+  Unit u{blockIdx.x, blockIdx.x, 0, 0, 0, 0, 0, 0};
+  R.item(u.it, u.x0, u.y0, u.k0, u.k1);
+  u.k = u.k0;
+  // the next plane of the item, or the first of the block's next item;
+  // false when there is none
+  auto advance = [&](Unit &v) {
+    ++v.job;
+    if (++v.k < v.k1) return true;
+    v.it += grid - v.slot;
+    v.slot += R.rot;
+    if (v.slot >= grid) v.slot -= grid;
+    v.it += v.slot;
+    if (v.it >= n_items) return false;
+    R.item(v.it, v.x0, v.y0, v.k0, v.k1);
+    v.k = v.k0;
+    return true;
+  };
+
+  if (tid >= kThreads) {
+    // ------------------------------------------------------------- copies
+    const int lane = tid - kThreads;
+    const bool nl = P.nl != 0, nlv = VEL && P.nl_vel != 0;
+    bool ok = true;
+    unsigned issued = 0;
+    do {
+      const bool fresh = u.k == u.k0;
+      // the job two before has the stage; a new item replaces every plane
+      if (u.job >= 2) ok = mbar_wait_bounded(&done[u.stage()], u.parity() ^ 1u);
+      if (ok && fresh && u.job >= 1) ok = mbar_wait_bounded(&done[u.stage() ^ 1], ((u.job - 1) >> 1) & 1u);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      if (lane == 0) {
+        const int k_hi = ring_first<VEL>(u.k) + 7;
+        issue3<N, VEL, CROSS, PS, MT>(T, R, smem + u.stage() * kStage, ring, nullptr, &full[u.stage()], u.x0, u.y0, u.k,
+                                      fresh ? k_hi - 7 : k_hi, k_hi, fresh ? u.k - 1 : u.k + 1, u.k + 1, nl, nlv);
+      }
+      ++issued;
+      if (!R.interior(u.x0, u.y0, u.k)) prefetch_strips<N, VEL ? 1 : 2, MT>(P, R, u.x0, u.y0, u.k, lane);
+    } while (advance(u));
+    if (!ok && lane == 0) report_status(P.status, kStatusWaitTimeout);
+    // every copy has landed before the block's shared memory goes
+    for (unsigned j = issued < 2 ? 0 : issued - 2; j < issued; ++j) mbar_wait_bounded(&full[j & 1u], (j >> 1) & 1u);
+    return;
+  }
+
+  // ------------------------------------------------------------- compute ---
+  const Psi<N> q{};  // the memory variables come with the stage
+#pragma unroll 1
+  while (true) {
+    if (!mbar_wait_bounded(&full[u.stage()], u.parity())) {
+      if ((tid & 31) == 0) report_status(P.status, kStatusWaitTimeout);
+      return;
+    }
+    Unit nu = u;
+    const bool more = advance(nu);
+    float *cur = smem + u.stage() * kStage;
+    if (R.interior(u.x0, u.y0, u.k)) {
+      if (VEL) vel3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, u.x0, u.y0, u.k, tid, q);
+      else prs3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, nullptr, u.x0, u.y0, u.k, tid, q);
+    } else {
+      if (VEL) vel3_compute<N, true, CROSS, PS, MT>(P, R, cur, ring, u.x0, u.y0, u.k, tid, q);
+      else prs3_compute<N, true, CROSS, PS, MT>(P, R, cur, ring, nullptr, u.x0, u.y0, u.k, tid, q);
+    }
+    __syncwarp();
+    if ((tid & 31) == 0) mbar_arrive(&done[u.stage()]);
+    if (!more) return;
+    u = nu;
+  }
+}
+
+#endif
 
 #ifndef FW2_PIPE3D_FLOAT
 // The same half step for several contexts in one launch (a batch of 3D
@@ -1078,11 +1196,23 @@ template <int N, bool VEL, bool CROSS, bool PS, typename MT>
 cudaError_t pipe3_launch(const StepParams &P, const Region3 &R, int grid, const PipeMaps &T, cudaStream_t st) {
   constexpr size_t bytes = Ring3<N, VEL, CROSS, PS, MT>::kBytes;
   static_assert(bytes + 64 <= 227 * 1024, "stages exceed shared memory");
-  cudaError_t e = cudaFuncSetAttribute(pipe3d_kernel<N, VEL, CROSS, PS, MT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  pipe3d_kernel<N, VEL, CROSS, PS, MT><<<grid, dim3(32, kThreads / 32), bytes, st>>>(P, R, T);
-  return cudaGetLastError();
+#ifndef FW2_PIPE3D_FLOAT
+  if constexpr (PS) {
+    cudaError_t e = cudaFuncSetAttribute(pipe3d_staged_kernel<N, VEL, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)bytes);
+    if (e != cudaSuccess) return e;
+    pipe3d_staged_kernel<N, VEL, MT><<<grid, dim3(32, kThreads / 32 + 1), bytes, st>>>(P, R, T);
+    return cudaGetLastError();
+  }
+#endif
+  if constexpr (!PS) {
+    cudaError_t e = cudaFuncSetAttribute(pipe3d_kernel<N, VEL, CROSS, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)bytes);
+    if (e != cudaSuccess) return e;
+    pipe3d_kernel<N, VEL, CROSS, MT><<<grid, dim3(32, kThreads / 32), bytes, st>>>(P, R, T);
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
 }
 
 template <bool VEL, bool CROSS, bool PS, typename MT>
