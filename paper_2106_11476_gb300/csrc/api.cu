@@ -1116,6 +1116,37 @@ fw2_status fw2_set_subdomain(fw2_ctx *c, const int64_t *global_n, const int64_t 
   return FW2_OK;
 }
 
+// `arrays` state arrays (npts_alloc apart, `rows` rows of nx values from
+// `dev`) to or from a dense caller buffer; synchronous.  Buffers in memory of
+// this device go through a kernel, everything else through the copy calls.
+static fw2_status copy_state(fw2_ctx *c, float *dev, long long rows, int arrays, float *buf, int32_t mem_space,
+                             bool out) {
+  cudaPointerAttributes at{};
+  int here = -1;
+  bool local = mem_space == FW2_MEM_DEVICE && cudaGetDevice(&here) == cudaSuccess &&
+               cudaPointerGetAttributes(&at, buf) == cudaSuccess &&
+               (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == here &&
+               reinterpret_cast<uintptr_t>(buf) % sizeof(float) == 0;
+  if (local) {
+    const long long dense = rows * c->nx;
+    CK(c, out ? launch_copy_rows(buf, c->nx, dense, dev, c->pitch, c->npts_alloc, c->nx, rows, arrays, c->stream)
+              : launch_copy_rows(dev, c->pitch, c->npts_alloc, buf, c->nx, dense, c->nx, rows, arrays, c->stream));
+    c->launches++;
+  } else {
+    (void)cudaGetLastError();
+    const size_t w = sizeof(float) * c->nx, dp = sizeof(float) * c->pitch;
+    const cudaMemcpyKind kind = mem_space == FW2_MEM_DEVICE ? cudaMemcpyDeviceToDevice
+                                : out ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
+    for (int m = 0; m < arrays; ++m) {
+      float *d = dev + (size_t)m * c->npts_alloc, *h = buf + (size_t)m * rows * c->nx;
+      if (out) CK(c, cudaMemcpy2DAsync(h, w, d, dp, w, (size_t)rows, kind, c->stream));
+      else CK(c, cudaMemcpy2DAsync(d, dp, h, w, w, (size_t)rows, kind, c->stream));
+    }
+  }
+  CK(c, cudaStreamSynchronize(c->stream));
+  return FW2_OK;
+}
+
 // Rows of a state array along the slowest axis (y rows in 2D, z planes in
 // 3D) to or from a dense buffer [n_rows][(ny)][nx]; synchronous.
 static fw2_status copy_rows(fw2_ctx *c, int32_t field, int64_t row0, int64_t n_rows, float *buf, int32_t mem_space,
@@ -1129,15 +1160,7 @@ static fw2_status copy_rows(fw2_ctx *c, int32_t field, int64_t row0, int64_t n_r
   if (n_rows == 0) return FW2_OK;
   float *f = field == FW2_FIELD_P ? c->p : c->v[field - FW2_FIELD_VX];
   const long long per_row = c->nd == 3 ? c->plane : c->pitch;
-  const size_t height = (size_t)n_rows * (c->nd == 3 ? c->ny : 1);
-  float *dev = f + row0 * per_row;
-  const size_t w = sizeof(float) * c->nx, dp = sizeof(float) * c->pitch;
-  const cudaMemcpyKind kind = out ? (mem_space == FW2_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost)
-                                  : (mem_space == FW2_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice);
-  if (out) CK(c, cudaMemcpy2DAsync(buf, w, dev, dp, w, height, kind, c->stream));
-  else CK(c, cudaMemcpy2DAsync(dev, dp, buf, w, w, height, kind, c->stream));
-  CK(c, cudaStreamSynchronize(c->stream));
-  return FW2_OK;
+  return copy_state(c, f + row0 * per_row, n_rows * (c->nd == 3 ? c->ny : 1), 1, buf, mem_space, out);
 }
 
 fw2_status fw2_get_rows(fw2_ctx *c, int32_t field, int64_t row0, int64_t n_rows, float *out, int32_t mem_space) {
@@ -1184,13 +1207,7 @@ fw2_status fw2_get_field(fw2_ctx *c, int32_t field, float *out, int32_t mem_spac
   int count;
   float *f = field_ptr(c, field, &count);
   if (!f) return fail(c, FW2_EINVAL, "field %d does not exist in this context", field);
-  const cudaMemcpyKind kind = mem_space == FW2_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  for (int m = 0; m < count; ++m) {
-    CK(c, cudaMemcpy2DAsync(out + (size_t)m * c->n_pts, sizeof(float) * c->nx, f + (size_t)m * c->npts_alloc,
-                            sizeof(float) * c->pitch, sizeof(float) * c->nx, (size_t)c->ny * c->nz, kind, c->stream));
-  }
-  CK(c, cudaStreamSynchronize(c->stream));
-  return FW2_OK;
+  return copy_state(c, f, (long long)c->ny * c->nz, count, out, mem_space, true);
 }
 
 fw2_status fw2_set_field(fw2_ctx *c, int32_t field, const float *in, int32_t mem_space) {
@@ -1198,13 +1215,7 @@ fw2_status fw2_set_field(fw2_ctx *c, int32_t field, const float *in, int32_t mem
   int count;
   float *f = field_ptr(c, field, &count);
   if (!f) return fail(c, FW2_EINVAL, "field %d does not exist in this context", field);
-  const cudaMemcpyKind kind = mem_space == FW2_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  for (int m = 0; m < count; ++m) {
-    CK(c, cudaMemcpy2DAsync(f + (size_t)m * c->npts_alloc, sizeof(float) * c->pitch, in + (size_t)m * c->n_pts,
-                            sizeof(float) * c->nx, sizeof(float) * c->nx, (size_t)c->ny * c->nz, kind, c->stream));
-  }
-  CK(c, cudaStreamSynchronize(c->stream));
-  return FW2_OK;
+  return copy_state(c, f, (long long)c->ny * c->nz, count, const_cast<float *>(in), mem_space, false);
 }
 
 fw2_status fw2_reset(fw2_ctx *c) {

@@ -65,6 +65,10 @@ cudaError_t launch_inject(float *field, const long long *tgt, const int *off, co
 // recording: out[g] = mean over e in [off[g], off[g+1]) of p[cell[e]]
 cudaError_t launch_record(const float *p, const long long *cell, const int *off, int n_groups,
                           float *out, cudaStream_t s);
+// `arrays` arrays of `rows` rows of nx floats between two layouts (row and
+// array strides in floats), device memory on both sides
+cudaError_t launch_copy_rows(float *dst, long long dst_row, long long dst_arr, const float *src, long long src_row,
+                             long long src_arr, int nx, long long rows, int arrays, cudaStream_t s);
 // field scan: max |x| over the cell layout (rows of nx valid values, pitch
 // apart), non-finite values reported as +inf; result in *out_bits (float bits)
 cudaError_t launch_absmax(const float *f, int nx, int pitch, long long rows,

@@ -135,3 +135,32 @@ def test_3d_float_maps_on_the_pipelined_path_equal_tile_kernels_bitwise(fw2, n, 
     if taps:
         prob.taps = tuple(fw2.fw2_taps_time_space(0.35, 3))
     _pipe_vs_tile(fw2, prob, 12, maps="f32", state=synth.random_state(prob, seed=21))
+
+
+@pytest.mark.parametrize("shape,offset", [((8, 8), 0), ((33, 9), 0), ((1024, 8), 0), ((1028, 11), 1), ((2051, 16), 0),
+                                          ((17, 9, 8), 0), ((64, 8, 10), 3)])
+def test_device_field_copies_round_trip(fw2, shape, offset):
+    """Fields to and from device buffers of any row alignment (rows of 4n and
+    odd lengths, longer than a segment, buffers off by `offset` floats) equal
+    the copies through host memory; what lies beside the buffer is untouched."""
+    import torch
+    prob = synth.homogeneous(shape, 1e-4, 2e-8, relax=synth.relaxation_sets()["N2_y1.0_a0.5"])
+    sim = fw2.Simulation(prob)
+    rng = np.random.default_rng(7)
+    for name in ("p", "v" + "xyz"[len(shape) - 1], "psi1x", "psi2y"):
+        g = ((2,) if name.startswith("psi") else ()) + prob.grid_shape
+        n = int(np.prod(g))
+        want = rng.standard_normal(n).astype(np.float32)
+        buf = torch.full((n + offset + 8,), -7.0, device="cuda")
+        buf[offset:offset + n] = torch.from_numpy(want).cuda()
+        fw2.fw2_set_field(sim.ctx, name, buf[offset:offset + n])
+        np.testing.assert_array_equal(sim.field(name).ravel(), want)
+        got = torch.full((n + offset + 8,), -7.0, device="cuda")
+        fw2.fw2_get_field(sim.ctx, name, got[offset:offset + n])
+        assert torch.equal(got, buf)
+        if not name.startswith("psi"):
+            rows = prob.grid_shape[0]
+            part = torch.empty((rows - 3,) + prob.grid_shape[1:], device="cuda")
+            fw2.fw2_get_rows(sim.ctx, name, 2, rows - 3, part)
+            np.testing.assert_array_equal(part.cpu().numpy(), want.reshape(g)[2:rows - 1])
+    sim.close()
