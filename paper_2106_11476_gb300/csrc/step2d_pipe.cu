@@ -554,6 +554,50 @@ __device__ __forceinline__ void y_strip_coef2(const StepParams &P, int nu, int i
   b = ldsb2(sb + off, P.ms[(OP == 1 ? kMsB1 : kMsB2) + nu]);
 }
 
+// C-PML coefficients of a pair of an edge half tile, every mechanism: the
+// values of the x strip where bit e of `x` is set (zero beyond the grid: those
+// cells are masked), those of the y strip where `y` is.  They depend on the
+// position alone, so they are loaded before the half tile's copies are waited
+// for.
+template <int N>
+struct EdgeCoef {
+  float2 xa[N > 0 ? N : 1], xb[N > 0 ? N : 1], ya[N > 0 ? N : 1], yb[N > 0 ? N : 1];
+  unsigned x;
+  bool y;
+};
+template <int N, int OP, typename Maps>
+__device__ __forceinline__ void load_edge(const StepParams &P, int x0, int y0, int tid, EdgeCoef<N> &c) {
+  c.x = 0;
+  c.y = false;
+  const int i0 = x0 + 2 * (tid & 63), j = y0 + (tid >> 6), L = P.L[0];
+  if (N == 0 || i0 >= P.nx || j >= P.ny) return;
+  if (L > 0 && (i0 < L || i0 + 1 >= P.nx - L)) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (i0 + e >= P.nx || strip_coord(i0 + e, P.nx, L) >= 0) c.x |= 1u << e;
+#pragma unroll
+    for (int nu = 0; nu < N; ++nu) {
+      c.xa[nu] = c.xb[nu] = make_float2(0.f, 0.f);
+      x_strip_coef2<OP, Maps>(P, nu, i0, j, c.xa[nu], c.xb[nu]);
+    }
+  }
+  const int sc = strip_coord(j, P.ny, P.L[1]);
+  if (sc >= 0) {
+    c.y = true;
+#pragma unroll
+    for (int nu = 0; nu < N; ++nu) y_strip_coef2<OP, Maps>(P, nu, i0, sc, c.ya[nu], c.yb[nu]);
+  }
+}
+// the coefficients of mechanism nu along x and y: a, b of the cells, or the strips'
+template <int N>
+__device__ __forceinline__ void pick_edge(const EdgeCoef<N> &c, int nu, float2 a, float2 b, float2 &ax, float2 &bx,
+                                          float2 &ay, float2 &by) {
+  ax = make_float2((c.x & 1u) ? c.xa[nu].x : a.x, (c.x & 2u) ? c.xa[nu].y : a.y);
+  bx = make_float2((c.x & 1u) ? c.xb[nu].x : b.x, (c.x & 2u) ? c.xb[nu].y : b.y);
+  ay = c.y ? c.ya[nu] : a;
+  by = c.y ? c.yb[nu] : b;
+}
+
 // Prefetch into L2 the C-PML strip rows an edge half tile will read (warp 0,
 // when its copies are issued): otherwise they come straight from DRAM while
 // the half tile computes.  OP: 1 velocity (a1, b1), 2 pressure (a2, b2).
@@ -594,7 +638,7 @@ __device__ __forceinline__ void prefetch_strips2(const StepParams &P, int x0, in
 
 template <int N, typename Maps, bool EDGE>
 __device__ __forceinline__ void vel_compute(const StepParams &P, const float *tab, float *st, int x0, int y0,
-                                            int tid) {
+                                            int tid, const EdgeCoef<N> &edge) {
   using S = VelStage<N, Maps>;
   using MT = typename S::F::MT;
   using IT = typename S::F::IT;
@@ -629,19 +673,14 @@ __device__ __forceinline__ void vel_compute(const StepParams &P, const float *ta
       B[nu] = ldbm2(mp + (1 + N + nu) * kArr, P.ms[kMsB1 + nu]);
     }
   }
-  // per-axis coefficients; in an edge pair the C-PML strips replace them,
-  // every strip value loaded before the first store (one memory latency)
+  // per-axis coefficients: in an edge pair the C-PML strips replace them
   float2 AX[N > 0 ? N : 1], BX[N > 0 ? N : 1], AY[N > 0 ? N : 1], BY[N > 0 ? N : 1];
 #pragma unroll
   for (int nu = 0; nu < N; ++nu) {
-    AX[nu] = A[nu]; BX[nu] = B[nu]; AY[nu] = A[nu]; BY[nu] = B[nu];
-  }
-  if (EDGE) {
-    const int scy = strip_coord(j, P.ny, P.L[1]);
-#pragma unroll
-    for (int nu = 0; nu < N; ++nu) {
-      x_strip_coef2<1, Maps>(P, nu, i0, j, AX[nu], BX[nu]);
-      if (scy >= 0) y_strip_coef2<1, Maps>(P, nu, i0, scy, AY[nu], BY[nu]);
+    if (EDGE) {
+      pick_edge<N>(edge, nu, A[nu], B[nu], AX[nu], BX[nu], AY[nu], BY[nu]);
+    } else {
+      AX[nu] = A[nu]; BX[nu] = B[nu]; AY[nu] = A[nu]; BY[nu] = B[nu];
     }
   }
   float2 vx = sld2(own), vy = sld2(own + kArr);
@@ -677,7 +716,7 @@ __device__ __forceinline__ void vel_compute(const StepParams &P, const float *ta
 
 template <int N, typename Maps, bool EDGE>
 __device__ __forceinline__ void prs_compute(const StepParams &P, const float *tab, float *st, int x0, int y0,
-                                            int tid) {
+                                            int tid, const EdgeCoef<N> &edge) {
   using S = PrsStage<N, Maps>;
   using MT = typename S::F::MT;
   using IT = typename S::F::IT;
@@ -714,17 +753,14 @@ __device__ __forceinline__ void prs_compute(const StepParams &P, const float *ta
       B[nu] = ldbm2(mp + (3 + N + nu) * kArr, P.ms[kMsB2 + nu]);
     }
   }
+  // per-axis coefficients: in an edge pair the C-PML strips replace them
   float2 AX[N > 0 ? N : 1], BX[N > 0 ? N : 1], AY[N > 0 ? N : 1], BY[N > 0 ? N : 1];
 #pragma unroll
   for (int nu = 0; nu < N; ++nu) {
-    AX[nu] = A[nu]; BX[nu] = B[nu]; AY[nu] = A[nu]; BY[nu] = B[nu];
-  }
-  if (EDGE) {
-    const int scy = strip_coord(j, P.ny, P.L[1]);
-#pragma unroll
-    for (int nu = 0; nu < N; ++nu) {
-      x_strip_coef2<2, Maps>(P, nu, i0, j, AX[nu], BX[nu]);
-      if (scy >= 0) y_strip_coef2<2, Maps>(P, nu, i0, scy, AY[nu], BY[nu]);
+    if (EDGE) {
+      pick_edge<N>(edge, nu, A[nu], B[nu], AX[nu], BX[nu], AY[nu], BY[nu]);
+    } else {
+      AX[nu] = A[nu]; BX[nu] = B[nu]; AY[nu] = A[nu]; BY[nu] = B[nu];
     }
   }
   float2 p = sld2(own);
@@ -1068,22 +1104,27 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   Walk w = start();
 #pragma unroll 1
   while (true) {
+    const bool vel = (w.ph & 1) == 0, interior = R.interior(w.x, w.y);
+    EdgeCoef<N> edge;
+    if (!interior) {
+      if (vel) load_edge<N, 1, Maps>(P, w.x, w.y, tid, edge);
+      else load_edge<N, 2, Maps>(P, w.x, w.y, tid, edge);
+    }
     if (!mbar_wait_bounded(&full[w.stage], w.parity)) {
       if ((tid & 31) == 0) report_status(P.status, kStatusWaitTimeout);
       return;
     }
-    const bool vel = (w.ph & 1) == 0;
     const long long n = w.ph >> 1;
     // the previous step's trace row, before this warp's first half tile of the
     // velocity phase (the operand is there, so every block's p is complete)
     if (vel && w.round == 0 && w.ph != ph0 && io.rec_groups > 0 && n - 1 < io.rec_steps) record_row(io, P.p, n - 1, tid);
     float *cur = smem + w.stage * kStage;
-    if (R.interior(w.x, w.y)) {
-      if (vel) vel_compute<N, Maps, false>(P, tab, cur, w.x, w.y, tid);
-      else prs_compute<N, Maps, false>(P, tab, cur, w.x, w.y, tid);
+    if (interior) {
+      if (vel) vel_compute<N, Maps, false>(P, tab, cur, w.x, w.y, tid, edge);
+      else prs_compute<N, Maps, false>(P, tab, cur, w.x, w.y, tid, edge);
     } else {
-      if (vel) vel_compute<N, Maps, true>(P, tab, cur, w.x, w.y, tid);
-      else prs_compute<N, Maps, true>(P, tab, cur, w.x, w.y, tid);
+      if (vel) vel_compute<N, Maps, true>(P, tab, cur, w.x, w.y, tid, edge);
+      else prs_compute<N, Maps, true>(P, tab, cur, w.x, w.y, tid, edge);
     }
     fence_proxy_async_smem();
     __syncwarp();
@@ -1188,12 +1229,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       ++hs;
     }
     float *stp = smem + s * kStage;
+    EdgeCoef<N> edge;
     if (e.w) {
-      if (VEL) vel_compute<N, Maps, false>(sP, tab, stp, e.y, e.z, tid);
-      else prs_compute<N, Maps, false>(sP, tab, stp, e.y, e.z, tid);
+      if (VEL) vel_compute<N, Maps, false>(sP, tab, stp, e.y, e.z, tid, edge);
+      else prs_compute<N, Maps, false>(sP, tab, stp, e.y, e.z, tid, edge);
     } else {
-      if (VEL) vel_compute<N, Maps, true>(sP, tab, stp, e.y, e.z, tid);
-      else prs_compute<N, Maps, true>(sP, tab, stp, e.y, e.z, tid);
+      load_edge<N, VEL ? 1 : 2, Maps>(sP, e.y, e.z, tid, edge);
+      if (VEL) vel_compute<N, Maps, true>(sP, tab, stp, e.y, e.z, tid, edge);
+      else prs_compute<N, Maps, true>(sP, tab, stp, e.y, e.z, tid, edge);
     }
     if constexpr (TmaStore<Maps>::value) fence_proxy_async_smem();
     prev = e;
