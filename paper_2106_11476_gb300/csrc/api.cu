@@ -215,6 +215,7 @@ fw2_status finalize(fw2_ctx *c) {
     strip_bytes[q] = align256(es * (size_t)(strip_nu[q] * (c->N ? c->N : 1)));
     if (strip_nu[q]) total += 4 * strip_bytes[q];
   }
+  total += strips ? align256(profile_bytes(Q)) : 0;  // (a small allocation of its own would split the pool's blocks)
   if (c->maps) {
     dfree(c, c->maps);
     c->maps = nullptr;
@@ -240,9 +241,7 @@ fw2_status finalize(fw2_ctx *c) {
     }
   }
   if (strips) {
-    void *pb;
-    if ((st = dalloc(c, profile_bytes(Q), &pb)) != FW2_OK) return st;
-    Q.profile = pb;
+    Q.profile = take(align256(profile_bytes(Q)));
     CK(c, launch_profiles(Q, c->stream));
     c->launches++;
   }
@@ -291,7 +290,6 @@ fw2_status finalize(fw2_ctx *c) {
   }
   dfree(c, c->raw_tissue);
   c->raw_tissue = nullptr;
-  dfree(c, Q.profile);
   c->medium_set = c->relax_set = false;
   // step parameters
   StepParams &P = c->P;
@@ -346,7 +344,7 @@ fw2_status finalize(fw2_ctx *c) {
 fw2_status build_sources(fw2_ctx *c) {
   if (!c->src_dirty) return FW2_OK;
   for (DevSource &d : c->dsrc) {
-    dfree(c, d.tgt); dfree(c, d.off); dfree(c, d.col); dfree(c, d.unit); dfree(c, d.pos);
+    dfree(c, d.tgt);  // the other arrays lie behind it
     d = DevSource{};
   }
   dfree(c, c->d_signal);
@@ -415,25 +413,28 @@ fw2_status build_sources(fw2_ctx *c) {
     DevSource &d = c->dsrc[kind];
     void *m;
     fw2_status st;
-    if ((st = dalloc(c, tgt.size() * sizeof(long long), &m)) != FW2_OK) return st;
-    d.tgt = (long long *)m;
-    if ((st = dalloc(c, off.size() * sizeof(int), &m)) != FW2_OK) return st;
-    d.off = (int *)m;
-    if ((st = dalloc(c, col.size() * sizeof(int), &m)) != FW2_OK) return st;
-    d.col = (int *)m;
-    d.n_tgt = (int)tgt.size();
-    if (c->nd == 2) {
+    if (c->nd == 2)
       for (size_t u = 1; u < unit.size(); ++u) unit[u] += unit[u - 1];
-      if ((st = dalloc(c, unit.size() * sizeof(int), &m)) != FW2_OK) return st;
-      d.unit = (int *)m;
-      if ((st = dalloc(c, pos.size() * sizeof(int), &m)) != FW2_OK) return st;
-      d.pos = (int *)m;
-      CK(c, cudaMemcpyAsync(d.unit, unit.data(), unit.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-      CK(c, cudaMemcpyAsync(d.pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    }
-    CK(c, cudaMemcpyAsync(d.tgt, tgt.data(), tgt.size() * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-    CK(c, cudaMemcpyAsync(d.off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    CK(c, cudaMemcpyAsync(d.col, col.data(), col.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    const size_t bt = align256(tgt.size() * sizeof(long long)), bo = align256(off.size() * sizeof(int)),
+                 bc = align256(col.size() * sizeof(int)), bu = align256(unit.size() * sizeof(int)),
+                 bp = align256(pos.size() * sizeof(int));
+    if ((st = dalloc(c, bt + bo + bc + bu + bp, &m)) != FW2_OK) return st;
+    char *cur = (char *)m;
+    auto put = [&](const void *src, size_t bytes, size_t room) {
+      void *dst = cur;
+      cur += room;
+      return std::make_pair(dst, bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream) : cudaSuccess);
+    };
+    const auto ct = put(tgt.data(), tgt.size() * sizeof(long long), bt), co = put(off.data(), off.size() * sizeof(int), bo),
+               cc = put(col.data(), col.size() * sizeof(int), bc), cu = put(unit.data(), unit.size() * sizeof(int), bu),
+               cp = put(pos.data(), pos.size() * sizeof(int), bp);
+    d.tgt = (long long *)ct.first;
+    d.off = (int *)co.first;
+    d.col = (int *)cc.first;
+    d.unit = c->nd == 2 ? (int *)cu.first : nullptr;
+    d.pos = c->nd == 2 ? (int *)cp.first : nullptr;
+    d.n_tgt = (int)tgt.size();
+    for (const cudaError_t e : {ct.second, co.second, cc.second, cu.second, cp.second}) CK(c, e);
     CK(c, cudaStreamSynchronize(c->stream));
   }
   c->src_dirty = false;
@@ -813,11 +814,15 @@ fw2_status fw2_create(const fw2_config *cfg_in, fw2_ctx **out) {
     for (int q = 0; q < c->nd; ++q) { c->v[q] = (float *)cur; cur += arr; }
     for (int q = 0; q < c->nd; ++q) { c->psi1[q] = (float *)cur; cur += arr * c->N; }
     for (int q = 0; q < c->nd; ++q) { c->psi2[q] = (float *)cur; cur += arr * c->N; }
-    if ((st = dalloc(c, sizeof(ScanOut), &m)) == FW2_OK) c->d_scan = (ScanOut *)m;
-    if (st == FW2_OK && (st = dalloc(c, sizeof(unsigned int), &m)) == FW2_OK) c->d_absmax = (unsigned int *)m;
-    if (st == FW2_OK && (st = dalloc(c, sizeof(unsigned int), &m)) == FW2_OK) c->d_status = (unsigned int *)m;
-    if (st == FW2_OK && (st = dalloc(c, sizeof(unsigned long long), &m)) == FW2_OK)
-      c->d_sync = (unsigned long long *)m;
+    // the small words in one allocation, 64 bytes apart
+    if ((st = dalloc(c, 256, &m)) == FW2_OK) {
+      char *w = (char *)m;
+      static_assert(sizeof(ScanOut) <= 64, "the scan result has 64 bytes");
+      c->d_scan = (ScanOut *)w;
+      c->d_absmax = (unsigned int *)(w + 64);
+      c->d_status = (unsigned int *)(w + 128);
+      c->d_sync = (unsigned long long *)(w + 192);
+    }
   }
   if (st == FW2_OK) {
     cudaError_t e2 = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned int), c->stream);
