@@ -68,12 +68,13 @@ enum { FW2_NL_OFF = 0, FW2_NL_PRESSURE = 1, FW2_NL_WESTERVELT = 2, FW2_NL_LITERA
 /* storage of the coefficient maps: float, bf16 (b kept as 1 - b), FP16
  * (every map, and the C-PML strips of a mechanism with its interior map,
  * divided by a power of two chosen from the map's largest magnitude so that
- * it lies in [2^14, 2^15); b kept as 1 - b; tile kernels), or a tissue index
+ * it lies in [2^14, 2^15); b kept as 1 - b), or a tissue index
  * per cell into per-tissue float tables (N <= 4; set the medium with
  * fw2_set_medium_indexed): uint8 for up to 256 tissues or uint16 for up to
  * 65536.  In 2D the uint8 tables sit in shared memory (pipelined or tile
- * kernels); the uint16 tables, and every table in 3D, are read through L2 by
- * the tile kernels. */
+ * kernels), the uint16 tables too on the pipelined kernels while they fit
+ * (about 1480 tissues with four mechanisms); larger ones, and every table in
+ * 3D, are read through L2 by the tile kernels. */
 enum { FW2_MAP_F32 = 0, FW2_MAP_BF16 = 1, FW2_MAP_IDX_U8 = 2, FW2_MAP_IDX_U16 = 3, FW2_MAP_F16 = 4 };
 /* C-PML geometry (Sec. 3.3, Table 1).  In both readings the nu >= 2
  * parameters fall to zero over the inner L_T cells with the cosine transition
@@ -108,9 +109,12 @@ enum { FW2_MEM_CENTRED = 0, FW2_MEM_ENDPOINT = 1 };
 /* kernel path of the half steps (bitwise the same results on every path):
  * TILE runs one block per tile; PIPE runs the persistent kernels that stage
  * every tile through shared memory with TMA copies, where they apply (2D
- * float or tissue-index maps; 3D bf16 maps with N <= 3, g_{1,1} cross taps
- * and the literal system included; no periodic axis), and TILE elsewhere;
- * AUTO (default) is PIPE where it applies.  The 3D pipelined half steps have two layouts:
+ * with N <= 4, every storage, the uint16 index while its tables fit; 3D float
+ * or bf16 maps with N <= 3; g_{1,1} cross taps and the literal system
+ * included; no periodic axis), and TILE elsewhere; AUTO (default) is PIPE
+ * where it applies.  On the 2D pipelined path fw2_step takes many steps per
+ * launch, with sources and recording inside.  The 3D pipelined half steps of
+ * bf16 maps have two layouts (float maps: the second):
  * the memory variables staged in shared memory with the other arrays, or
  * loaded into registers one unit ahead, which leaves room to stage every
  * C-PML strip (faster where edge units dominate); the cross taps and the
@@ -492,10 +496,11 @@ fw2_status fw2_pipe_layout(fw2_ctx *ctx, int32_t *vel, int32_t *prs);
 fw2_status fw2_release_memory(void);
 /* Bytes of device memory held by the context. */
 fw2_status fw2_device_bytes(fw2_ctx *ctx, int64_t *bytes);
-/* Launches of library kernels since creation (all kinds). */
+/* Launches of library kernels since creation (all kinds; one launch may cover
+ * many time steps). */
 fw2_status fw2_kernel_launches(fw2_ctx *ctx, int64_t *count);
-/* Per-kernel timing: with enable = 1, fw2_step brackets every velocity and
- * pressure kernel launch with CUDA events on the context stream. */
+/* Per-kernel timing: with enable = 1, fw2_step launches every half step by
+ * itself and brackets the launch with CUDA events on the context stream. */
 fw2_status fw2_profile(fw2_ctx *ctx, int32_t enable);
 /* Synchronise and return the summed event time [ms] and launch counts of the
  * velocity and pressure kernels since profiling was enabled; clears them. */

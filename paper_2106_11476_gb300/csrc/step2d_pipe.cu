@@ -884,7 +884,9 @@ __device__ __forceinline__ void inject_unit(const StepIO &io, int u, long long n
   }
 }
 
-// Trace row of one step, groups spread over the blocks' last threads: the
+// Trace row of one step, groups spread over the blocks' last threads (the
+// copying warp had it on the path of its stores: 250 x 186 took 10.3 us a step
+// and not 9.1): the
 // mean of p over a group's cells, summed in their order.  p was written by
 // other SMs during this launch: read through L2, eight loads in flight.
 __device__ __forceinline__ void record_row(const StepIO &io, const float *p, long long n, int tid) {
@@ -910,15 +912,15 @@ __device__ __forceinline__ void record_row(const StepIO &io, const float *p, lon
 // stores and adds the sources.  More than one phase needs a cooperative launch, since the blocks
 // wait for one another between phases.
 //
-// What bounds it: HBM on grids beyond L2 (4096^2, N = 4: 655 us a step,
-// 0.91 of the copy bandwidth on the step's bytes), the latency chain of a phase
+// What bounds it: HBM on grids beyond L2 (4096^2, N = 4: 650 us a step,
+// 0.92 of the copy bandwidth on the step's bytes), the latency chain of a phase
 // (operand copy, compute, store, grid barrier: about 5 us) on small ones.
 // Four launches per step (two half steps, sources, recording) added to every
 // one of them a start and a drain and left the SMs without copies in flight
 // meanwhile; here the next phase's first half tiles are copied (all but the
 // operand) while the barrier is under way, and sources and recording need no
-// launch of their own.  A step of 250 x 186 (N = 2) took 21 us and takes 9.8,
-// 512^2 (N = 4) 30 and 17, 1501 x 1237 111 and 87.  The velocity phases walk
+// launch of their own.  A step of 250 x 186 (N = 2) took 21 us and takes 8.5,
+// 512^2 (N = 4) 30 and 15.8, 1501 x 1237 111 and 75.  The velocity phases walk
 // the half tiles forwards and the pressure phases backwards, so each starts on
 // the rows whose operand the previous one left in L2 (0.8 % at 1501 x 1237).
 //
@@ -1134,7 +1136,11 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   }
 }
 
-// Batched half step over a unit table of several contexts (one group: same
+// Batched half step over a unit table of several contexts, 512 threads and one
+// barrier per unit (a warp of its own for the copies, as in steps2d_kernel,
+// was slower here, 12.1 against 11.2 ms for six contexts and 32 steps: every
+// context change empties the pipeline and leaves the index table to one warp)
+// (one group: same
 // N and map kind, no periodic axis): entry (ctx, x0, y0, interior).  The
 // contexts' step parameters and tensor maps sit in device memory (TMA reads
 // the maps from there); a block copies a context's parameters to shared

@@ -1,6 +1,8 @@
-// Pipelined persistent 3D half steps (sm_103a) for bf16 coefficient maps;
-// same arithmetic as step3d.cu (bitwise the same results), one launch per
-// half step, one block of 512 threads per SM (two x cells per thread).
+// Pipelined persistent 3D half steps (sm_103a) for bf16 and float coefficient
+// maps; same arithmetic as step3d.cu (bitwise the same results), one launch per
+// half step, one block per SM, 512 computing threads (two x cells each).  This
+// file is compiled twice: for bf16 maps, and with FW2_PIPE3D_FLOAT the kernels
+// for float maps.
 //
 // Work unit: a 128 x 8 half tile of one z plane.  A block marches a column
 // of units through z (a work item: one xy position and a range of planes;
@@ -15,21 +17,22 @@
 // v_z slots carry the same halo.  For a coming unit one thread issues tiled
 // TMA tensor copies, one box per array, into a free stage of a two-stage
 // ring: the operand planes the unit adds, the density of the plane and of
-// the next one, the velocity (or pressure) of the unit, the bf16 maps (a and
-// b of the N mechanisms in one 4D box each), K of planes k and k + 1 for the
+// the next one, the velocity (or pressure) of the unit, the maps (a and b
+// of the N mechanisms in one 4D box each), K of planes k and k + 1 for the
 // literal system's momentum factor, and in edge units the C-PML strip
 // coefficients of each axis the unit reaches.  The memory variables, read
-// once and written once by the thread that owns the cell, bypass shared
-// memory: every thread loads the next unit's into registers while it
-// computes the current one.  Copies complete on the stage's mbarrier while
-// all threads compute the current unit from the other stage.
+// once and written once by the thread that owns the cell, come with the stage
+// too (staged layout) or bypass shared memory, every thread loading the next
+// unit's into registers while it computes the current one (register layout).
+// Copies complete on the stage's mbarrier while the threads compute the
+// current unit from the other stage.
 //
 // Boundaries as in the 2D pipeline: the copies read zero outside the grid;
 // units at the grid's edge or in a C-PML strip clamp the density to the last
 // cell, take each axis' C-PML coefficients from its strip (staged, or read
 // per cell where a box cannot serve: a strip wider than 64 cells or not a
 // multiple of 8 along x, a grid too small for a unit to reach one side only
-// along y) and store nothing outside the grid.  Periodic axes are not taken
+// along y; float maps: every y and z strip) and store nothing outside the grid.  Periodic axes are not taken
 // by this path (the tile kernels run them).
 #include <climits>
 #include <cstring>
