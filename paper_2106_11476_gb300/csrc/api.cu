@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "ctx.h"
+#include "routes.h"
 
 using namespace fw2;
 
@@ -372,6 +373,7 @@ fw2_status build_sources(fw2_ctx *c) {
     CK(c, cudaMemcpyAsync(c->d_signal, table.data(), table.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
   }
+  long long half_tiles = 0, targets = 0, entries = 0;  // of every field (2D)
   for (int kind = 0; kind < 4; ++kind) {
     struct E { long long tgt; int unit, pos, col; long long order; };
     const int ntx = (c->nx + kTX - 1) / kTX, nhy = (c->ny + kPipeHalf - 1) / kPipeHalf;
@@ -413,8 +415,14 @@ fw2_status build_sources(fw2_ctx *c) {
     DevSource &d = c->dsrc[kind];
     void *m;
     fw2_status st;
-    if (c->nd == 2)
-      for (size_t u = 1; u < unit.size(); ++u) unit[u] += unit[u - 1];
+    if (c->nd == 2) {
+      for (size_t u = 1; u < unit.size(); ++u) {
+        half_tiles += unit[u] > 0;
+        unit[u] += unit[u - 1];
+      }
+      targets += (long long)tgt.size();
+      entries += (long long)col.size();
+    }
     const size_t bt = align256(tgt.size() * sizeof(long long)), bo = align256(off.size() * sizeof(int)),
                  bc = align256(col.size() * sizeof(int)), bu = align256(unit.size() * sizeof(int)),
                  bp = align256(pos.size() * sizeof(int));
@@ -437,6 +445,7 @@ fw2_status build_sources(fw2_ctx *c) {
     for (const cudaError_t e : {ct.second, co.second, cc.second, cu.second, cp.second}) CK(c, e);
     CK(c, cudaStreamSynchronize(c->stream));
   }
+  c->src_apart = sources_apart(half_tiles, targets, entries - targets, c->n_sm);
   c->src_dirty = false;
   return FW2_OK;
 }
@@ -508,7 +517,7 @@ StepIO step_io(const fw2_ctx *c) {
   StepIO io{};
   for (int k = 0; k < 3; ++k) {
     const DevSource &d = c->dsrc[k];
-    if (d.n_tgt > 0) io.src[k] = {d.unit, d.pos, d.off, d.col};
+    if (d.n_tgt > 0 && !c->src_apart) io.src[k] = {d.unit, d.pos, d.off, d.col};
   }
   io.signal = c->d_signal;
   io.sig_cols = c->sig_cols;
@@ -553,7 +562,7 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
     return pipe3d_layout_allowed(vel, P, l) ? l : kLayoutRegisters;
   };
   const bool do_vel = part != 1, do_prs = part != 0;
-  const bool pipe2 = c->pipe && c->nd == 2;  // its sources are part of the half steps
+  const bool inside = c->pipe && c->nd == 2 && !c->src_apart;  // the sources are part of the half steps
   struct TrialEvents {  // destroyed on every return, error paths included
     cudaEvent_t e[4] = {nullptr, nullptr, nullptr, nullptr};
     ~TrialEvents() {
@@ -582,7 +591,7 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
     c->ev_vel.push_back(ev);
     ev = {take_event(c), take_event(c)};
   }
-  if (!pipe2 && n < c->sig_steps) {
+  if (!inside && n < c->sig_steps) {
     for (int kind = 1; kind <= c->nd; ++kind) {
       const DevSource &d = c->dsrc[kind];
       if (d.n_tgt == 0) continue;
@@ -611,7 +620,7 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
     CK(c, cudaEventRecord(ev.second, c->stream));
     c->ev_prs.push_back(ev);
   }
-  if (!pipe2 && n < c->sig_steps && c->dsrc[0].n_tgt > 0) {
+  if (!inside && n < c->sig_steps && c->dsrc[0].n_tgt > 0) {
     const DevSource &d = c->dsrc[0];
     CK(c, launch_inject(c->p, d.tgt, d.off, d.col, c->d_signal + n * c->sig_cols, d.n_tgt, c->stream));
     c->launches++;
@@ -1053,10 +1062,10 @@ fw2_status fw2_step(fw2_ctx *c, int64_t n_steps) {
   fw2_status st;
   if ((st = finalize(c)) != FW2_OK) return st;
   if ((st = build_sources(c)) != FW2_OK) return st;
-  // many steps a launch, up to the next scan (per-launch timing: one launch
-  // per half step)
-  const bool multi = c->pipe && c->nd == 2 && !c->profiling;
   for (int64_t s = 0; s < n_steps;) {
+    // many steps a launch, up to the next scan (per-launch timing, and while
+    // sources fire that have kernels of their own: one launch per half step)
+    const bool multi = c->pipe && c->nd == 2 && !c->profiling && !(c->src_apart && c->step < c->sig_steps);
     int64_t take = 1;
     if (multi) {
       // at most 2^28 cell-steps (about 11 ms) and 256 steps, so that work on

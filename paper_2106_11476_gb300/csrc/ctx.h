@@ -69,6 +69,7 @@ struct fw2_ctx {
   std::vector<HostSource> sources;
   bool src_dirty = false;
   DevSource dsrc[4];
+  bool src_apart = false;  // 2D: they run as kernels of their own on the pipelined path too (sources_apart)
   float *d_signal = nullptr;
   long long sig_steps = 0, sig_cols = 0;
   // recording

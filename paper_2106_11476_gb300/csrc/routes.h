@@ -1,0 +1,25 @@
+// Host rules that choose how a call runs (no CUDA types, so that they can be
+// compiled and checked without a device).
+#pragma once
+
+namespace fw2 {
+
+// Sources of a 2D pipelined context: inside the half steps (one warp of each
+// block adds those of its half tiles) or by a kernel of their own after each
+// half step.  Inside, a block's warp takes about 1.5 us for a half tile with
+// sources, 9 ns more for each of its targets and a memory latency (0.6 us) for
+// each further entry of a target, one after the other; kernels of their own,
+// with a launch per half step, cost about 16 us a step more.  The line is
+// where the two meet, at ten half tiles per SM: 2048 x 1024 (N = 4, float)
+// with every cell a source took 223 us a step inside and takes 104 apart, a
+// quarter of the cells 123 and 96, one in 64 100 and 94; 512 x 512 with every
+// cell 25 either way, with a quarter of them 19 inside.  It also keeps what a
+// block adds within a few ms, far below the limit of the waits that the other
+// blocks spend on it.
+// half_tiles: half tiles with sources, targets: cells fed, extra: entries
+// beyond the first of a target, each summed over the fields.
+inline bool sources_apart(long long half_tiles, long long targets, long long extra, int n_sm) {
+  return (double)half_tiles + (double)targets / 170.0 + 0.4 * (double)extra > 10.0 * n_sm;
+}
+
+}  // namespace fw2

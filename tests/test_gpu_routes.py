@@ -1,0 +1,70 @@
+"""Calls that the pipelined 2D path hands to kernels of their own, and launches
+that it does not make: the same bits as the tile kernels either way, and the
+route that the rule of the sizes says (counted in launches)."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fw2(fw2lib):
+    from paper_2106_11476_gb300 import fw2 as m
+    return m
+
+
+def problem(nx, ny, N=2, steps=6):
+    prob = synth.homogeneous((nx, ny), 1e-4, 0.0, relax=synth.relaxation_sets()["N2_y1.0_a0.5"] if N else None, beta=4.0)
+    prob.c = (1500 + 100 * np.random.default_rng(3).random(prob.grid_shape)).astype(np.float32)
+    prob.nl_mode = "pressure"
+    prob.dt = 0.3 * 1e-4 / 2200.0
+    if N:
+        prob.pml_transition, prob.pml_bound = 5, 3
+    prob.n_steps = steps
+    prob.sensors = synth.Sensors(idx=np.arange(40, dtype=np.int64) * 5, group=np.zeros(40, np.int32), n_groups=1)
+    return prob
+
+
+def run(fw2, prob, steps, path):
+    """Fields, trace and the launches of one fw2_step call."""
+    sim = fw2.Simulation(prob, kernel_path=path)
+    sim.set_state(synth.random_state(prob, seed=4))
+    before = sim.launches
+    sim.step(steps)
+    n = sim.launches - before
+    sim.synchronize()
+    assert fw2.fw2_kernel_path(sim.ctx) == ("tile" if path == "tile" else "pipe")
+    out = {f: sim.field(f) for f in ("p", "vx", "vy") + (("psi1x", "psi2y") if prob.nrelax else ())}
+    out["trace"] = sim.trace.cpu().numpy()
+    sim.close()
+    return out, n
+
+
+def same(fw2, prob, steps):
+    want, _ = run(fw2, prob, steps, "tile")
+    got, launches = run(fw2, prob, steps, "auto")
+    assert np.isfinite(want["p"]).all()
+    for f, w in want.items():
+        np.testing.assert_array_equal(got[f], w, err_msg=f)
+    return launches
+
+
+def sources(idx, group, rows, n_groups):
+    sig = np.random.default_rng(5).standard_normal((rows, n_groups)).astype(np.float32)
+    return [synth.Source("p", idx, group, 1e3 * sig), synth.Source("vy", idx[:7], group[:7], 1e-3 * sig)]
+
+
+@pytest.mark.parametrize("nx,ny,cells,repeat,apart", [
+    (600, 500, 600 * 500, 1, True),      # every cell
+    (600, 500, 2000, 1, False), (203, 77, 203 * 77, 1, False),
+    (203, 77, 5, 900, True)])            # 900 entries in each of five cells
+def test_dense_and_chained_sources_run_as_kernels_of_their_own(fw2, nx, ny, cells, repeat, apart):
+    prob = problem(nx, ny)
+    idx = np.tile(np.random.default_rng(6).choice(nx * ny, cells, replace=False), repeat).astype(np.int64)
+    prob.sources = sources(idx, (np.arange(idx.size) % 3).astype(np.int32), 4, 3)
+    # six steps, sources for four: apart, two half steps, two source kernels
+    # and the recording a step, then one launch (and the last recording);
+    # inside, one launch
+    assert same(fw2, prob, 6) == (4 * 5 + 2 if apart else 2)
