@@ -1037,6 +1037,7 @@ fw2_status fw2_record(fw2_ctx *c, int64_t n_pts, const int64_t *idx, const int32
     if (grp[e] < 0 || grp[e] >= n_groups) return fail(c, FW2_EINVAL, "sensor group %d out of range", grp[e]);
     count[grp[e] + 1]++;
   }
+  const long long longest = *std::max_element(count.begin(), count.end());
   for (long long g = 0; g < n_groups; ++g) count[g + 1] += count[g];
   std::vector<long long> cells((size_t)n_pts);
   std::vector<int> fill(count.begin(), count.end() - 1);
@@ -1049,6 +1050,7 @@ fw2_status fw2_record(fw2_ctx *c, int64_t n_pts, const int64_t *idx, const int32
   CK(c, cudaMemcpyAsync(c->rec_cell, cells.data(), cells.size() * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
   CK(c, cudaMemcpyAsync(c->rec_off, count.data(), count.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
+  c->rec_apart = record_apart(longest, n_pts);
   c->rec_groups = (int)n_groups;
   c->rec_out = out;
   c->rec_steps = n_steps;
@@ -1072,6 +1074,8 @@ fw2_status fw2_step(fw2_ctx *c, int64_t n_steps) {
       // other streams of the device gets its turn
       const int64_t cap = std::max<int64_t>(1, (1ll << 28) / c->n_pts);
       take = std::min<int64_t>(n_steps - s, std::min<int64_t>(cap, 256));
+      // the recording of a launch's last step is a kernel of its own
+      if (c->rec_apart && c->rec_groups > 0 && c->step < c->rec_steps) take = 1;
       if (c->watch_every > 0) take = std::min<int64_t>(take, c->watch_every - c->step % c->watch_every);
     }
     if ((st = multi ? enqueue_steps2d(c, c->step, take) : enqueue_step(c, c->step)) != FW2_OK) return st;

@@ -76,6 +76,7 @@ struct fw2_ctx {
   long long *rec_cell = nullptr;
   int *rec_off = nullptr;
   int rec_groups = 0;
+  bool rec_apart = false;  // by a kernel of its own on the 2D pipelined path too (record_apart)
   float *rec_out = nullptr;
   long long rec_steps = 0;
   // scratch words for scans

@@ -22,4 +22,16 @@ inline bool sources_apart(long long half_tiles, long long targets, long long ext
   return (double)half_tiles + (double)targets / 170.0 + 0.4 * (double)extra > 10.0 * n_sm;
 }
 
+// Recording of a 2D pipelined context: inside a launch of many steps (each
+// group summed by one thread in the following half step, while the others of
+// its warp wait), or by a kernel of its own after launches of one step.
+// Inside, a long group costs 55 to 80 ns a cell that the whole grid waits for
+// (35 to 50 in its own kernel), with a limit on that wait of 2 s; launches of
+// one step cost 3 to 7 us a step and the kernel 4.  512 x 512 and 2048 x 1024
+// (N = 4), groups of 256 cells: 31 and 111 us a step inside; of 512: 46 and
+// 126 apart; of 10000: 554 and 844 inside, 350 and 594 apart.  Many sensors:
+// every cell of 2048 x 1024 140 inside and 107 apart, a quarter 95 and 96.
+// longest: cells of the longest group, cells: of all groups.
+inline bool record_apart(long long longest, long long cells) { return longest > 384 || cells > (1ll << 19); }
+
 }  // namespace fw2

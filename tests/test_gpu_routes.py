@@ -68,3 +68,17 @@ def test_dense_and_chained_sources_run_as_kernels_of_their_own(fw2, nx, ny, cell
     # and the recording a step, then one launch (and the last recording);
     # inside, one launch
     assert same(fw2, prob, 6) == (4 * 5 + 2 if apart else 2)
+
+
+@pytest.mark.parametrize("nx,ny,groups,apart", [
+    (203, 77, [384, 1, 40], False), (203, 77, [3, 385], True), (203, 77, [203 * 77], True),
+    (800, 700, [1] * (800 * 700), True), (800, 500, [1] * (800 * 500), False)])
+def test_long_groups_and_dense_sensors_are_recorded_by_a_kernel_of_its_own(fw2, nx, ny, groups, apart):
+    prob = problem(nx, ny, N=0, steps=5)
+    k = sum(groups)
+    idx = np.sort(np.random.default_rng(8).choice(nx * ny, k, replace=False)).astype(np.int64)
+    prob.sensors = synth.Sensors(idx=idx, group=np.repeat(np.arange(len(groups)), groups).astype(np.int32),
+                                 n_groups=len(groups))
+    # seven steps with trace rows for five: apart, a launch and the recording
+    # a step, then one launch; inside, one launch whose last step has no row
+    assert same(fw2, prob, 7) == (5 * 2 + 1 if apart else 1)

@@ -11,6 +11,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 WRAPPER = r"""
 #include "routes.h"
 extern "C" int sources_apart(long long h, long long t, long long e, int n) { return fw2::sources_apart(h, t, e, n); }
+extern "C" int record_apart(long long l, long long c) { return fw2::record_apart(l, c); }
 """
 
 
@@ -22,6 +23,7 @@ def rules(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", str(lib)], check=True)
     m = C.CDLL(str(lib))
     m.sources_apart.argtypes = [C.c_longlong, C.c_longlong, C.c_longlong, C.c_int]
+    m.record_apart.argtypes = [C.c_longlong, C.c_longlong]
     return m
 
 
@@ -39,3 +41,10 @@ def test_dense_sources_and_long_chains_run_apart(rules):
     assert apart(2048, 1024, 2048 * 1024) and apart(2048, 1024, 2048 * 256)
     assert apart(4096, 4096, 20000)                              # scattered over every half tile
     assert not apart(250, 186, 13, extra=3000, half_tiles=3) and apart(250, 186, 13, extra=4000, half_tiles=3)
+
+
+@pytest.mark.parametrize("longest,cells,apart", [(1, 256, False), (11, 704, False), (384, 6144, False), (385, 385, True),
+                                                 (1, 1 << 19, False), (1, (1 << 19) + 1, True),
+                                                 (2**31, 2**31, True)])
+def test_long_groups_and_dense_sensors_are_recorded_apart(rules, longest, cells, apart):
+    assert bool(rules.record_apart(longest, cells)) is apart
