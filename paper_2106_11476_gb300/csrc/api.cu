@@ -809,6 +809,7 @@ fw2_status fw2_create(const fw2_config *cfg_in, fw2_ctx **out) {
   c->n_pts = (long long)c->nx * c->ny * c->nz;
   c->stream = (cudaStream_t)cfg.stream;
   c->map_kind = cfg.map_precision;
+  c->device = dev;
   c->n_sm = prop.multiProcessorCount;
   // state: p, v_q, psi1_q[N], psi2_q[N]
   const size_t arr = align256(sizeof(float) * (size_t)c->npts_alloc);
@@ -1135,16 +1136,18 @@ fw2_status fw2_set_subdomain(fw2_ctx *c, const int64_t *global_n, const int64_t 
 }
 
 // `arrays` state arrays (npts_alloc apart, `rows` rows of nx values from
-// `dev`) to or from a dense caller buffer; synchronous.  Buffers in memory of
-// this device go through a kernel, everything else through the copy calls.
+// `dev`) to or from a dense caller buffer; synchronous (by a kernel or the
+// copy calls: copy_by_kernel).
 static fw2_status copy_state(fw2_ctx *c, float *dev, long long rows, int arrays, float *buf, int32_t mem_space,
                              bool out) {
   cudaPointerAttributes at{};
-  int here = -1;
-  bool local = mem_space == FW2_MEM_DEVICE && cudaGetDevice(&here) == cudaSuccess &&
-               cudaPointerGetAttributes(&at, buf) == cudaSuccess &&
-               (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == here &&
-               reinterpret_cast<uintptr_t>(buf) % sizeof(float) == 0;
+  int here = -1, buf_device = -1;
+  bool local = false;
+  if (mem_space == FW2_MEM_DEVICE && cudaGetDevice(&here) == cudaSuccess &&
+      cudaPointerGetAttributes(&at, buf) == cudaSuccess) {
+    if (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) buf_device = at.device;
+    local = copy_by_kernel(c->device, here, buf_device, reinterpret_cast<uintptr_t>(buf) % sizeof(float) == 0);
+  }
   if (local) {
     const long long dense = rows * c->nx;
     CK(c, out ? launch_copy_rows(buf, c->nx, dense, dev, c->pitch, c->npts_alloc, c->nx, rows, arrays, c->stream)

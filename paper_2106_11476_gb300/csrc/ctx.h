@@ -61,6 +61,7 @@ struct fw2_ctx {
   char *maps = nullptr;
   StepParams P{};
   int map_kind = 0;  // FW2_MAP_*
+  int device = 0;    // its memory and streams are this device's
   int n_sm = 152;    // multiprocessors of the device
   bool pipe = false; // 2D half steps by the pipelined kernels
   fw2::PipeMaps tm_vel{}, tm_prs{};  // their tensor maps

@@ -34,4 +34,13 @@ inline bool sources_apart(long long half_tiles, long long targets, long long ext
 // longest: cells of the longest group, cells: of all groups.
 inline bool record_apart(long long longest, long long cells) { return longest > 384 || cells > (1ll << 19); }
 
+// Field copies between a context and a caller's device buffer: by a kernel
+// where the context's device is current and holds the buffer, else by the copy
+// calls, which reach any device from any other (a kernel would be launched on
+// the current device and follow the pointers of another).
+// buf_device: device of the buffer, -1 where it is not device memory.
+inline bool copy_by_kernel(int ctx_device, int current_device, int buf_device, bool aligned) {
+  return aligned && buf_device >= 0 && buf_device == ctx_device && current_device == ctx_device;
+}
+
 }  // namespace fw2

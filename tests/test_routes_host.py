@@ -12,6 +12,7 @@ WRAPPER = r"""
 #include "routes.h"
 extern "C" int sources_apart(long long h, long long t, long long e, int n) { return fw2::sources_apart(h, t, e, n); }
 extern "C" int record_apart(long long l, long long c) { return fw2::record_apart(l, c); }
+extern "C" int copy_by_kernel(int c, int h, int b, int a) { return fw2::copy_by_kernel(c, h, b, a); }
 """
 
 
@@ -48,3 +49,12 @@ def test_dense_sources_and_long_chains_run_apart(rules):
                                                  (2**31, 2**31, True)])
 def test_long_groups_and_dense_sensors_are_recorded_apart(rules, longest, cells, apart):
     assert bool(rules.record_apart(longest, cells)) is apart
+
+
+@pytest.mark.parametrize("ctx,current,buf,aligned,kernel", [
+    (0, 0, 0, 1, True), (1, 1, 1, 1, True),
+    (0, 0, 0, 0, False), (0, 0, -1, 1, False),            # odd address, host memory
+    (0, 0, 1, 1, False), (1, 0, 1, 1, False),             # a buffer of another device, another device current
+    (0, 1, 1, 1, False), (1, 0, 0, 1, False)])            # both: the buffer's device is current, the context's is not
+def test_field_copies_take_the_kernel_on_the_contexts_own_device_only(rules, ctx, current, buf, aligned, kernel):
+    assert bool(rules.copy_by_kernel(ctx, current, buf, aligned)) is kernel
