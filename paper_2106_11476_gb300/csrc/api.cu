@@ -140,6 +140,23 @@ long long to_pitched(const fw2_ctx *c, long long flat) {
   return k * c->plane + j * c->pitch + i;
 }
 
+// Multiprocessors that work on the stream may use: fewer than the device's on
+// a stream of a green context.
+int sms_of_stream(cudaStream_t stream, int n_sm) {
+  using GetCtx = CUresult (*)(CUstream, CUcontext *);
+  using GetResource = CUresult (*)(CUcontext, CUdevResource *, CUdevResourceType);
+  void *gc = nullptr, *gr = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  CUcontext ctx;
+  CUdevResource r{};
+  if (cudaGetDriverEntryPointByVersion("cuStreamGetCtx", &gc, 12000, cudaEnableDefault, &q) != cudaSuccess || !gc ||
+      cudaGetDriverEntryPointByVersion("cuCtxGetDevResource", &gr, 12040, cudaEnableDefault, &q) != cudaSuccess || !gr ||
+      reinterpret_cast<GetCtx>(gc)(stream, &ctx) != CUDA_SUCCESS ||
+      reinterpret_cast<GetResource>(gr)(ctx, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS)
+    return n_sm;
+  return (int)r.sm.smCount;
+}
+
 double taps_abs_sum(const fw2_config &cfg) {
   double s = 0.0;
   for (int i = 0; i < 4; ++i) s += std::fabs(cfg.g[i]);
@@ -539,15 +556,6 @@ fw2_status enqueue_record(fw2_ctx *c, long long n) {
   return FW2_OK;
 }
 
-// Enqueue n_steps whole steps of a pipelined 2D context from step n: one
-// launch for all of them, then the last step's recording.
-fw2_status enqueue_steps2d(fw2_ctx *c, long long n, long long n_steps) {
-  CK(c, launch_steps2d(c->P, c->map_kind, c->n_sm, c->tm_vel, c->tm_prs, step_io(c), 2 * n, 2 * (n + n_steps),
-                       c->stream));
-  c->launches++;
-  return enqueue_record(c, n + n_steps - 1);
-}
-
 // Enqueue the launches of time step n (Sec. 3.1 order): velocity half step,
 // velocity sources (part 0), pressure half step, pressure sources,
 // recording (part 1); part -1 enqueues both, and only whole steps take part
@@ -643,6 +651,24 @@ fw2_status enqueue_step(fw2_ctx *c, long long n, int part = -1) {
       }
   }
   return FW2_OK;
+}
+
+// Enqueue n_steps whole steps of a pipelined 2D context from step n: one
+// launch for all of them, then the last step's recording; launches of half
+// steps from here on where the device cannot hold every block at once.
+fw2_status enqueue_steps2d(fw2_ctx *c, long long n, long long n_steps) {
+  const cudaError_t e = launch_steps2d(c->P, c->map_kind, c->n_sm, c->tm_vel, c->tm_prs, step_io(c), 2 * n,
+                                       2 * (n + n_steps), c->stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {
+    (void)cudaGetLastError();
+    c->half_launches = true;
+    fw2_status st = FW2_OK;
+    for (long long k = 0; k < n_steps && st == FW2_OK; ++k) st = enqueue_step(c, n + k);
+    return st;
+  }
+  CK(c, e);
+  c->launches++;
+  return enqueue_record(c, n + n_steps - 1);
 }
 
 // max |p| of the context (+inf when a value is not finite); synchronises the
@@ -844,6 +870,9 @@ fw2_status fw2_create(const fw2_config *cfg_in, fw2_ctx **out) {
     if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(c->stream);
     if (e2 != cudaSuccess) st = cuda_fail(c, e2, "state initialisation");
   }
+  // the blocks of a launch of many steps wait for one another: it needs the
+  // whole device, and half steps in launches of their own do not
+  c->half_launches = st == FW2_OK && c->nd == 2 && sms_of_stream(c->stream, c->n_sm) < c->n_sm;
   if (st != FW2_OK) {
     g_create_error = c->err;
     fw2_destroy(c);
@@ -1066,9 +1095,11 @@ fw2_status fw2_step(fw2_ctx *c, int64_t n_steps) {
   if ((st = finalize(c)) != FW2_OK) return st;
   if ((st = build_sources(c)) != FW2_OK) return st;
   for (int64_t s = 0; s < n_steps;) {
-    // many steps a launch, up to the next scan (per-launch timing, and while
-    // sources fire that have kernels of their own: one launch per half step)
-    const bool multi = c->pipe && c->nd == 2 && !c->profiling && !(c->src_apart && c->step < c->sig_steps);
+    // many steps a launch, up to the next scan (per-launch timing, sources
+    // with kernels of their own while they fire, and streams without the whole
+    // device: one launch per half step)
+    const bool multi = c->pipe && c->nd == 2 && !c->profiling && !c->half_launches &&
+                       !(c->src_apart && c->step < c->sig_steps);
     int64_t take = 1;
     if (multi) {
       // at most 2^28 cell-steps (about 11 ms) and 256 steps, so that work on

@@ -63,6 +63,7 @@ struct fw2_ctx {
   int map_kind = 0;  // FW2_MAP_*
   int device = 0;    // its memory and streams are this device's
   int n_sm = 152;    // multiprocessors of the device
+  bool half_launches = false;  // 2D: no launches of many steps (its blocks would not all be resident)
   bool pipe = false; // 2D half steps by the pipelined kernels
   fw2::PipeMaps tm_vel{}, tm_prs{};  // their tensor maps
   double dt = 0.0, cmax_eff = 0.0, cmax = 0.0;

@@ -82,3 +82,58 @@ def test_long_groups_and_dense_sensors_are_recorded_by_a_kernel_of_its_own(fw2, 
     # seven steps with trace rows for five: apart, a launch and the recording
     # a step, then one launch; inside, one launch whose last step has no row
     assert same(fw2, prob, 7) == (5 * 2 + 1 if apart else 1)
+
+
+class _GreenContext:
+    """A stream that may use some of the device's SMs only (driver API)."""
+
+    def __init__(self, sms):
+        import ctypes as C
+        import torch
+        torch.cuda.current_stream().synchronize()          # the primary context exists
+        self.C, self.cu = C, C.CDLL("libcuda.so.1")
+        whole, part = (C.c_char * 144)(), (C.c_char * 144)()   # CUdevResource; the SM count at byte 96
+        desc, self.ctx, self.ptr = C.c_void_p(), C.c_void_p(), C.c_void_p()
+        dev, one = C.c_int(torch.cuda.current_device()), C.c_uint(1)
+        self.call("cuDeviceGetDevResource", dev, whole, C.c_int(1))
+        self.call("cuDevSmResourceSplitByCount", part, C.byref(one), whole, None, C.c_uint(0), C.c_uint(sms))
+        self.sms = C.c_uint.from_buffer(part, 96).value
+        self.call("cuDevResourceGenerateDesc", C.byref(desc), part, C.c_uint(1))
+        self.call("cuGreenCtxCreate", C.byref(self.ctx), desc, dev, C.c_uint(1))
+        self.call("cuGreenCtxStreamCreate", C.byref(self.ptr), self.ctx, C.c_uint(1), C.c_int(0))
+        self.cuda_stream = self.ptr.value
+
+    def call(self, name, *args):
+        r = getattr(self.cu, name)(*args)
+        if r == 801:
+            pytest.skip("green contexts are not supported here")
+        assert r == 0, f"{name}: {r}"
+
+    def close(self):
+        self.call("cuStreamSynchronize", self.ptr)
+        self.call("cuStreamDestroy_v2", self.ptr)
+        self.call("cuGreenCtxDestroy", self.ctx)
+
+
+def test_stream_with_part_of_the_device_takes_half_steps_in_launches_of_their_own(fw2):
+    """The blocks of a launch of many steps wait for one another; on a stream
+    that holds some of the SMs they would not all be resident."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    prob = problem(600, 500)
+    prob.sources = sources(np.arange(0, 600 * 500, 977, dtype=np.int64), np.zeros(308, np.int32), 4, 1)
+    want, _ = run(fw2, prob, 6, "tile")
+    green = _GreenContext(sms // 2)
+    try:
+        assert 0 < green.sms < sms
+        sim = fw2.Simulation(prob, stream=green)
+        sim.set_state(synth.random_state(prob, seed=4))
+        before = sim.launches
+        sim.step(6)
+        assert sim.launches - before == 6 * 3               # two half steps and the recording a step
+        sim.synchronize()
+        for f, w in want.items():
+            np.testing.assert_array_equal(sim.trace.cpu().numpy() if f == "trace" else sim.field(f), w, err_msg=f)
+        sim.close()
+    finally:
+        green.close()
