@@ -73,6 +73,16 @@ __host__ __device__ constexpr int floats_of(int n) { return (n * (int)sizeof(T) 
 // shared-memory regions start on 128-byte boundaries (TMA destinations)
 __host__ __device__ constexpr int round32(int n) { return (n + 31) & ~31; }
 
+// The tensor maps that a 2D half step uses: both half steps' then fit in 4 KB
+// of kernel parameters.
+constexpr int kMaps2d = 10;
+struct StepMaps {
+  CUtensorMap m[kMaps2d];
+  explicit StepMaps(const PipeMaps &T) {
+    for (int i = 0; i < kMaps2d; ++i) m[i] = T.m[i];
+  }
+};
+
 // Work of one launch: the half tiles of the grid (tiles of 128 x 8 cells,
 // x fastest).
 struct Region {
@@ -171,8 +181,8 @@ __host__ __device__ constexpr unsigned stage_bytes(bool nl, bool nl_vel) {
 // and the maps; the second the stencil operand, which the neighbouring half
 // tiles of the previous half step wrote.  Boxes may reach outside the grid:
 // those cells read as zero.
-template <int N, typename Maps, bool VEL>
-__device__ __forceinline__ void issue_own(const StepParams &P, const PipeMaps &T, float *st, uint64_t *bar, int x0,
+template <int N, typename Maps, bool VEL, typename TM>
+__device__ __forceinline__ void issue_own(const StepParams &P, const TM &T, float *st, uint64_t *bar, int x0,
                                           int y0) {
   fence_proxy_async_smem();
   if (VEL) {
@@ -218,8 +228,8 @@ __device__ __forceinline__ void issue_own(const StepParams &P, const PipeMaps &T
     }
   }
 }
-template <int N, typename Maps, bool VEL>
-__device__ __forceinline__ void issue_operand(const PipeMaps &T, float *st, uint64_t *bar, int x0, int y0) {
+template <int N, typename Maps, bool VEL, typename TM>
+__device__ __forceinline__ void issue_operand(const TM &T, float *st, uint64_t *bar, int x0, int y0) {
   if (VEL) {
     tma_load_2d(st, &T.m[0], x0 - 4, y0 - 3, bar);
   } else {
@@ -227,8 +237,8 @@ __device__ __forceinline__ void issue_operand(const PipeMaps &T, float *st, uint
     tma_load_2d(st + PrsStage<N, Maps>::kX, &T.m[1], x0 - 4, y0 - 4, bar);
   }
 }
-template <int N, typename Maps, bool VEL>
-__device__ __forceinline__ void issue_stage(const StepParams &P, const PipeMaps &T, float *st, uint64_t *bar,
+template <int N, typename Maps, bool VEL, typename TM>
+__device__ __forceinline__ void issue_stage(const StepParams &P, const TM &T, float *st, uint64_t *bar,
                                             int x0, int y0) {
   mbar_arrive_expect_tx(bar, stage_bytes<N, Maps, VEL>(P.nl != 0, P.nl_vel != 0));
   issue_own<N, Maps, VEL>(P, T, st, bar, x0, y0);
@@ -238,8 +248,8 @@ __device__ __forceinline__ void issue_stage(const StepParams &P, const PipeMaps 
 // Store the updated arrays of a half tile from its stage (one thread, after
 // every thread's fence and a barrier): velocity v_x, v_y, psi1_x, psi1_y;
 // pressure p, psi2_x, psi2_y.  The copies write nothing outside the grid.
-template <int N, typename Maps, bool VEL>
-__device__ __forceinline__ void store_stage(const PipeMaps &T, const float *st, int x0, int y0) {
+template <int N, typename Maps, bool VEL, typename TM>
+__device__ __forceinline__ void store_stage(const TM &T, const float *st, int x0, int y0) {
   if (VEL) {
     using S = VelStage<N, Maps>;
     const float *ss = st + S::kP + S::kR;
@@ -834,9 +844,8 @@ struct SourceBits {
     return round >= 32 * kSrcWords || ((w[half][round >> 5] >> (round & 31)) & 1u);
   }
 };
+// Set the bits (computing threads), once they are zero.
 __device__ __forceinline__ void mark_sources(const StepIO &io, const Region &R, int per, SourceBits &bits, int tid) {
-  for (int i = tid; i < 2 * kSrcWords; i += kThreads) (&bits.w[0][0])[i] = 0u;
-  __syncthreads();
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
     const int *unit = io.src[f].unit;
@@ -933,8 +942,8 @@ __device__ __forceinline__ void record_row(const StepIO &io, const float *p, lon
 // 681 at 4096^2 (655).
 template <int N, typename Maps>
 __global__ void __launch_bounds__(kStepThreads, 1)
-    steps2d_kernel(const StepParams P, const Region R, const __grid_constant__ PipeMaps TV,
-                   const __grid_constant__ PipeMaps TP, const StepIO io, const long long ph0, const long long ph1) {
+    steps2d_kernel(const StepParams P, const Region R, const __grid_constant__ StepMaps TV,
+                   const __grid_constant__ StepMaps TP, const StepIO io, const long long ph0, const long long ph1) {
   using G = StepRing<N, Maps>;
   constexpr int kS = G::kStages, kStage = G::kStage;
   extern __shared__ __align__(128) float smem_raw[];
@@ -946,7 +955,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   float *smem = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   float *tab = smem + kS * kStage;
   const int tid = threadIdx.y * 32 + threadIdx.x;
-  if (tid < kThreads) stage_table<N, Maps>(P, tab, tid);  // made visible by the barrier below
+  for (int i = tid; i < 2 * kSrcWords; i += kStepThreads) (&sources.w[0][0])[i] = 0u;
   if (tid == 0) {
     for (int q = 0; q < kS; ++q) {
       mbar_init(&full[q], 1);
@@ -961,7 +970,6 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   const int grid = (int)gridDim.x;
   const int per = R.rounds(blockIdx.x, grid);
   const int last_slot = R.slot(per - 1, blockIdx.x, grid);
-  mark_sources(io, R, per, sources, tid);
   __syncthreads();
   if (blocked) return;
   // Walk over the jobs (phase, half tile): rounds upwards in velocity phases,
@@ -1103,6 +1111,17 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   }
 
   // ------------------------------------------------------------- compute ---
+  // The first half tiles are being copied meanwhile; the copying warp looks at
+  // the marks after every computing warp's first arrival only.  With both ahead
+  // of the copies, and the parameters above 4 KB, the two half steps of a step
+  // in launches of their own took 16.6 us at 250 x 186 (N = 4, float; 14.7
+  // now), 20.7 at 640 x 640 (N = 2; 18.5), 36.3 at 512 x 512 of the uint16
+  // index with 1160 tissues (33.0).
+  mark_sources(io, R, per, sources, tid);
+  if constexpr (Form<Maps>::kIdx) {
+    stage_table<N, Maps>(P, tab, tid);
+    asm volatile("bar.sync 1, %0;\n" ::"n"(kThreads) : "memory");
+  }
   Walk w = start();
 #pragma unroll 1
   while (true) {
@@ -1281,9 +1300,12 @@ cudaError_t pipe_batched_dispatch(const StepParams *Ps, const PipeMaps *Ts, cons
 }
 
 template <int N, typename Maps>
-cudaError_t steps_launch(const StepParams &P, const Region &R, int grid, const PipeMaps &TV, const PipeMaps &TP,
+cudaError_t steps_launch(const StepParams &P, const Region &R, int grid, const PipeMaps &vel, const PipeMaps &prs,
                          const StepIO &io, long long ph0, long long ph1, cudaStream_t st) {
   constexpr size_t bytes = StepRing<N, Maps>::kBytes;
+  static_assert(sizeof(StepParams) + sizeof(Region) + 2 * sizeof(StepMaps) + sizeof(StepIO) + 128 <= 4096,
+                "kernel parameters");
+  const StepMaps TV(vel), TP(prs);
   cudaError_t e = cudaFuncSetAttribute(steps2d_kernel<N, Maps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   const dim3 block(32, kStepThreads / 32);

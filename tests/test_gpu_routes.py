@@ -137,3 +137,32 @@ def test_stream_with_part_of_the_device_takes_half_steps_in_launches_of_their_ow
         sim.close()
     finally:
         green.close()
+
+
+@pytest.mark.parametrize("maps", ["f32", "idx", "idx16"])
+def test_half_steps_in_launches_of_their_own_with_sources_in_the_first_half_tiles(fw2, maps):
+    """A launch copies its first half tiles while it looks up which of them
+    hold sources and stages the index table: sources in every block's first
+    and last half tile, one half step a launch, against the tile kernels."""
+    prob = synth.indexed_abdominal_problem(nx=390, ny=1000, n_steps=12, n_elements=8, nl="literal", levels=64)
+    if maps == "f32":
+        prob = synth.abdominal_problem(n=256, n_steps=12, seed=3)
+    elif maps == "idx16":
+        prob.tissue = prob.tissue.astype(np.uint16)
+    nx, ny = prob.shape
+    cells = np.concatenate([np.arange(0, nx * ny, 1024), nx * ny - 1 - np.arange(40)]).astype(np.int64)
+    prob.sources = [synth.Source(k, cells, np.zeros(cells.size, np.int32), a * np.ones((12, 1), np.float32))
+                    for k, a in (("p", 10.0), ("vx", 1e-5), ("vy", 1e-5))]
+    out = []
+    for path in ("tile", "auto"):
+        sim = fw2.Simulation(prob, map_precision=maps, kernel_path=path)
+        for _ in range(12):
+            fw2.fw2_step_part(sim.ctx, 0)
+            fw2.fw2_step_part(sim.ctx, 1)
+        sim.synchronize()
+        assert fw2.fw2_kernel_path(sim.ctx) == ("tile" if path == "tile" else "pipe")
+        out.append({f: sim.field(f) for f in ("p", "vx", "vy", "psi1x", "psi2y")})
+        sim.close()
+    assert np.abs(out[0]["p"]).max() > 0
+    for f, w in out[0].items():
+        np.testing.assert_array_equal(out[1][f], w, err_msg=f)
