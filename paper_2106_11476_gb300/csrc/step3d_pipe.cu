@@ -525,23 +525,42 @@ __device__ __forceinline__ Face3 face3(const StepParams &P, const MT *rb, int x0
                at(pz, r0, c0), at(pz, r0, c1)};
 }
 
+// Arithmetic on the two cells of a thread: packed instructions or one cell at a
+// time; both round alike.
+template <bool PACKED>
+struct Two {
+  static __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) {
+    return PACKED ? fma2(a, b, c) : make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+  }
+  static __device__ __forceinline__ float2 mul(float2 a, float2 b) {
+    return PACKED ? mul2(a, b) : make_float2(a.x * b.x, a.y * b.y);
+  }
+  static __device__ __forceinline__ float2 add(float2 a, float2 b) {
+    return PACKED ? add2(a, b) : make_float2(a.x + b.x, a.y + b.y);
+  }
+  static __device__ __forceinline__ float2 sub(float2 a, float2 b) {
+    return PACKED ? sub2(a, b) : make_float2(a.x - b.x, a.y - b.y);
+  }
+};
+
 // The memory-variable update of mechanism nu on the three axes and its
 // contribution to the stretched derivatives (Eqs. relaxation4,
 // relaxation_psi), writing psi back; A[a], B[a] are the coefficients of
 // axis a, q[a] its memory variable before the update.
+template <bool PK>
 __device__ __forceinline__ void relax3(const StepParams &P, float *const *psi, long long o, int i0, bool edge,
                                        const float2 (&q)[3], const float2 (&A)[3], const float2 (&B)[3],
                                        const float2 (&D)[3], float2 (&S)[3]) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    float2 n = fma2(B[a], q[a], mul2(A[a], D[a]));
-    S[a] = add2(S[a], fma2(dup2(P.w_new), n, mul2(dup2(P.w_old), q[a])));
+    float2 n = Two<PK>::fma(B[a], q[a], Two<PK>::mul(A[a], D[a]));
+    S[a] = Two<PK>::add(S[a], Two<PK>::fma(dup2(P.w_new), n, Two<PK>::mul(dup2(P.w_old), q[a])));
     if (edge) n = mask_pad2(n, i0, P.nx);
     st_state2(psi[a], o, n);
   }
 }
 
-template <int N, bool EDGE, bool CROSS, bool PS, typename MT>
+template <int N, bool EDGE, bool CROSS, bool PS, typename MT, bool PK>
 __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 &R, float *st, const float *ring,
                                              int x0, int y0, int k, int tid, const Psi<N> &q) {
   using S = Vel3<N, PS, MT>;
@@ -572,17 +591,17 @@ __device__ __forceinline__ void vel3_compute(const StepParams &P, const Region3 
     float2 col[8];
 #pragma unroll
     for (int m = 0; m < 8; ++m) col[m] = sld2(sp + (sy - 3 + m) * kCW + lx + 4);
-D[1] = make_float2(0.f, 0.f);
+    D[1] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int m = 1; m <= 4; ++m) D[1] = fma2(dup2(P.gh[m - 1]), sub2(col[3 + m], col[4 - m]), D[1]);
+    for (int m = 1; m <= 4; ++m) D[1] = Two<PK>::fma(dup2(P.gh[m - 1]), Two<PK>::sub(col[3 + m], col[4 - m]), D[1]);
   }
   {
     float2 zc[8];
 #pragma unroll
     for (int m = 0; m < 8; ++m) zc[m] = sld2(ring + slot_after(s0, m) * kPl + sy * kCW + lx + 4);
-D[2] = make_float2(0.f, 0.f);
+    D[2] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int m = 1; m <= 4; ++m) D[2] = fma2(dup2(P.gh[m - 1]), sub2(zc[3 + m], zc[4 - m]), D[2]);
+    for (int m = 1; m <= 4; ++m) D[2] = Two<PK>::fma(dup2(P.gh[m - 1]), Two<PK>::sub(zc[3 + m], zc[4 - m]), D[2]);
   }
   if (CROSS) {
     // cross taps (Sec. 3.1) over both transverse axes, in the order of the
@@ -607,7 +626,7 @@ D[2] = make_float2(0.f, 0.f);
   float2 v0 = sld2(st + S::oV + o), v1 = sld2(st + S::oV + kArr + o), v2 = sld2(st + S::oV + 2 * kArr + o);
   float2 Sd[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) Sd[a] = mul2(D[a], k1);
+  for (int a = 0; a < 3; ++a) Sd[a] = Two<PK>::mul(D[a], k1);
   const int xside = EDGE ? R.xs_side(x0) : -1;
   const bool ys = EDGE && R.ys_row(y0) != INT_MIN, zs = EDGE && R.zs_plane(k) >= 0;
   // coefficients of every mechanism and axis first, C-PML strips included,
@@ -630,7 +649,7 @@ D[2] = make_float2(0.f, 0.f);
     float2 qq[3];
 #pragma unroll
     for (int a3 = 0; a3 < 3; ++a3) qq[a3] = PS ? sld2(st + S::oPsi + (a3 * N + nu) * kArr + o) : q[a3][nu];
-    relax3(P, P.psi1, nu * Sn + c, i0, EDGE, qq, A[nu], B[nu], D, Sd);
+    relax3<PK>(P, P.psi1, nu * Sn + c, i0, EDGE, qq, A[nu], B[nu], D, Sd);
   }
   const Face3 f = face3<EDGE, MT>(P, reinterpret_cast<const MT *>(st + S::oRho), x0, y0, k, lx, ly);
   const float rr[3] = {f.r0, f.r1, f.r2}, ru[2] = {f.u0, f.u1}, rz[2] = {f.z0, f.z1};
@@ -671,7 +690,7 @@ D[2] = make_float2(0.f, 0.f);
   st_state2(P.v[2], c, v2);
 }
 
-template <int N, bool EDGE, bool CROSS, bool PS, typename MT>
+template <int N, bool EDGE, bool CROSS, bool PS, typename MT, bool PK>
 __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 &R, const float *st, const float *ring,
                                              const float *sub, int x0, int y0, int k, int tid, const Psi<N> &q) {
   using S = Prs3<N, CROSS, PS, MT>;
@@ -704,9 +723,9 @@ __device__ __forceinline__ void prs3_compute(const StepParams &P, const Region3 
     for (int m = 0; m < 8; ++m)
       col[m] = CROSS ? sld2(suby + sub_slot(k) * S::kYPlane + (ly + m) * kCW + lx + 4)
                      : sld2(st + S::oVy + (ly + m) * kTX + lx);
-D[1] = make_float2(0.f, 0.f);
+    D[1] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int m = 1; m <= 4; ++m) D[1] = fma2(dup2(P.gh[m - 1]), sub2(col[4 + m - 1], col[4 - m]), D[1]);
+    for (int m = 1; m <= 4; ++m) D[1] = Two<PK>::fma(dup2(P.gh[m - 1]), Two<PK>::sub(col[4 + m - 1], col[4 - m]), D[1]);
   }
   {
     // v_z planes k-4 .. k+3 of the ring
@@ -715,9 +734,9 @@ D[1] = make_float2(0.f, 0.f);
     for (int m = 0; m < 8; ++m)
       zc[m] = CROSS ? sld2(ring + slot_after(s0, m) * kPl + (ly + 1) * kCW + lx + 4)
                     : sld2(ring + slot_after(s0, m) * kPl + o);
-D[2] = make_float2(0.f, 0.f);
+    D[2] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int m = 1; m <= 4; ++m) D[2] = fma2(dup2(P.gh[m - 1]), sub2(zc[4 + m - 1], zc[4 - m]), D[2]);
+    for (int m = 1; m <= 4; ++m) D[2] = Two<PK>::fma(dup2(P.gh[m - 1]), Two<PK>::sub(zc[4 + m - 1], zc[4 - m]), D[2]);
   }
   if (CROSS) {
     // cross taps (Sec. 3.1) at the centres, in the order of the tile
@@ -761,7 +780,7 @@ D[2] = make_float2(0.f, 0.f);
   float2 p = sld2(st + S::oP + o);
   float2 Sd[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) Sd[a] = mul2(D[a], k2);
+  for (int a = 0; a < 3; ++a) Sd[a] = Two<PK>::mul(D[a], k2);
   const int xside = EDGE ? R.xs_side(x0) : -1;
   const bool ys = EDGE && R.ys_row(y0) != INT_MIN, zs = EDGE && R.zs_plane(k) >= 0;
   // coefficients of every mechanism and axis first, C-PML strips included,
@@ -784,7 +803,7 @@ D[2] = make_float2(0.f, 0.f);
     float2 qq[3];
 #pragma unroll
     for (int a3 = 0; a3 < 3; ++a3) qq[a3] = PS ? sld2(st + S::oPsi + (a3 * N + nu) * kArr + o) : q[a3][nu];
-    relax3(P, P.psi2, nu * Sn + c, i0, EDGE, qq, A[nu], B[nu], D, Sd);
+    relax3<PK>(P, P.psi2, nu * Sn + c, i0, EDGE, qq, A[nu], B[nu], D, Sd);
   }
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
@@ -885,11 +904,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (more) psi_of(nx0, ny0, nk, qn);
     float *cur = smem + s * kStage;
     if (R.interior(x0, y0, k)) {
-      if (VEL) vel3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, x0, y0, k, tid, qc);
-      else prs3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, sub, x0, y0, k, tid, qc);
+      if (VEL) vel3_compute<N, false, CROSS, PS, MT, true>(P, R, cur, ring, x0, y0, k, tid, qc);
+      else prs3_compute<N, false, CROSS, PS, MT, true>(P, R, cur, ring, sub, x0, y0, k, tid, qc);
     } else {
-      if (VEL) vel3_compute<N, true, CROSS, PS, MT>(P, R, cur, ring, x0, y0, k, tid, qc);
-      else prs3_compute<N, true, CROSS, PS, MT>(P, R, cur, ring, sub, x0, y0, k, tid, qc);
+      if (VEL) vel3_compute<N, true, CROSS, PS, MT, true>(P, R, cur, ring, x0, y0, k, tid, qc);
+      else prs3_compute<N, true, CROSS, PS, MT, true>(P, R, cur, ring, sub, x0, y0, k, tid, qc);
     }
     if (!more) break;
     if (fresh) {  // a new column: all ring planes, once every thread is done with the rings
@@ -1013,11 +1032,11 @@ __global__ void __launch_bounds__(kThreads + 32, 1)
     const bool more = advance(nu);
     float *cur = smem + u.stage() * kStage;
     if (R.interior(u.x0, u.y0, u.k)) {
-      if (VEL) vel3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, u.x0, u.y0, u.k, tid, q);
-      else prs3_compute<N, false, CROSS, PS, MT>(P, R, cur, ring, nullptr, u.x0, u.y0, u.k, tid, q);
+      if (VEL) vel3_compute<N, false, CROSS, PS, MT, true>(P, R, cur, ring, u.x0, u.y0, u.k, tid, q);
+      else prs3_compute<N, false, CROSS, PS, MT, true>(P, R, cur, ring, nullptr, u.x0, u.y0, u.k, tid, q);
     } else {
-      if (VEL) vel3_compute<N, true, CROSS, PS, MT>(P, R, cur, ring, u.x0, u.y0, u.k, tid, q);
-      else prs3_compute<N, true, CROSS, PS, MT>(P, R, cur, ring, nullptr, u.x0, u.y0, u.k, tid, q);
+      if (VEL) vel3_compute<N, true, CROSS, PS, MT, true>(P, R, cur, ring, u.x0, u.y0, u.k, tid, q);
+      else prs3_compute<N, true, CROSS, PS, MT, true>(P, R, cur, ring, nullptr, u.x0, u.y0, u.k, tid, q);
     }
     __syncwarp();
     if ((tid & 31) == 0) mbar_arrive(&done[u.stage()]);
@@ -1041,6 +1060,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     pipe3d_batched_kernel(const StepParams *Ps, const Region3 *Rs, const PipeMaps *Ts, const int2 *items,
                           const int *runs) {
   using G = Ring3<N, VEL, CROSS, PS, bf16>;
+  // The register layout with three mechanisms spills here, and with packed
+  // arithmetic more in the literal system's velocity and the cross taps'
+  // pressure half step.  130 x 120 x 110, 200 x 160 x 120 and 96^3 in one
+  // batch, us a step packed throughout and as chosen: literal 825 and 819,
+  // cross taps 1002 and 982, both 1020 and 1008 (one cell at a time
+  // throughout: 820, 1009 and 1026)
+  constexpr bool kPk = N < 3 || PS || (VEL && CROSS);
   constexpr int kStage = G::kStage;
   extern __shared__ __align__(128) float smem_raw[];
   __shared__ __align__(8) uint64_t bar[2];
@@ -1136,11 +1162,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!PS && more) psi_of(nctx == ctx ? sP : Ps[nctx], nx0, ny0, nk, qn);
     float *cur = smem + s * kStage;
     if (sR.interior(x0, y0, k)) {
-      if (VEL) vel3_compute<N, false, CROSS, PS, bf16>(sP, sR, cur, ring, x0, y0, k, tid, qc);
-      else prs3_compute<N, false, CROSS, PS, bf16>(sP, sR, cur, ring, sub, x0, y0, k, tid, qc);
+      if (VEL) vel3_compute<N, false, CROSS, PS, bf16, kPk>(sP, sR, cur, ring, x0, y0, k, tid, qc);
+      else prs3_compute<N, false, CROSS, PS, bf16, kPk>(sP, sR, cur, ring, sub, x0, y0, k, tid, qc);
     } else {
-      if (VEL) vel3_compute<N, true, CROSS, PS, bf16>(sP, sR, cur, ring, x0, y0, k, tid, qc);
-      else prs3_compute<N, true, CROSS, PS, bf16>(sP, sR, cur, ring, sub, x0, y0, k, tid, qc);
+      if (VEL) vel3_compute<N, true, CROSS, PS, bf16, kPk>(sP, sR, cur, ring, x0, y0, k, tid, qc);
+      else prs3_compute<N, true, CROSS, PS, bf16, kPk>(sP, sR, cur, ring, sub, x0, y0, k, tid, qc);
     }
     if (!more) break;
     if (fresh) {  // a new item: every thread is done with the rings (and the context's parameters)

@@ -166,3 +166,37 @@ def test_half_steps_in_launches_of_their_own_with_sources_in_the_first_half_tile
     assert np.abs(out[0]["p"]).max() > 0
     for f, w in out[0].items():
         np.testing.assert_array_equal(out[1][f], w, err_msg=f)
+
+
+@pytest.mark.parametrize("N,nl,taps", [(3, "literal", False), (3, "pressure", True), (3, "literal", True), (2, "literal", True)])
+def test_3d_batches_equal_their_contexts_alone_in_every_arithmetic_form(fw2, N, nl, taps):
+    """The batched half steps of the register layout, two cells at a time or
+    one, give the bits of the contexts stepped alone."""
+    def sims():
+        out = []
+        for i, shape in enumerate(((140, 40, 24), (70, 33, 41))):
+            prob = synth.homogeneous(shape, 1e-4, 0.0, relax=synth.relaxation_sets()[{2: "N2_y1.0_a0.5", 3: "N3_y1.2_brain"}[N]],
+                                     beta=4.0)
+            prob.c = (1500 + 100 * np.random.default_rng(i).random(prob.grid_shape)).astype(np.float32)
+            prob.nl_mode, prob.dt = nl, 0.2 * 1e-4 / 2200.0
+            prob.pml_transition, prob.pml_bound = 6, 2
+            if taps:
+                prob.taps = tuple(fw2.fw2_taps_time_space(0.25, 3))
+            sim = fw2.Simulation(prob, map_precision="bf16")
+            sim.set_state(synth.random_state(prob, seed=i))
+            out.append(sim)
+        return out
+    alone, joined = sims(), sims()
+    batch = fw2.fw2_batch_create([s.ctx for s in joined])
+    fw2.fw2_batch_step(batch, 8)
+    fw2.fw2_batch_synchronize(batch)
+    for a, b in zip(alone, joined):
+        a.step(8)
+        a.synchronize()
+        for f in ("p", "vx", "vz", "psi1x", "psi1z", "psi2y"):
+            want = a.field(f)
+            assert np.isfinite(want).all() and np.abs(want).max() > 0
+            np.testing.assert_array_equal(b.field(f), want, err_msg=f)
+    fw2.fw2_batch_destroy(batch)
+    for s in alone + joined:
+        s.close()
