@@ -483,6 +483,19 @@ fw2_status fw2_taps_time_space(double r, int32_t ndim, double *g);
  * 0 otherwise.  Synchronous on the default stream; needs no context.  Errors:
  * FW2_EINVAL (null pointer, limit out of range), FW2_ECUDA. */
 fw2_status fw2_selftest_bounded_wait(int64_t limit_ns, int32_t *timed_out);
+/* Self-test of the grid barrier of the launches of many steps (the paper has
+ * no counterpart).  Launches one block that passes a barrier by itself and
+ * then waits, at most limit_ns nanoseconds (1 .. 10^10), for one that another
+ * block would have to reach; status_set != 0: with the status word set, as
+ * after another block's wait gave up, which ends the wait at once.  *timed_out
+ * (host) becomes 1 when the first wait returned and the second gave up, as
+ * they must, and 0 otherwise.  Synchronous on the default stream.  Errors:
+ * FW2_EINVAL (null pointer, limit out of range), FW2_ECUDA. */
+fw2_status fw2_selftest_grid_barrier(int64_t limit_ns, int32_t status_set, int32_t *timed_out);
+/* For tests of what follows a wait that gave up: leaves the context as such a
+ * launch does, its status word set and its barrier counter short of a whole
+ * barrier (stream-ordered).  Errors: FW2_EINVAL (ctx NULL), FW2_ECUDA. */
+fw2_status fw2_selftest_abandon(fw2_ctx *ctx);
 /* Kernel path the context's half steps take, resolved once the coefficients
  * are built (first fw2_step): FW2_PATH_TILE or FW2_PATH_PIPE; FW2_PATH_AUTO
  * before the first step. */

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "ctx.h"
+#include "async.cuh"
 #include "routes.h"
 
 using namespace fw2;
@@ -738,6 +739,28 @@ fw2_status fw2_selftest_bounded_wait(int64_t limit_ns, int32_t *timed_out) {
   if (d) cudaFree(d);
   if (e != cudaSuccess) return fail(nullptr, FW2_ECUDA, "bounded-wait self-test: %s", cudaGetErrorString(e));
   *timed_out = h;
+  return FW2_OK;
+}
+
+fw2_status fw2_selftest_grid_barrier(int64_t limit_ns, int32_t status_set, int32_t *timed_out) {
+  if (!timed_out || limit_ns < 1 || limit_ns > 10000000000ll)
+    return fail(nullptr, FW2_EINVAL, "timed_out is required and limit_ns must lie in [1, 1e10]");
+  // barrier counter (as after 7 barriers), status word, result
+  unsigned long long h[2] = {7ull, status_set ? (unsigned long long)kStatusWaitTimeout : 0ull}, *d = nullptr;
+  cudaError_t e = cudaMalloc(&d, sizeof h);
+  if (e == cudaSuccess) e = cudaMemcpy(d, h, sizeof h, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = launch_grid_barrier_selftest((unsigned long long)limit_ns, d);
+  if (e == cudaSuccess) e = cudaMemcpy(h, d, sizeof h, cudaMemcpyDeviceToHost);
+  if (d) cudaFree(d);
+  if (e != cudaSuccess) return fail(nullptr, FW2_ECUDA, "grid barrier self-test: %s", cudaGetErrorString(e));
+  *timed_out = (int32_t)(h[1] >> 32);
+  return FW2_OK;
+}
+
+fw2_status fw2_selftest_abandon(fw2_ctx *c) {
+  if (!c) return FW2_EINVAL;
+  CK(c, cudaMemsetAsync(c->d_status, kStatusWaitTimeout, 1, c->stream));
+  CK(c, cudaMemsetAsync(c->d_sync, 1, 1, c->stream));
   return FW2_OK;
 }
 

@@ -139,7 +139,22 @@ __global__ void bounded_wait_kernel(unsigned long long limit_ns, int *timed_out)
   fence_mbarrier_init();
   *timed_out = mbar_wait_bounded(&bar, 0, limit_ns) ? 0 : 1;
 }
+// one block: a barrier that it completes, then one that it does not
+__global__ void grid_barrier_kernel(unsigned long long limit_ns, unsigned long long *words) {
+  unsigned int *status = reinterpret_cast<unsigned int *>(words + 1);
+  GridBarrier gb;
+  gb.init(words);
+  gb.arrive();
+  const bool passed = gb.wait(nullptr, limit_ns);
+  gb.target += gridDim.x;
+  status[1] = passed && !gb.wait(status, limit_ns) ? 1 : 0;
+}
 }  // namespace
+
+cudaError_t launch_grid_barrier_selftest(unsigned long long limit_ns, unsigned long long *words) {
+  grid_barrier_kernel<<<1, 1>>>(limit_ns, words);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_bounded_wait_selftest(unsigned long long limit_ns, int *timed_out) {
   bounded_wait_kernel<<<1, 1>>>(limit_ns, timed_out);

@@ -77,5 +77,7 @@ cudaError_t launch_absmax(const float *f, int nx, int pitch, long long rows,
 // one block waits on an mbarrier that never completes, with the bounded wait
 // of the pipelined kernels; *timed_out (device) = 1 when it gave up
 cudaError_t launch_bounded_wait_selftest(unsigned long long limit_ns, int *timed_out);
+// words (device): the barrier counter (64 bits), the status word, the result
+cudaError_t launch_grid_barrier_selftest(unsigned long long limit_ns, unsigned long long *words);
 
 }  // namespace fw2

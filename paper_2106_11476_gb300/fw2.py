@@ -104,6 +104,8 @@ EXPORTS = {
     "fw2_field_absmax_noalloc": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_int64, C.c_void_p,
                                            C.c_void_p]),
     "fw2_selftest_bounded_wait": (C.c_int, [C.c_int64, C.POINTER(C.c_int32)]),
+    "fw2_selftest_grid_barrier": (C.c_int, [C.c_int64, C.c_int32, C.POINTER(C.c_int32)]),
+    "fw2_selftest_abandon": (C.c_int, [C.c_void_p]),
     "fw2_kernel_path": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32)]),
     "fw2_pipe_layout": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "fw2_taps_time_space": (C.c_int, [C.c_double, C.c_int32, C.POINTER(C.c_double)]),
@@ -494,6 +496,20 @@ def fw2_selftest_bounded_wait(limit_ns: int) -> bool:
     t = C.c_int32(-1)
     _check(lib().fw2_selftest_bounded_wait(int(limit_ns), C.byref(t)))
     return bool(t.value)
+
+
+def fw2_selftest_grid_barrier(limit_ns: int, status_set: bool = False) -> bool:
+    """True when a wait for a block that never reaches the grid barrier gave up
+    (fw2_selftest_grid_barrier)."""
+    t = C.c_int32(-1)
+    _check(lib().fw2_selftest_grid_barrier(int(limit_ns), int(status_set), C.byref(t)))
+    return bool(t.value)
+
+
+def fw2_selftest_abandon(ctx):
+    """Leave the context as after a device-side wait that gave up
+    (fw2_selftest_abandon)."""
+    _check(lib().fw2_selftest_abandon(ctx), ctx)
 
 
 def fw2_field_absmax_noalloc(field, row_len: int, n_rows: int, row_pitch: int, out, stream=None) -> int:
