@@ -1404,7 +1404,8 @@ cudaError_t build_pipe3d_maps(const StepParams &P, PipeMaps *vel, PipeMaps *prs,
     ok = ok && encode_tensor_map(&prs->m[10], P.sa2[0], es, 4, dxs, sxs, bxs);
     ok = ok && encode_tensor_map(&prs->m[11], P.sb2[0], es, 4, dxs, sxs, bxs);
   }
-  if (y_strip_staged(P)) {  // y strips [N][z][2L][x], boxes 128 x 8 x 1 x N
+  // (float maps: read per cell)
+  if (P.map_kind == 1 && y_strip_staged(P)) {  // y strips [N][z][2L][x], boxes 128 x 8 x 1 x N
     const ull L = (ull)P.L[1];
     const ull dys[4] = {nx, 2 * L, nz, (ull)N},
               sys[3] = {(ull)P.pitch * es, 2 * L * (ull)P.pitch * es, (ull)P.strip_nu[1] * es};
@@ -1413,7 +1414,7 @@ cudaError_t build_pipe3d_maps(const StepParams &P, PipeMaps *vel, PipeMaps *prs,
     ok = ok && encode_tensor_map(&prs->m[13], P.sa2[1], es, 4, dys, sys, ab4);
     ok = ok && encode_tensor_map(&prs->m[14], P.sb2[1], es, 4, dys, sys, ab4);
   }
-  if (z_strip_staged(P)) {  // z strips [N][2L][y][x], boxes 128 x 8 x 1 x N
+  if (P.map_kind == 1 && z_strip_staged(P)) {  // z strips [N][2L][y][x], boxes 128 x 8 x 1 x N
     const ull L = (ull)P.L[2];
     const ull dzs[4] = {nx, ny, 2 * L, (ull)N},
               szs[3] = {(ull)P.pitch * es, ny * (ull)P.pitch * es, (ull)P.strip_nu[2] * es};
