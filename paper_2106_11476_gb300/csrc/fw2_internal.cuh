@@ -207,25 +207,26 @@ cudaError_t launch_pipe2d_batched(bool vel, const StepParams *Ps, const PipeMaps
                                   int n_units, const int *runs, int n_relax, int map_kind, int grid,
                                   cudaStream_t s);
 // persistent pipelined 3D half step (bf16 or float maps, N <= 3, no periodic
-// axis); float maps take the register layout, bf16 maps one of two layouts that compute the same result: the memory variables
-// staged in shared memory with the other arrays (kLayoutStaged; not with
-// cross taps, nor for the literal system's velocity half step), or loaded
-// into registers one unit ahead with every C-PML strip staged
-// (kLayoutRegisters); kLayoutDefault takes the staged one where it applies
+// axis); float maps take the register layout, bf16 maps one of two layouts
+// that compute the same result: the memory variables staged in shared memory
+// with the other arrays (kLayoutStaged; not with cross taps, nor for the
+// literal system's velocity half step), or loaded into registers one unit
+// ahead with every C-PML strip staged (kLayoutRegisters); kLayoutDefault takes
+// the staged one where it applies
 constexpr int kLayoutDefault = 0, kLayoutStaged = 1, kLayoutRegisters = 2;
 bool pipe3d_supported(const StepParams &P, int map_kind);
 bool pipe3d_layout_allowed(bool vel, const StepParams &P, int layout);
 cudaError_t build_pipe3d_maps(const StepParams &P, PipeMaps *vel, PipeMaps *prs, const char **why);
 cudaError_t launch_pipe3d(bool vel, const StepParams &P, int grid, const PipeMaps &T, cudaStream_t s,
                           int layout = kLayoutDefault);
+// the kernels for float maps (a second compilation of the file); region: a Region3
+cudaError_t launch_pipe3d_float(bool vel, const StepParams &P, const void *region, int grid, const PipeMaps &T,
+                                cudaStream_t s);
 // batched form: per context the parameters, the work layout (an opaque
 // record of pipe3d_region_bytes(), written by pipe3d_region, which returns
 // the context's item count) and the tensor maps, in device memory; items
 // {context, item}; the layout of every context is the default one
 // (pipe3d_staged_layout), which must agree within a launch
-// the kernels for float maps (a second compilation of the file); region: a Region3
-cudaError_t launch_pipe3d_float(bool vel, const StepParams &P, const void *region, int grid, const PipeMaps &T,
-                                cudaStream_t s);
 size_t pipe3d_region_bytes();
 long long pipe3d_region(const StepParams &P, int grid, bool vel, void *out);
 // edge units of each of the context's items (n_edge) and units per item

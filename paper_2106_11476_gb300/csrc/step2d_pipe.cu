@@ -280,33 +280,11 @@ constexpr int kThreads = 512;
 constexpr int kStepThreads = kThreads + 32;  // and the warp that copies and stores (steps2d_kernel)
 
 __device__ __forceinline__ float2 sld2(const float *s) { return *reinterpret_cast<const float2 *>(s); }
-__device__ __forceinline__ void st_state2(float *p, long long i, float2 v) {
-  __stcs(reinterpret_cast<float2 *>(p + i), v);
-}
-// zero the cells of a pair that fall in the row padding (x >= nx)
-__device__ __forceinline__ float2 mask_pad2(float2 v, int i0, int nx) {
-  if (i0 + 1 >= nx) v.y = 0.f;
-  if (i0 >= nx) v.x = 0.f;
-  return v;
-}
-// Results leave through the stage and TMA tensor stores (fewer store
-// instructions than per-thread stores; the store of a unit overlaps the
-// compute of the next).
-template <typename Maps>
-struct TmaStore {
-  static constexpr bool value = true;
-};
-// one result pair of array `a` (stage offset in arrays) of cell c
-template <typename Maps, bool EDGE>
-__device__ __forceinline__ void put2(float *own, int a, float *g, long long gi, float2 v, int i0, int nx) {
-  if constexpr (TmaStore<Maps>::value) {
-    *reinterpret_cast<float2 *>(own + a * kArr) = v;
-  } else {
-    st_state2(g, gi, EDGE ? mask_pad2(v, i0, nx) : v);
-  }
-}
+// One result pair of array `a` of the stage: results leave through the stage
+// and TMA tensor stores (fewer store instructions than per-thread stores; the
+// store of a unit overlaps the compute of the next).
+__device__ __forceinline__ void put2(float *own, int a, float2 v) { *reinterpret_cast<float2 *>(own + a * kArr) = v; }
 __device__ __forceinline__ float &el2(float2 &v, int e) { return e == 0 ? v.x : v.y; }
-__device__ __forceinline__ float el2(const float2 &v, int e) { return e == 0 ? v.x : v.y; }
 // ten consecutive shared-memory values from column c of a row (c even)
 struct Win10 {
   float v[10];
@@ -661,8 +639,6 @@ __device__ __forceinline__ void vel_compute(const StepParams &P, const float *ta
   const int i0 = x0 + lx, j = y0 + ly;
   if (EDGE && (i0 >= P.nx || j >= P.ny)) return;
   float *own = const_cast<float *>(ss) + ly * kTX + lx;
-  const long long c = (long long)j * P.pitch + i0;
-  const long long Sn = P.npts_alloc;
   float2 Dx, Dy;
   vel_derivs2(P, sp, ly + 3, lx, Dx, Dy);
   float2 k1, A[N > 0 ? N : 1], B[N > 0 ? N : 1];
@@ -703,8 +679,8 @@ __device__ __forceinline__ void vel_compute(const StepParams &P, const float *ta
     const float2 tx = fma2(wn, nx_, mul2(wo, px)), ty = fma2(wn, ny_, mul2(wo, py));
     Sx = add2(Sx, tx);
     Sy = add2(Sy, ty);
-    put2<Maps, EDGE>(own, 2 + nu, P.psi1[0], nu * Sn + c, nx_, i0, P.nx);
-    put2<Maps, EDGE>(own, 2 + N + nu, P.psi1[1], nu * Sn + c, ny_, i0, P.nx);
+    put2(own, 2 + nu, nx_);
+    put2(own, 2 + N + nu, ny_);
   }
   const FaceRho fr = face_rho<N, Maps, EDGE>(P, T, sr, si, x0, y0, lx, ly);
   if (P.nl_vel) {
@@ -720,8 +696,8 @@ __device__ __forceinline__ void vel_compute(const StepParams &P, const float *ta
     vy.x = vel_upd(vy.x, qdiv(P.two_dt, fr.r0 + fr.u0), Sy.x);
     vy.y = vel_upd(vy.y, qdiv(P.two_dt, fr.r1 + fr.u1), Sy.y);
   }
-  put2<Maps, EDGE>(own, 0, P.v[0], c, vx, i0, P.nx);
-  put2<Maps, EDGE>(own, 1, P.v[1], c, vy, i0, P.nx);
+  put2(own, 0, vx);
+  put2(own, 1, vy);
 }
 
 template <int N, typename Maps, bool EDGE>
@@ -737,8 +713,6 @@ __device__ __forceinline__ void prs_compute(const StepParams &P, const float *ta
   const int i0 = x0 + lx, j = y0 + ly;
   if (EDGE && (i0 >= P.nx || j >= P.ny)) return;
   float *own = ss + ly * kTX + lx;
-  const long long c = (long long)j * P.pitch + i0;
-  const long long Sn = P.npts_alloc;
   float2 Dx, Dy;
   prs_derivs2(P, sx, sy, ly, lx, Dx, Dy);
   float2 k2, K, ch = make_float2(0.f, 0.f), A[N > 0 ? N : 1], B[N > 0 ? N : 1];
@@ -783,8 +757,8 @@ __device__ __forceinline__ void prs_compute(const StepParams &P, const float *ta
     const float2 tx = fma2(wn, nx_, mul2(wo, px)), ty = fma2(wn, ny_, mul2(wo, py));
     Sx = add2(Sx, tx);
     Sy = add2(Sy, ty);
-    put2<Maps, EDGE>(own, 1 + nu, P.psi2[0], nu * Sn + c, nx_, i0, P.nx);
-    put2<Maps, EDGE>(own, 1 + N + nu, P.psi2[1], nu * Sn + c, ny_, i0, P.nx);
+    put2(own, 1 + nu, nx_);
+    put2(own, 1 + N + nu, ny_);
   }
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
@@ -792,7 +766,7 @@ __device__ __forceinline__ void prs_compute(const StepParams &P, const float *ta
     if (P.nl) upd = qdiv(upd, fmaf(el2(ch, e), el2(p, e), 1.f));
     el2(p, e) -= upd;
   }
-  put2<Maps, EDGE>(own, 0, P.p, c, p, i0, P.nx);
+  put2(own, 0, p);
 }
 
 // Ring of stages: as many as fit next to the maps' table (2 .. 4).
@@ -806,7 +780,7 @@ struct Ring {
   // stored (the store has read it by then: no wait on it), two units ahead
   // of its compute; with two or three, right after its store, kStages - 1
   // units ahead.
-  static constexpr int kLag = (TmaStore<Maps>::value && kStages >= 4) ? 1 : 0;
+  static constexpr int kLag = kStages >= 4 ? 1 : 0;
   static constexpr int kAhead = kStages - 1 - kLag;
   static constexpr size_t kBytes = sizeof(float) * ((size_t)kStages * kStage + Maps::kSmemFloats) + 128;
   static_assert(kStages >= 2, "two stages must fit in shared memory");
@@ -1155,15 +1129,15 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   }
 }
 
-// Batched half step over a unit table of several contexts, 512 threads and one
-// barrier per unit (a warp of its own for the copies, as in steps2d_kernel,
-// was slower here, 12.1 against 11.2 ms for six contexts and 32 steps: every
-// context change empties the pipeline and leaves the index table to one warp)
-// (one group: same
-// N and map kind, no periodic axis): entry (ctx, x0, y0, interior).  The
+// Batched half step over a unit table of several contexts (one group: same N
+// and map kind, no periodic axis): entry (ctx, x0, y0, interior).  The
 // contexts' step parameters and tensor maps sit in device memory (TMA reads
 // the maps from there); a block copies a context's parameters to shared
 // memory, and stages its tissue-index table, when the context changes.
+// 512 threads and one barrier per unit: a warp of its own for the copies, as
+// in steps2d_kernel, was slower here (12.1 against 11.2 ms for six contexts
+// and 32 steps), since every context change empties the pipeline and leaves
+// the index table to one warp.
 template <int N, typename Maps, bool VEL>
 __global__ void __launch_bounds__(kThreads, 1)
     pipe2d_batched_kernel(const StepParams *Ps, const PipeMaps *Ts, const int4 *units, const int *runs) {
@@ -1207,7 +1181,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     pending |= 1u << q;
   }
   int s = 0, cur = -1;
-  // one barrier per unit (see pipe2d_kernel); a context change adds one
+  // one barrier per unit: after the wait for stage s it also marks the previous
+  // unit computed, so its stage is stored and refilled; a context change adds one
   int4 prev = make_int4(-1, 0, 0, 0);
 #pragma unroll 1
   for (; h < h_end; ++h) {
@@ -1226,9 +1201,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     pending &= ~(1u << s);
     const int sp = (s + kS - 1) % kS;       // the previous unit's stage
     const int q = (s + G::kAhead) % kS;     // the stage refilled now
-    if constexpr (TmaStore<Maps>::value) {
-      if (tid == 0 && prev.x >= 0) store_stage<N, Maps, VEL>(Ts[prev.x], smem + sp * kStage, prev.y, prev.z);
-    }
+    if (tid == 0 && prev.x >= 0) store_stage<N, Maps, VEL>(Ts[prev.x], smem + sp * kStage, prev.y, prev.z);
     const int4 e = units[h];
     if (e.x != cur) {
       // new context: parameters (and index table) into shared memory
@@ -1263,15 +1236,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (VEL) vel_compute<N, Maps, true>(sP, tab, stp, e.y, e.z, tid, edge);
       else prs_compute<N, Maps, true>(sP, tab, stp, e.y, e.z, tid, edge);
     }
-    if constexpr (TmaStore<Maps>::value) fence_proxy_async_smem();
+    fence_proxy_async_smem();
     prev = e;
     s = (s + 1) % kS;
   }
-  if constexpr (TmaStore<Maps>::value) {
-    __syncthreads();
-    if (tid == 0 && prev.x >= 0)
-      store_stage<N, Maps, VEL>(Ts[prev.x], smem + ((s + kS - 1) % kS) * kStage, prev.y, prev.z);
-  }
+  __syncthreads();
+  if (tid == 0 && prev.x >= 0)
+    store_stage<N, Maps, VEL>(Ts[prev.x], smem + ((s + kS - 1) % kS) * kStage, prev.y, prev.z);
   if (tid == 0) bulk_wait_all();
 }
 
