@@ -93,8 +93,8 @@ struct Region {
   // rotated by `rot` blocks from round to round.  Without the rotation a
   // block meets few columns (grid and ntx share factors: 152 blocks and 16 or
   // 32 columns), and those at the x edges, whose half tiles take longer, hold
-  // up the rest: 2048 x 1024 cells of the index form took 90 us a step
-  // without it and 78 us with it.
+  // up the rest: 12 % of a step of 2048 x 1024 cells of the index form (when
+  // the rotation came in; such a step takes 61 us now).
   int rot;
   __host__ __device__ __forceinline__ int halves() const { return ntx * nhy; }
   __device__ __forceinline__ int slot(int round, int b, int grid) const {
@@ -867,11 +867,12 @@ __device__ __forceinline__ void inject_unit(const StepIO &io, int u, long long n
   }
 }
 
-// Trace row of one step, groups spread over the blocks' last threads (the
-// copying warp had it on the path of its stores: 250 x 186 took 10.3 us a step
-// and not 9.1): the
-// mean of p over a group's cells, summed in their order.  p was written by
-// other SMs during this launch: read through L2, eight loads in flight.
+// Trace row of one step, groups spread over the blocks' last threads: the mean
+// of p over a group's cells, summed in their order.  p was written by other
+// SMs during this launch: read through L2, eight loads in flight.  (By the
+// copying warp, on the path of its stores, a step of 250 x 186 took 1.2 us
+// more.)  Long groups and many sensors are left to record_kernel
+// (record_apart).
 __device__ __forceinline__ void record_row(const StepIO &io, const float *p, long long n, int tid) {
   for (int g = blockIdx.x + (kThreads - 1 - tid) * gridDim.x; g < io.rec_groups; g += kThreads * gridDim.x) {
     const int b = __ldg(io.rec_off + g), e = __ldg(io.rec_off + g + 1);
@@ -892,28 +893,33 @@ __device__ __forceinline__ void record_row(const StepIO &io, const float *p, lon
 // half step of step n with its v sources, 2n + 1: pressure half step with its
 // p sources; the recording of step n runs in phase 2n + 2).  Block (32, 17),
 // one per SM: sixteen warps compute, the last one issues the copies and
-// stores and adds the sources.  More than one phase needs a cooperative launch, since the blocks
-// wait for one another between phases.
+// stores and adds the sources.  More than one phase needs a cooperative
+// launch, since the blocks wait for one another between phases.
 //
-// What bounds it: HBM on grids beyond L2 (4096^2, N = 4: 650 us a step,
-// 0.92 of the copy bandwidth on the step's bytes), the latency chain of a phase
-// (operand copy, compute, store, grid barrier: about 5 us) on small ones.
+// What bounds it: HBM on grids beyond L2 (4096^2, N = 4: 654 us a step, 0.92
+// of the copy bandwidth on the step's bytes), the latency chain of a phase
+// (operand copy, compute, store, grid barrier: about 4.4 us) on small ones.
 // Four launches per step (two half steps, sources, recording) added to every
 // one of them a start and a drain and left the SMs without copies in flight
 // meanwhile; here the next phase's first half tiles are copied (all but the
 // operand) while the barrier is under way, and sources and recording need no
-// launch of their own.  A step of 250 x 186 (N = 2) took 21 us and takes 8.5,
-// 512^2 (N = 4) 30 and 15.8, 1501 x 1237 111 and 75.  The velocity phases walk
-// the half tiles forwards and the pressure phases backwards, so each starts on
-// the rows whose operand the previous one left in L2 (0.8 % at 1501 x 1237).
+// launch of their own.  The velocity phases walk the half tiles forwards and
+// the pressure phases backwards, so each starts on the rows whose operand the
+// previous one left in L2 (0.8 % at 1501 x 1237).
 //
 // A stage goes round full -> computed -> stored -> refilled.  The computing
 // warps wait for "full" and announce "computed" each on its own, so that a
 // warp starts on the next stage while others are still busy with the last one
-// and nobody waits for a store to leave; one barrier per half tile for all
-// threads, with the copies issued by one of the computing threads, took 19
-// us a step at 512^2 (17 now), 82 at 2048 x 1024 of the uint8 index form (74),
-// 681 at 4096^2 (655).
+// and nobody waits for a store to leave (10 % at 512^2 and 2048 x 1024 of the
+// uint8 index, 4 % at 4096^2, over one barrier per half tile for all threads
+// and copies issued by one of them).
+//
+// us a step with four launches of half-step kernels and now: 250 x 186 (N = 2)
+// 20.6 and 8.8, 512^2 (N = 4) 28.8 and 15.7, 1501 x 1237 with cross taps 104
+// and 75, 2048 x 1024 of the uint8 index 91 and 61, 4096^2 681 and 654.  A
+// launch keeps its SMs to its end: contexts that step on several streams at
+// once take turns unless their half tiles fit side by side (three of 250 x 186
+// 5.4 and 2.6 us a step of each; three of 512^2, N = 2, 7.8 and 11.9).
 template <int N, typename Maps>
 __global__ void __launch_bounds__(kStepThreads, 1)
     steps2d_kernel(const StepParams P, const Region R, const __grid_constant__ StepMaps TV,
