@@ -818,13 +818,13 @@ struct SourceBits {
     return round >= 32 * kSrcWords || ((w[half][round >> 5] >> (round & 31)) & 1u);
   }
 };
-// Set the bits (computing threads), once they are zero.
-__device__ __forceinline__ void mark_sources(const StepIO &io, const Region &R, int per, SourceBits &bits, int tid) {
+// Set the bits (one warp), once they are zero.
+__device__ __forceinline__ void mark_sources(const StepIO &io, const Region &R, int per, SourceBits &bits, int lane) {
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
     const int *unit = io.src[f].unit;
     if (!unit) continue;
-    for (int r = tid; r < per && r < 32 * kSrcWords; r += kThreads) {
+    for (int r = lane; r < per && r < 32 * kSrcWords; r += 32) {
       const int u = r * (int)gridDim.x + R.slot(r, blockIdx.x, gridDim.x);
       if (__ldg(unit + u) < __ldg(unit + u + 1)) atomicOr(&bits.w[f == 0 ? 1 : 0][r >> 5], 1u << (r & 31));
     }
@@ -1030,6 +1030,13 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       }
     };
     fill(ph0);
+    // With the source marks and the index table ahead of the first copies, and
+    // the parameters above 4 KB, the two half steps of a step in launches of
+    // their own took 16.6 us at 250 x 186 (N = 4, float; 14.7 now), 20.7 at 640
+    // x 640 (N = 2; 18.5), 36.3 at 512 x 512 of the uint16 index with 1160
+    // tissues (33.0).
+    mark_sources(io, R, per, sources, lane);
+    __syncwarp();
     bool ok = true;
 #pragma unroll 1
     while (true) {
@@ -1091,13 +1098,6 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   }
 
   // ------------------------------------------------------------- compute ---
-  // The first half tiles are being copied meanwhile; the copying warp looks at
-  // the marks after every computing warp's first arrival only.  With both ahead
-  // of the copies, and the parameters above 4 KB, the two half steps of a step
-  // in launches of their own took 16.6 us at 250 x 186 (N = 4, float; 14.7
-  // now), 20.7 at 640 x 640 (N = 2; 18.5), 36.3 at 512 x 512 of the uint16
-  // index with 1160 tissues (33.0).
-  mark_sources(io, R, per, sources, tid);
   if constexpr (Form<Maps>::kIdx) {
     stage_table<N, Maps>(P, tab, tid);
     asm volatile("bar.sync 1, %0;\n" ::"n"(kThreads) : "memory");
