@@ -1032,9 +1032,9 @@ __global__ void __launch_bounds__(kStepThreads, 1)
     fill(ph0);
     // With the source marks and the index table ahead of the first copies, and
     // the parameters above 4 KB, the two half steps of a step in launches of
-    // their own took 16.6 us at 250 x 186 (N = 4, float; 14.7 now), 20.7 at 640
-    // x 640 (N = 2; 18.5), 36.3 at 512 x 512 of the uint16 index with 1160
-    // tissues (33.0).
+    // their own took 16.6 us at 250 x 186 (N = 4, float; 12.9 now) and 36.5 at
+    // 512 x 512 of the uint16 index with 1160 tissues (33.0).  (Marked by the
+    // computing warps, steps in one launch took 1.7 % more at 250 x 186.)
     mark_sources(io, R, per, sources, lane);
     __syncwarp();
     bool ok = true;

@@ -840,8 +840,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   // this block's items: one per round of gridDim.x consecutive ones, rotated
   // by R.rot blocks from round to round (without it a block whose grid and
   // column counts share factors meets few columns: 152 blocks and 4 columns
-  // give half the blocks nothing but x-edge units; 512^3, bf16: 6.15 ms a step
-  // without it and 5.65 ms with it)
+  // give half the blocks nothing but x-edge units; 512^3, bf16, when it came
+  // in: 6.15 ms a step without it and 5.65 with it)
   const long long grid = gridDim.x;
   long long slot = blockIdx.x, it = slot;
   if (it >= n_items) return;
