@@ -1319,8 +1319,11 @@ Region3 region3_of(const StepParams &P, int grid, bool ps) {
       R.nseg = used;
     }
   }
+  // a round advances a block by grid + rot columns: every column in turn, or
+  // every second one, which holds one of the two at the x edges as well
+  // (six columns: 768^3, bf16, 17.25 ms a step with all in turn, 17.16 so)
   R.rot = 0;
-  while (R.rot + 1 < grid && std::gcd(grid + R.rot, R.tnx) != 1) ++R.rot;
+  while (R.rot + 1 < grid && std::gcd(grid + R.rot, R.tnx) > 2) ++R.rot;
   return R;
 }
 
