@@ -206,7 +206,7 @@ def test_3d_batches_equal_their_contexts_alone_in_every_arithmetic_form(fw2, N, 
 @pytest.mark.parametrize("shape", [(700, 240, 20), (500, 312, 20), (250, 640, 20)])   # six, four and two columns of units
 def test_3d_rounds_over_the_blocks_reach_every_item(fw2, maps, shape):
     """More items than blocks, with the rounds rotated over the blocks (four
-    columns) and not (six and two): the bits of the tile kernels."""
+    and two columns) and not (six): the bits of the tile kernels."""
     from tests.test_gpu_parity import _pipe_vs_tile, small_3d
     prob = small_3d(n=shape, N=2, nl="pressure", steps=6, pml=(4, 1))
     _pipe_vs_tile(fw2, prob, 6, maps=maps, state=synth.random_state(prob, seed=2))
