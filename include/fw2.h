@@ -326,9 +326,10 @@ fw2_status fw2_batch_create(fw2_ctx *const *ctxs, int32_t n_ctx, fw2_batch **out
  * except where the set of active contexts changes (see budgets).  One launch
  * per half step and group.  For many small contexts (up to about 512 x 512)
  * this is the faster way; large 2D contexts step faster one after the other
- * through fw2_step's launches of many steps (six of 2048 x 1024 of the uint8
- * index: 4 %; 1024 x 1024, float maps, N = 4: 10 to 25 %), those with bf16,
- * FP16 or uint16 index storage by twice, and so do 3D contexts (20 to 40 %). */
+ * through fw2_step's launches of many steps (six of up to 2048 x 1024 of the
+ * uint8 index: 4 %; 1024 x 1024, float maps, N = 4: 10 to 25 %; bf16, FP16 and
+ * uint16 index storage: about twice as fast), and so do 3D contexts of a
+ * million cells and more (a batch takes 35 to 75 % longer). */
 fw2_status fw2_batch_step(fw2_batch *b, int64_t n_steps);
 /* Step budgets: context i leaves the batch once its step counter reaches
  * last_step[i] (< 0: no budget; NULL clears every budget).  fw2_batch_step
